@@ -119,8 +119,15 @@ typedef struct {
                                  0 = default: 512); raised to the longest track.  A
                                  tuning knob: the chunking groups the per-camera partial
                                  sums, so results agree up to rounding. */
-  int32_t spmv_variant;       /* Schur-product kernel: 0 = automatic (pipelined for BF16
-                                 and FP32 storage, classic for FP64), 1 = staged
+  int32_t spmv_variant;       /* Schur-product kernel: 0 = automatic (explicit where it
+                                 pays: the blocks of the camera Schur complement are
+                                 formed once per damped system and the whole PCG runs in
+                                 one launch; it takes device memory for the blocks and
+                                 for one row of 3 values per edge and camera coordinate,
+                                 and is left out where the memory budget holds the graph
+                                 only without, a camera sees a point twice, or forming
+                                 the blocks costs more than it saves; then pipelined for
+                                 BF16 and FP32 storage, classic for FP64), 1 = staged
                                  (persistent CTAs streaming chunks into shared memory
                                  with bulk copies), 2 = classic (one CTA per chunk),
                                  3 = pipelined (persistent CTAs prefetching the next
@@ -138,9 +145,9 @@ typedef struct {
                                  segmented warp scan, one barrier per chunk; BF16 and
                                  FP32 storage).  1, 3 and 5 need chunks of at most 1024
                                  edges, 4 of at most 512, else classic runs (5 with
-                                 FP64 storage too).  0..3 give bit-identical results;
-                                 5 sums each point's terms in another order and 4 uses
-                                 unrounded rows, so their products agree with the
+                                 FP64 storage too).  1..3 give bit-identical results;
+                                 the explicit product and 5 sum in another order and 4
+                                 uses unrounded rows, so their products agree with the
                                  others up to rounding. */
 } gpo_graph_desc;
 
@@ -353,7 +360,7 @@ typedef struct {
   int32_t spmv_variant;       /* as requested in gpo_graph_desc */
   int32_t spmv_kernel;        /* the Schur-product kernel the PCG runs, in spmv_variant's
                                  numbering (1 staged, 2 classic, 3 pipelined, 4 dynamic,
-                                 5 warp groups; 0: no observation edges) */
+                                 5 warp groups, 7 explicit; 0: no observation edges) */
   int32_t reserved0;
   int64_t j_bytes;            /* device bytes of the stored Jacobian rows (0 with dynamic
                                  Jacobians, which store none) */

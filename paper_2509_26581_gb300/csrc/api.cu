@@ -117,6 +117,8 @@ struct Plan {
   }
 };
 
+constexpr size_t kClusterBytes = 1 << 20;   // see plan_explicit
+
 size_t at_size(Prec p) { return p == Prec::F64 ? 8 : 4; }
 size_t jt_size(Prec p) { return p == Prec::F64 ? 8 : (p == Prec::F32 ? 4 : 2); }
 
@@ -204,6 +206,15 @@ struct Prepared {
       *xe_kind_d = nullptr, *xo_off_d = nullptr, *xk_off_d = nullptr, *xk_list_d = nullptr, *ch_prob_d = nullptr,
       *cb_prob_d = nullptr, *pb_prob_d = nullptr, *base_d = nullptr, *running_d = nullptr,
       *old2new_d = nullptr;
+  // explicit Schur complement (ex false: not planned)
+  bool ex = false, ex_cluster = false;
+  int ex_nb_max = 0, ex_ctas = 0, ex_res = 0;
+  size_t ex_smem = 0;
+  std::vector<int32_t> ex_loff, ex_lcol, ex_lidx, ex_lown, ex_xl;
+  int *ex_loff_d = nullptr, *ex_lcol_d = nullptr, *ex_lidx_d = nullptr, *ex_lown_d = nullptr, *ex_xl_d = nullptr;
+  std::vector<int32_t> ex_row, ex_col, ex_uoff, ex_ublk, ex_crow, ex_slot_y0, ex_doff, ex_dcam, zeros_xf, zeros_xd;
+  int *ex_row_d = nullptr, *ex_col_d = nullptr, *ex_uoff_d = nullptr, *ex_ublk_d = nullptr, *ex_crow_d = nullptr,
+      *ex_slot_y0_d = nullptr, *ex_doff_d = nullptr, *ex_dcam_d = nullptr, *xf_prob_d = nullptr, *xd_prob_d = nullptr;
   uint16_t *e_pos_d = nullptr, *e_slot_d = nullptr, *ch_sorted_d = nullptr, *ch_grp_d = nullptr;
   uint32_t* e_meta_d = nullptr;
   uint8_t *cam_fixed_d = nullptr, *pt_fixed_d = nullptr;
@@ -213,6 +224,195 @@ struct Prepared {
 };
 
 void PrepDeleter::operator()(Prepared* p) const { delete p; }
+
+// Plans the explicit Schur complement: which camera pairs share points, the camera-major
+// rows and the work items.  Leaves R.ex false where the product stays matrix-free: a
+// product other than the automatic one was asked for, a camera sees a point twice, or
+// forming the blocks costs more than they save.
+//
+// The rule compares times on the GB300.  Forming: 0.014 ns per row pair in FP32 (about
+// four cycles per pair and SM), 0.46 ns in FP64 (243 FP64 multiply-adds per pair at the
+// pipe's rate).  A matrix-free iteration: 0.026 ns per edge in FP32 and BF16 storage, 0.21
+// ns in FP64, and 20 us of launches and barriers; an explicit one: the blocks' bytes at 6
+// TB/s and 6 us.  A solve is taken to have 16 iterations (solves to 1e-6 took 11 to 100).
+static void plan_explicit(gpo_graph* g, Prepared& R, const gpo::KernelSet& ks, int C, int P, int E, int NS) {
+  R.ex = false;
+  if (g->desc.spmv_variant != 0 || E == 0 || C < 2 || C > 32768) return;
+  int64_t pairs = 0;
+  for (int p = 0; p < P; ++p) {
+    const int64_t k = R.pt_off[p + 1] - R.pt_off[p];
+    pairs += k * (k - 1) / 2;
+  }
+  const bool f64 = g->prec == Prec::F64;
+  const double form = pairs * (f64 ? 4.6e-10 : 1.4e-11), free_it = E * (f64 ? 2.1e-10 : 2.6e-11) + 20e-6;
+  const int EL = ks.DC * ks.DC;
+  const size_t sA = at_size(g->prec);
+  auto pays = [&](size_t nb) { return form + 16 * ((double)nb * EL * sA / 6e12 + 6e-6) < 16 * free_it; };
+  if (pairs == 0 || pairs > (int64_t)1 << 30 || !pays(0)) return;
+  // cameras sharing a point: a bit row per camera; a point ORs the words its cameras fall
+  // into onto each of their rows
+  const int W = (C + 63) / 64;
+  std::vector<uint64_t> bits((size_t)C * W, 0);
+  std::vector<int32_t> seen(C, -1);
+  std::vector<std::pair<int, uint64_t>> words;
+  for (int p = 0; p < P; ++p) {
+    const int a = R.pt_off[p], b = R.pt_off[p + 1];
+    words.clear();
+    for (int e = a; e < b; ++e) {
+      const int c = R.e_cam_s[e], w = c >> 6;
+      if (seen[c] == p) return;   // the camera sees the point twice
+      seen[c] = p;
+      if (words.empty() || words.back().first != w) words.push_back({w, 0});
+      words.back().second |= (uint64_t)1 << (c & 63);
+    }
+    for (int e = a; e < b; ++e) {
+      uint64_t* row = &bits[(size_t)R.e_cam_s[e] * W];
+      for (const auto& x : words) row[x.first] |= x.second;
+    }
+  }
+  R.ex_row.assign(C + 1, 0);
+  R.ex_uoff.assign(C + 1, 0);
+  R.ex_col.clear();
+  for (int c = 0; c < C; ++c) {
+    int up = 0;
+    for (int w = 0; w < W; ++w) {
+      uint64_t v = bits[(size_t)c * W + w];
+      while (v) {
+        const int j = 64 * w + __builtin_ctzll(v);
+        v &= v - 1;
+        if (j == c) continue;
+        R.ex_col.push_back(j);
+        up += j > c;
+      }
+    }
+    R.ex_row[c + 1] = (int)R.ex_col.size();
+    R.ex_uoff[c + 1] = R.ex_uoff[c] + up;
+    R.ex_nb_max = std::max(R.ex_nb_max, up);
+    if (R.ex_col.size() > (size_t)1 << 28) return;
+  }
+  const size_t NB = R.ex_col.size();
+  if (R.ex_nb_max > 5000 || !pays(NB)) return;
+  const int NBU = R.ex_uoff[C];
+  R.ex_ublk.resize(2 * (size_t)NBU);
+  {
+    std::vector<int32_t> low(R.ex_row.begin(), R.ex_row.end() - 1);   // next left-of-diagonal block of a row
+    for (int c = 0, u = 0; c < C; ++c)
+      for (int b = R.ex_row[c + 1] - (R.ex_uoff[c + 1] - R.ex_uoff[c]); b < R.ex_row[c + 1]; ++b, ++u) {
+        R.ex_ublk[2 * (size_t)u] = b;
+        R.ex_ublk[2 * (size_t)u + 1] = low[R.ex_col[b]]++;
+      }
+  }
+  // camera-major rows: a camera's slots in chunk order
+  R.ex_crow.assign(C + 1, 0);
+  for (int s = 0; s < NS; ++s) R.ex_crow[R.slot_cam[s] + 1] += R.slot_e0[s + 1] - R.slot_e0[s];
+  for (int c = 0; c < C; ++c) R.ex_crow[c + 1] += R.ex_crow[c];
+  R.ex_slot_y0.resize(NS);
+  {
+    std::vector<int32_t> fill(R.ex_crow.begin(), R.ex_crow.end() - 1);
+    for (int s = 0; s < NS; ++s) {
+      R.ex_slot_y0[s] = fill[R.slot_cam[s]];
+      fill[R.slot_cam[s]] += R.slot_e0[s + 1] - R.slot_e0[s];
+    }
+  }
+  // Work items of up to 1,024 row pairs or rows; small problems are cut finer, until there
+  // are about as many items as the chip has sub-partitions (608): a warp alone issues an
+  // FP64 multiply-add every 70 cycles or so, so the work has to spread
+  auto segment = [](int64_t n, int lo) {
+    int s = lo;
+    while (s < 1024 && s < n / 608) s *= 2;
+    return s;
+  };
+  DevBA& d = R.d;
+  const int seg = d.ex_seg = segment(pairs, f64 ? 32 : 128);
+  d.ex_dseg = segment(E, f64 ? 32 : 64);
+  R.ex_doff.assign(C + 1, 0);
+  R.ex_dcam.clear();
+  for (int c = 0; c < C; ++c) {
+    const int n = (R.ex_crow[c + 1] - R.ex_crow[c] + d.ex_dseg - 1) / d.ex_dseg;
+    R.ex_doff[c + 1] = R.ex_doff[c] + n;
+    R.ex_dcam.insert(R.ex_dcam.end(), n, c);
+  }
+  size_t row_bytes = 0;
+  int wpc = 1;
+  ks.ex_sizes(g->prec, &row_bytes, &wpc);
+  const int64_t items = NBU + pairs / seg;
+  const size_t parts = 2 * (size_t)(pairs / seg) + 1;
+  d.ex = 1;
+  d.ex_nb = (int)NB;
+  d.ex_nbu = NBU;
+  d.ex_nd = (int)R.ex_dcam.size();
+  d.ex_nxf = (int)std::min<int64_t>((items + 3) / 4, f64 ? INT32_MAX : 3 * 152);   // FP32: the CTAs that are resident
+  R.zeros_xf.assign(d.ex_nxf, 0);
+  R.zeros_xd.assign((d.ex_nd + wpc - 1) / wpc, 0);
+  // a problem whose blocks fit the shared memory of a cluster is solved by one (its barriers
+  // are the cheapest), a larger one by the whole grid
+  R.ex_cluster = NB * EL * sA <= (size_t)kClusterBytes && C <= gpo::kExThreads / 32 * gpo::kExCluster;
+  const int G = R.ex_ctas = R.ex_cluster ? gpo::kExCluster : std::min(gpo::kExGrid, C);
+  const int rpc = (C + G - 1) / G;
+  R.ex_loff.assign(1, 0);
+  R.ex_lcol.clear();
+  R.ex_lidx.resize(NB);
+  R.ex_lown.resize(C);
+  R.ex_xl.assign(R.xk_list.size(), -1);
+  {
+    auto other = [&](int u) { return (R.xk_list[u] & 1) ? R.xi_s[R.xk_list[u] >> 1] : R.xj_s[R.xk_list[u] >> 1]; };
+    std::vector<int32_t> at(C, -1), set;
+    size_t nloc = 0;
+    for (int k = 0; k < G; ++k) {
+      const int r0 = std::min(k * rpc, C), r1 = std::min(r0 + rpc, C);
+      set.clear();
+      auto add = [&](int c) {
+        if (c >= 0 && at[c] < 0) {
+          at[c] = 0;
+          set.push_back(c);
+        }
+      };
+      if (R.ex_cluster)   // a cluster keeps every camera (z is sent to all of its CTAs)
+        for (int c = 0; c < C; ++c) add(c);
+      for (int c = r0; c < r1; ++c) {
+        add(c);
+        for (int b = R.ex_row[c]; b < R.ex_row[c + 1]; ++b) add(R.ex_col[b]);
+        for (int u = R.xk_off[c]; u < R.xk_off[c + 1]; ++u) add(other(u));
+      }
+      std::sort(set.begin(), set.end());
+      for (size_t i = 0; i < set.size(); ++i) at[set[i]] = (int)i;
+      for (int c = r0; c < r1; ++c) {
+        R.ex_lown[c] = at[c];
+        for (int b = R.ex_row[c]; b < R.ex_row[c + 1]; ++b) R.ex_lidx[b] = at[R.ex_col[b]];
+        for (int u = R.xk_off[c]; u < R.xk_off[c + 1]; ++u) R.ex_xl[u] = other(u) >= 0 ? at[other(u)] : -1;
+      }
+      for (int c : set) at[c] = -1;
+      R.ex_lcol.insert(R.ex_lcol.end(), set.begin(), set.end());
+      R.ex_loff.push_back((int)R.ex_lcol.size());
+      nloc = std::max(nloc, set.size());
+    }
+    int nres = 0;   // most blocks of a CTA
+    for (int k = 0; k < G; ++k) nres = std::max(nres, R.ex_row[std::min((k + 1) * rpc, C)] - R.ex_row[std::min(k * rpc, C)]);
+    R.ex_smem = ks.ex_smem(g->prec, C, G, (int)nloc, nres);
+    R.ex_res = 1;
+    if (R.ex_smem > 224 * 1024) {   // the blocks stay in global memory
+      R.ex_smem = ks.ex_smem(g->prec, C, G, (int)nloc, 0);
+      R.ex_res = 0;
+    }
+    if (R.ex_smem > 224 * 1024 || (R.ex_cluster && !R.ex_res)) return;
+  }
+  R.ex = true;
+  Plan& pl = R.pl;
+  pl.up(&R.ex_row_d, C + 1, R.ex_row); pl.up(&R.ex_col_d, NB, R.ex_col); pl.up(&R.ex_uoff_d, C + 1, R.ex_uoff);
+  pl.up(&R.ex_ublk_d, 2 * (size_t)NBU, R.ex_ublk); pl.up(&R.ex_crow_d, C + 1, R.ex_crow);
+  pl.up(&R.ex_slot_y0_d, NS, R.ex_slot_y0); pl.up(&R.ex_doff_d, C + 1, R.ex_doff);
+  pl.up(&R.ex_dcam_d, d.ex_nd, R.ex_dcam); pl.up(&R.xf_prob_d, d.ex_nxf, R.zeros_xf);
+  pl.up(&R.xd_prob_d, R.zeros_xd.size(), R.zeros_xd);
+  pl.add(&d.ex_poff, (size_t)NBU + 1); pl.add(&d.ex_pair, (size_t)pairs); pl.add(&d.ex_item, (size_t)items);
+  pl.add(&d.ex_multi, (size_t)(pairs / seg) + 1); pl.add(&d.ex_count, 2);
+  pl.add_raw(&d.ex_Y, row_bytes * (((size_t)E + 31) / 32 * 32));
+  pl.add_raw(&d.ex_S, NB * EL * sA); pl.add_raw(&d.ex_part, parts * EL * sA);
+  pl.add_raw(&d.ex_dpart, (size_t)d.ex_nd * ks.NPA * sA);
+  pl.add(&d.ex_red, 8 * (size_t)gpo::kExMaxCtas + 2); pl.add(&d.ex_z, (size_t)C * ks.DB * (sA / 4));
+  pl.up(&R.ex_loff_d, R.ex_loff.size(), R.ex_loff); pl.up(&R.ex_lcol_d, R.ex_lcol.size(), R.ex_lcol);
+  pl.up(&R.ex_lidx_d, NB, R.ex_lidx); pl.up(&R.ex_lown_d, C, R.ex_lown);
+  pl.up(&R.ex_xl_d, std::max<size_t>(R.ex_xl.size(), 1), R.ex_xl);
+}
 
 static gpo_status prepare(gpo_graph* g) {
   const gpo::KernelSet& ks = gpo_host::kernels_of(g);
@@ -228,23 +428,31 @@ static gpo_status prepare(gpo_graph* g) {
   if (!pp) return fail(g, GPO_ERR_OOM, "host allocation failed");
   Prepared& R = *pp;
 
-  // point order: by the smallest camera index among the point's active edges
-  // (points without active edges last), ties by point index.  Consecutive points
-  // then share cameras, which keeps the per-chunk camera slot count small.
-  std::vector<int32_t> key(P, C);
+  // point order: by the smallest, then the largest camera index among the point's active
+  // edges (points without active edges last), ties by point index.  Consecutive points
+  // then share cameras, which keeps the per-chunk camera slot count small, and points with
+  // the same span of cameras are adjacent, which makes the rows that a pair of cameras
+  // shares (k_ex_form) runs of consecutive ones.
+  std::vector<int32_t> key(P, C), last(P, 0);
   std::vector<int32_t> deg(P, 0);
   for (int64_t e = 0; e < Eall; ++e)
     if (g->e_active[e]) {
       const int p = g->e_pt[e];
       key[p] = std::min(key[p], g->e_cam[e]);
+      last[p] = std::max(last[p], g->e_cam[e]);
       deg[p]++;
     }
-  std::vector<int32_t> cnt(C + 2, 0);
+  std::vector<int32_t> cnt(C + 2, 0), by_last(P);
+  for (int p = 0; p < P; ++p) cnt[last[p] + 1]++;
+  for (int k = 0; k <= C; ++k) cnt[k + 1] += cnt[k];
+  for (int p = 0; p < P; ++p) by_last[cnt[last[p]]++] = p;
+  std::fill(cnt.begin(), cnt.end(), 0);
   for (int p = 0; p < P; ++p) cnt[key[p] + 1]++;
   for (int k = 0; k <= C; ++k) cnt[k + 1] += cnt[k];
   R.pt_new2old.assign(P, 0);
   R.pt_old2new.assign(P, 0);
-  for (int p = 0; p < P; ++p) {
+  for (int q = 0; q < P; ++q) {
+    const int p = by_last[q];
     const int np = cnt[key[p]]++;
     R.pt_new2old[np] = p;
     R.pt_old2new[p] = np;
@@ -519,6 +727,18 @@ static gpo_status prepare(gpo_graph* g) {
   pl.add(&d.hist, gpo::kMaxHistory);
   pl.add(&R.desc_d, 1);
   R.bytes = pl.total();
+  // the explicit Schur complement, unless the memory budget holds the graph only without
+  {
+    Plan plain = pl;
+    plan_explicit(g, R, ks, C, P, E, NS);
+    if (R.ex && g->desc.memory_budget && pl.total() > g->desc.memory_budget) R.ex = false;
+    if (R.ex) {
+      R.bytes = pl.total();
+    } else {
+      pl = std::move(plain);
+      d.ex = 0;
+    }
+  }
   g->prep.reset(pp.release());
   return GPO_OK;
 }
@@ -572,6 +792,12 @@ gpo_status gpo_host::finalize(gpo_graph* g, size_t* plan_bytes) {
   d.ch_grp = R.ch_grp_d;
   d.dbg_r = nullptr;
   const cudaStream_t st = g->stream;
+  if (R.ex && !R.ex_cluster && !gpo_host::kernels_of(g).ex_grid_ok(g->prec, R.ex_smem)) R.ex = false;
+  d.ex_loff = R.ex_loff_d; d.ex_lcol = R.ex_lcol_d; d.ex_lidx = R.ex_lidx_d; d.ex_lown = R.ex_lown_d; d.ex_xl = R.ex_xl_d;
+  d.ex = R.ex ? 1 : 0;
+  d.ex_row = R.ex_row_d; d.ex_col = R.ex_col_d; d.ex_uoff = R.ex_uoff_d;
+  d.ex_ublk = reinterpret_cast<const int2*>(R.ex_ublk_d);
+  d.ex_crow = R.ex_crow_d; d.ex_slot_y0 = R.ex_slot_y0_d; d.ex_doff = R.ex_doff_d; d.ex_dcam = R.ex_dcam_d;
   {
     std::vector<char> img;
     const size_t n = R.pl.image(img);
@@ -593,8 +819,26 @@ gpo_status gpo_host::finalize(gpo_graph* g, size_t* plan_bytes) {
   ls.ch_max = R.ch;
   ls.ns_max = d.ns_max;
   ls.np_max = d.np_max;
-  g->ls = ls;
   g->ks = &gpo_host::kernels_of(g);
+  ls.mf = 1;
+  if (R.ex) {
+    ls.ex = 1;
+    ls.mf = 0;
+    ls.xf_prob = R.xf_prob_d; ls.xf_base = R.base_d;
+    ls.xd_prob = R.xd_prob_d; ls.xd_base = R.base_d;
+    ls.cl_prob = R.base_d;
+    ls.n_xf = d.ex_nbu > 0 ? d.ex_nxf : 0;
+    ls.n_xd = (int)R.zeros_xd.size();
+    g->ex_cluster = R.ex_cluster;
+    g->ex_grid = make_int4(0, R.ex_ctas, (int)R.ex_smem, R.ex_res);
+    ls.xg_host = &g->ex_grid;
+    (R.ex_cluster ? ls.n_cl : ls.n_xg) = 1;
+    ls.cl_smem = (int)R.ex_smem;
+    ls.ex_scratch = d.ex_Y;
+    g->ks->ex_plan(ls, g->prec, d.C, R.ex_nb_max, d.E, st);
+    ls.ex_scratch = nullptr;
+  }
+  g->ls = ls;
   g->dev_desc = R.desc_d;
   g->ch_max = R.ch;
   g->j_elems = R.jpos;
@@ -846,11 +1090,36 @@ static gpo_status ensure_full(gpo_graph* g) {
   return GPO_OK;
 }
 
+static gpo_status solve_matrix_free(gpo_graph* g, const gpo::LaunchSet& ls, int max_it);
+
 gpo_status gpo_host::solve_system(gpo_graph* g, const gpo::LaunchSet& ls, int max_it, bool force_lin) {
   if (g->pcg_full) {
     if (gpo_status s = ensure_full(g); s != GPO_OK) return s;
   }
   run(g, KK_LINEARIZE, [&] { return g->ks->linearize(ls, g->prec, force_lin, g->stream); });
+  if (ls.ex && !g->pcg_full) {   // explicit Schur complement (of the problems that have one planned)
+    if (ls.mf) run(g, KK_SCHUR, [&] { return g->ks->schur_prepare(ls, g->prec, g->stream); });
+    run(g, KK_EX_FORM, [&] { return g->ks->ex_form(ls, g->prec, g->stream); });
+    if (ls.mf) GPO_CUDA(g, cudaMemsetAsync(ls.running, 0, 6 * sizeof(int), g->stream));
+    run(g, KK_CAM_FINALIZE, [&] { return g->ks->cam_finalize(ls, g->prec, g->stream); });
+    int n = 0;
+    run(g, KK_EX_PCG, [&] { n = g->ks->ex_pcg(ls, g->prec, g->stream); return std::max(n, 0); });
+    GPO_CUDA(g, cudaGetLastError());
+    if (n < 0) return fail(g, GPO_ERR_CUDA, "the launch of the PCG solve was refused");
+    if (ls.mf) {
+      if (gpo_status s = pcg_solve(g, ls, max_it); s != GPO_OK) return s;
+    }
+    g->cur_pcg_k = 0;
+    run(g, KK_BACKSUB, [&] { return g->ks->backsub(ls, g->prec, g->stream); });
+    GPO_CUDA(g, cudaGetLastError());
+    return GPO_OK;
+  }
+  gpo::LaunchSet lm = ls;
+  lm.ex = 0;
+  return solve_matrix_free(g, lm, max_it);
+}
+
+static gpo_status solve_matrix_free(gpo_graph* g, const gpo::LaunchSet& ls, int max_it) {
   run(g, KK_SCHUR, [&] { return g->ks->schur_prepare(ls, g->prec, g->stream); });
   GPO_CUDA(g, cudaMemsetAsync(ls.running, 0, 6 * sizeof(int), g->stream));   // flags and work counters
   if (g->pcg_full) run(g, KK_FULL_INIT, [&] { return g->ks->full_init(ls, g->prec, g->stream); });
@@ -861,6 +1130,19 @@ gpo_status gpo_host::solve_system(gpo_graph* g, const gpo::LaunchSet& ls, int ma
   g->cur_pcg_k = 0;
   run(g, KK_BACKSUB, [&] { return g->ks->backsub(ls, g->prec, g->stream); });
   GPO_CUDA(g, cudaGetLastError());
+  return GPO_OK;
+}
+
+// The flags and counters of the whole-grid PCG solves start at zero; end_solves waits for
+// the stream and reports a solve whose grid barrier gave up.
+gpo_status gpo_host::begin_solves(gpo_graph* g, const gpo::LaunchSet& ls) {
+  if (ls.ex) GPO_CUDA(g, cudaMemsetAsync(ls.running, 0, 6 * sizeof(int), g->stream));
+  return GPO_OK;
+}
+gpo_status gpo_host::end_solves(gpo_graph* g, const gpo::LaunchSet& ls) {
+  if (ls.n_xg) GPO_CUDA(g, cudaMemcpyAsync(g->h_flag, ls.running, 2 * sizeof(int), cudaMemcpyDeviceToHost, g->stream));
+  GPO_CUDA(g, cudaStreamSynchronize(g->stream));
+  if (ls.n_xg && g->h_flag[1]) return fail(g, GPO_ERR_TIMEOUT, "a bounded device wait in the PCG solve gave up");
   return GPO_OK;
 }
 
@@ -1407,6 +1689,7 @@ gpo_status gpo_optimize(gpo_graph* g, int32_t max_iters, const gpo_lm_params* pa
   if (cont) F0 = g->last_cost;
   else if ((s = compute_cost(g, &F0)) != GPO_OK) return s;
   if (!std::isfinite(F0)) return fail(g, GPO_ERR_NUMERIC, "initial cost is not finite (%g)", F0);
+  if ((s = begin_solves(g, g->ls)) != GPO_OK) return s;
   for (int it = 0; it < max_iters; ++it) {
     g->cur_lm_iter = it;
     if ((s = solve_system(g, g->ls, sc.max_it, false)) != GPO_OK) return s;
@@ -1419,7 +1702,7 @@ gpo_status gpo_optimize(gpo_graph* g, int32_t max_iters, const gpo_lm_params* pa
   if (nh)
     GPO_CUDA(g, cudaMemcpyAsync(g->hist.data(), g->dev.hist, nh * sizeof(gpo::IterRecord),
                                 cudaMemcpyDeviceToHost, g->stream));
-  GPO_CUDA(g, cudaStreamSynchronize(g->stream));
+  if ((s = end_solves(g, g->ls)) != GPO_OK) return s;
   if (g->prof.on) prof_resolve(g);
   g->last_cost = g->h_sc->cost;
   g->cost_valid = true;
@@ -1523,7 +1806,7 @@ gpo_status gpo_graph_info(gpo_graph* g, gpo_graph_info_t* out) {
   out->slots = d.NS;
   out->chunk_edges = g->ch_max;
   out->spmv_variant = g->desc.spmv_variant;
-  out->spmv_kernel = d.E > 0 ? g->ks->spmv_kind(g->ls, g->prec) : 0;
+  out->spmv_kernel = d.E > 0 ? (g->ls.ex ? 7 : g->ks->spmv_kind(g->ls, g->prec)) : 0;
   out->j_bytes = d.J ? (int64_t)(g->j_elems * jt_size(g->prec)) : 0;
   return GPO_OK;
 }
@@ -1741,6 +2024,7 @@ gpo_status gpo_debug_step(gpo_graph* g, double lambda, const gpo_lm_params* para
   fill_scalars(g, prm, lambda, sc);
   if ((s = upload_scalars(g, sc)) != GPO_OK) return s;
   g->ks->cam_prepare(g->ls, false, g->stream);
+  if ((s = begin_solves(g, g->ls)) != GPO_OK) return s;
   if ((s = solve_system(g, g->ls, sc.max_it, true)) != GPO_OK) return s;
   const DevBA& d = g->dev;
   const int DB = g->ks->DB;
@@ -1750,7 +2034,7 @@ gpo_status gpo_debug_step(gpo_graph* g, double lambda, const gpo_lm_params* para
   if ((s = fetch(g, xraw, static_cast<const char*>(d.x), (size_t)DB * d.C * sA)) != GPO_OK) return s;
   if ((s = fetch(g, xbraw, static_cast<const char*>(d.xbest), (size_t)DB * d.C * sA)) != GPO_OK) return s;
   if ((s = fetch(g, praw, static_cast<const char*>(d.dp), 3 * (size_t)d.P * sA)) != GPO_OK) return s;
-  GPO_CUDA(g, cudaStreamSynchronize(g->stream));
+  if ((s = end_solves(g, g->ls)) != GPO_OK) return s;
   const Scalars* hs = reinterpret_cast<const Scalars*>(sraw.data());
   const std::vector<char>& xs = hs->use_best ? xbraw : xraw;
   if (pcg_iters) *pcg_iters = hs->pcg_it;
@@ -1783,12 +2067,14 @@ gpo_status gpo_debug_wait_timeout(gpo_graph* g) {
   if ((s = upload_scalars(g, sc)) != GPO_OK) return s;
   g->ks->cam_prepare(g->ls, false, g->stream);
   g->ks->linearize(g->ls, g->prec, true, g->stream);
-  g->ks->schur_prepare(g->ls, g->prec, g->stream);
-  GPO_CUDA(g, cudaMemsetAsync(g->ls.running, 0, 6 * sizeof(int), g->stream));
-  g->ks->cam_finalize(g->ls, g->prec, g->stream);
   gpo::LaunchSet ls = g->ls;
+  if (!ls.n_xg) ls.ex = 0;   // a cluster's solve has no such wait: the matrix-free camera kernel's
+  if (ls.ex) g->ks->ex_form(ls, g->prec, g->stream);
+  else g->ks->schur_prepare(ls, g->prec, g->stream);
+  GPO_CUDA(g, cudaMemsetAsync(g->ls.running, 0, 6 * sizeof(int), g->stream));
+  g->ks->cam_finalize(ls, g->prec, g->stream);
   ls.debug_wait = 1;   // one CTA more than the grid: nothing completes the barrier
-  const int fused = g->ks->pcg_camera(ls, g->prec, g->stream);
+  const int fused = ls.ex ? g->ks->ex_pcg(ls, g->prec, g->stream) > 0 : g->ks->pcg_camera(ls, g->prec, g->stream);
   GPO_CUDA(g, cudaGetLastError());
   int flags[2] = {0, 0};
   GPO_CUDA(g, cudaMemcpyAsync(flags, ls.running, sizeof(flags), cudaMemcpyDeviceToHost, g->stream));
@@ -1796,7 +2082,7 @@ gpo_status gpo_debug_wait_timeout(gpo_graph* g) {
   GPO_CUDA(g, cudaMemsetAsync(g->ls.running, 0, 6 * sizeof(int), g->stream));   // leave clean counters
   GPO_CUDA(g, cudaStreamSynchronize(g->stream));
   if (!fused) return fail(g, GPO_ERR_UNSUPPORTED, "the camera blocks do not fit one resident wave");
-  if (flags[1]) return fail(g, GPO_ERR_TIMEOUT, "the camera kernel's grid barrier gave up");
+  if (flags[1]) return fail(g, GPO_ERR_TIMEOUT, "the PCG kernel's grid barrier gave up");
   return fail(g, GPO_ERR_STATE, "the grid barrier did not give up");
 }
 
@@ -1813,7 +2099,8 @@ gpo_status gpo_debug_schur(gpo_graph* g, double lambda, const gpo_lm_params* par
   const gpo::KernelSet& ks = *g->ks;
   ks.cam_prepare(g->ls, false, g->stream);
   ks.linearize(g->ls, g->prec, true, g->stream);
-  ks.schur_prepare(g->ls, g->prec, g->stream);
+  if (g->ls.ex) ks.ex_form(g->ls, g->prec, g->stream);
+  else ks.schur_prepare(g->ls, g->prec, g->stream);
   GPO_CUDA(g, cudaMemsetAsync(g->ls.running, 0, sizeof(int), g->stream));
   ks.cam_finalize(g->ls, g->prec, g->stream);
   GPO_CUDA(g, cudaGetLastError());

@@ -34,6 +34,7 @@ struct BatchSet {
   gpo::LaunchSet ls{};
   char* mem = nullptr;
   Scalars* staging = nullptr;    // device [n]
+  std::vector<int4> grids;       // problems whose PCG takes a whole grid (ls.xg_host)
   int n = 0;
 
   void release(cudaStream_t st) {
@@ -47,7 +48,9 @@ gpo_status build_set(gpo_graph* owner, const std::vector<gpo_graph*>& gs, BatchS
   const int n = (int)gs.size();
   std::vector<DevBA> probs(n);
   std::vector<int> ch_prob, cb_prob, pb_prob, ch_base(n), cb_base(n), pb_base(n);
-  int ch_max = 32, ns_max = 1, np_max = 1;
+  std::vector<int> xf_prob, xd_prob, cl_prob, xf_base(n), xd_base(n);   // explicit Schur complement
+  int ch_max = 32, ns_max = 1, np_max = 1, mf = 0, ex = 0, cl_smem = 0;
+  out.grids.clear();
   for (int q = 0; q < n; ++q) {
     const gpo_graph* g = gs[q];
     probs[q] = g->dev;
@@ -60,12 +63,28 @@ gpo_status build_set(gpo_graph* owner, const std::vector<gpo_graph*>& gs, BatchS
     ch_max = std::max(ch_max, g->ls.ch_max);
     ns_max = std::max(ns_max, g->ls.ns_max);
     np_max = std::max(np_max, g->ls.np_max);
+    xf_base[q] = (int)xf_prob.size();
+    xd_base[q] = (int)xd_prob.size();
+    if (!g->ls.ex) {
+      mf = 1;
+      continue;
+    }
+    ex = 1;
+    xf_prob.insert(xf_prob.end(), g->ls.n_xf, q);
+    xd_prob.insert(xd_prob.end(), g->ls.n_xd, q);
+    if (g->ex_cluster) {
+      cl_prob.push_back(q);
+      cl_smem = std::max(cl_smem, g->ex_grid.z);
+    } else {
+      out.grids.push_back(make_int4(q, g->ex_grid.y, g->ex_grid.z, g->ex_grid.w));
+    }
   }
   auto al = [](size_t b) { return (b + 255) / 256 * 256; };
   const size_t b_probs = al(n * sizeof(DevBA)), b_stage = al(n * sizeof(Scalars));
   const size_t b_ch = al(std::max<size_t>(1, ch_prob.size()) * 4), b_cb = al(std::max<size_t>(1, cb_prob.size()) * 4);
   const size_t b_pb = al(std::max<size_t>(1, pb_prob.size()) * 4), b_base = al(n * 4);
-  const size_t total = b_probs + b_stage + b_ch + b_cb + b_pb + 3 * b_base + 256;
+  const size_t b_xf = al(std::max<size_t>(1, xf_prob.size()) * 4), b_xd = al(std::max<size_t>(1, xd_prob.size()) * 4);
+  const size_t total = b_probs + b_stage + b_ch + b_cb + b_pb + b_xf + b_xd + 6 * b_base + 256;
   cudaStream_t st = owner->stream;
   char* mem = nullptr;
   GPO_CUDA(owner, cudaMallocAsync(reinterpret_cast<void**>(&mem), total, st));
@@ -80,6 +99,18 @@ gpo_status build_set(gpo_graph* owner, const std::vector<gpo_graph*>& gs, BatchS
   int* cbb_d = reinterpret_cast<int*>(take(b_base));
   int* pbb_d = reinterpret_cast<int*>(take(b_base));
   int* running_d = reinterpret_cast<int*>(take(256));
+  int* xf_d = reinterpret_cast<int*>(take(b_xf));
+  int* xd_d = reinterpret_cast<int*>(take(b_xd));
+  int* xfb_d = reinterpret_cast<int*>(take(b_base));
+  int* xdb_d = reinterpret_cast<int*>(take(b_base));
+  int* cl_d = reinterpret_cast<int*>(take(b_base));
+  if (!xf_prob.empty()) GPO_CUDA(owner, cudaMemcpyAsync(xf_d, xf_prob.data(), xf_prob.size() * 4, cudaMemcpyHostToDevice, st));
+  if (!xd_prob.empty()) GPO_CUDA(owner, cudaMemcpyAsync(xd_d, xd_prob.data(), xd_prob.size() * 4, cudaMemcpyHostToDevice, st));
+  if (!cl_prob.empty()) GPO_CUDA(owner, cudaMemcpyAsync(cl_d, cl_prob.data(), cl_prob.size() * 4, cudaMemcpyHostToDevice, st));
+  if (ex) {
+    GPO_CUDA(owner, cudaMemcpyAsync(xfb_d, xf_base.data(), n * 4, cudaMemcpyHostToDevice, st));
+    GPO_CUDA(owner, cudaMemcpyAsync(xdb_d, xd_base.data(), n * 4, cudaMemcpyHostToDevice, st));
+  }
   GPO_CUDA(owner, cudaMemcpyAsync(probs_d, probs.data(), n * sizeof(DevBA), cudaMemcpyHostToDevice, st));
   if (!ch_prob.empty()) GPO_CUDA(owner, cudaMemcpyAsync(ch_d, ch_prob.data(), ch_prob.size() * 4, cudaMemcpyHostToDevice, st));
   if (!cb_prob.empty()) GPO_CUDA(owner, cudaMemcpyAsync(cb_d, cb_prob.data(), cb_prob.size() * 4, cudaMemcpyHostToDevice, st));
@@ -106,6 +137,16 @@ gpo_status build_set(gpo_graph* owner, const std::vector<gpo_graph*>& gs, BatchS
   ls.ch_max = ch_max;
   ls.ns_max = ns_max;
   ls.np_max = np_max;
+  ls.ex = ex; ls.mf = mf;
+  ls.xf_prob = xf_d; ls.xf_base = xfb_d;
+  ls.xd_prob = xd_d; ls.xd_base = xdb_d;
+  ls.cl_prob = cl_d;
+  ls.xg_host = out.grids.data();
+  ls.n_xf = (int)xf_prob.size();
+  ls.n_xd = (int)xd_prob.size();
+  ls.n_cl = (int)cl_prob.size();
+  ls.n_xg = (int)out.grids.size();
+  ls.cl_smem = cl_smem;
   out.ls = ls;
   out.mem = mem;
   out.staging = stage_d;
@@ -269,11 +310,13 @@ gpo_status gpo_optimize_batch(gpo_graph* const* graphs, int32_t n, int32_t max_i
         break;
       }
     }
+    if (s == GPO_OK && (s = ensure_runtime(owner)) == GPO_OK) s = begin_solves(owner, bs.ls);
     for (int it = 0; s == GPO_OK && it < max_iters; ++it) {
       owner->cur_lm_iter = -1;
       if ((s = solve_system(owner, bs.ls, max_it, false)) != GPO_OK) break;
       s = finish_iteration(owner, bs.ls);
     }
+    if (s == GPO_OK) s = end_solves(owner, bs.ls);
     if (s == GPO_OK && (s = get_scalars(owner, bs, sc)) == GPO_OK) {
       for (int i = 0; i < n; ++i) {
         graphs[i]->last_cost = sc[i].cost;
@@ -452,8 +495,10 @@ gpo_status gpo_server_step(gpo_server* sv, int32_t* n_resident, int32_t* n_queue
     int max_it = 1;
     for (auto& r : sv->resident) max_it = std::max(max_it, r.prm.pcg_max_iters);
     owner->cur_lm_iter = -1;
-    gpo_status s = solve_system(owner, sv->set.ls, max_it, false);
+    gpo_status s = begin_solves(owner, sv->set.ls);
+    if (s == GPO_OK) s = solve_system(owner, sv->set.ls, max_it, false);
     if (s == GPO_OK) s = finish_iteration(owner, sv->set.ls);
+    if (s == GPO_OK && sv->set.ls.n_xg) s = end_solves(owner, sv->set.ls);
     if (s != GPO_OK) return s;
     ++sv->steps;
     // 3. retirement of graphs that ran all their iterations

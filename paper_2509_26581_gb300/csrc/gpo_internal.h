@@ -29,6 +29,11 @@ constexpr int kMaxDevices = 64;     // per-device launch caches
 constexpr int kGroupEdges = 64;     // edges of a warp group (two per lane) of a chunk
 constexpr int kMaxGroups = 16;      // warp groups per chunk
 constexpr int kMaxHistory = 4096;
+// explicit Schur complement (schur_explicit.cuh)
+constexpr int kExThreads = 512;     // CTA size of the PCG solve
+constexpr int kExCluster = 8;       // CTAs of a small problem's solve (a cluster)
+constexpr int kExGrid = 152;        // CTAs of a larger one's (one per SM)
+constexpr int kExMaxCtas = 160;     // posting slots of a solve
 
 // Edge models (the kernel set a graph runs).
 enum class ModelKind { BA = 0, STEREO = 1 };
@@ -182,6 +187,38 @@ struct DevBA {
   int ch_max;                // max edges per chunk
   int ns_max, np_max;        // max slots / points of a chunk
   int ncblk;                 // CTAs of the camera kernels
+  // explicit Schur complement (ex = 0: none planned, the product is matrix-free).  Block
+  // rows hold the cameras that share points with a camera, both triangles, columns
+  // ascending; "upper" blocks are those right of the diagonal, numbered row by row
+  int ex;
+  int ex_nb, ex_nbu;         // off-diagonal blocks, upper ones
+  int ex_nd, ex_nxf;         // work items of k_ex_diag, CTAs of k_ex_form
+  int ex_seg, ex_dseg;       // row pairs of a k_ex_form item, camera rows of a k_ex_diag item
+  const int* ex_row;         // [C+1] block rows
+  const int* ex_col;         // [ex_nb] camera of a block's column
+  const int* ex_uoff;        // [C+1] upper blocks of a row
+  const int2* ex_ublk;       // [ex_nbu] positions of an upper block and its transpose
+  const int* ex_crow;        // [C+1] camera-major rows (edges) of a camera
+  const int* ex_slot_y0;     // [NS] camera-major row of a slot's first edge
+  const int* ex_doff;        // [C+1] k_ex_diag items of a camera
+  const int* ex_dcam;        // [ex_nd] camera of an item
+  int* ex_poff;              // [ex_nbu + 1] row pairs of an upper block
+  int2* ex_pair;             // row pairs (camera-major rows of the two edges of one point)
+  int4* ex_item;             // k_ex_form items: pair range, upper block, partial (-1: none)
+  int4* ex_multi;            // blocks of several items: block, first partial, partials
+  int* ex_count;             // [2] items, blocks of several items
+  void* ex_Y;                // camera-major rows (16-byte pieces in tiles of 32 rows)
+  void* ex_S;                // AT [ex_nb][DC * DC] blocks, column-major
+  void* ex_part;             // AT [partials][DC * DC]
+  void* ex_dpart;            // AT [ex_nd][NPA] diagonal partials, laid out as a slot partial
+  const int* ex_loff;        // [CTAs + 1] column sets of the PCG solve's CTAs (the cameras its
+                             // rows touch and its own, ascending)
+  const int* ex_lcol;        // ... their cameras
+  const int* ex_lidx;        // [ex_nb] a block's column in its row's CTA's set
+  const int* ex_lown;        // [C] a row's own camera in its CTA's set
+  const int* ex_xl;          // [2 NX] xk_list entry's other camera in the row's CTA's set (-1: none)
+  unsigned long long* ex_red;   // [2][kExMaxCtas][4] posted partial sums of the PCG solve, and their count
+  unsigned long long* ex_z;     // [C][DB] posted z (one word in FP32, two in FP64)
 };
 
 enum class Prec { F64 = 0, F32 = 1, BF16 = 2 };
@@ -213,6 +250,16 @@ struct LaunchSet {
   int nprob, n_ch, n_cb, n_pb;
   int ch_max;            // largest chunk over the problems (shared-memory sizing)
   int ns_max, np_max;    // most slots / points in one chunk over the problems
+  // explicit Schur complement: problems that use it (DevBA::ex; 0: none of the launch
+  // uses it, whatever they have planned), problems that do not
+  int ex, mf;
+  const int* xf_prob; const int* xf_base;   // CTAs of k_ex_form and k_ex_merge
+  const int* xd_prob; const int* xd_base;   // CTAs of k_ex_diag
+  const int* cl_prob;                       // problems solved by a cluster each
+  const int4* xg_host;                      // host memory: problems solved by a grid (problem, CTAs, shared memory, resident blocks)
+  int n_xf, n_xd, n_cl, n_xg;
+  int cl_smem;                              // most shared memory of a cluster's problem
+  void* ex_scratch;                         // k_ex_rows' output while the plan is made
 };
 
 // Kernel set of one edge model.  Every launcher is asynchronous on `st` and returns
@@ -237,6 +284,15 @@ struct KernelSet {
   int (*full_update)(const LaunchSet& ls, Prec pr, cudaStream_t st);
   // forward-mode automatic differentiation of the observation edges (checker)
   int (*autodiff)(const LaunchSet& ls, int n_edges, double* r, double* J, cudaStream_t st);
+  // explicit Schur complement: row pairs and work items of one graph (once, after its
+  // upload); camera rows, diagonal and off-diagonal blocks; the PCG solves (negative: a
+  // launch was refused)
+  int (*ex_plan)(const LaunchSet& ls, Prec pr, int C, int nb_max, int E, cudaStream_t st);
+  int (*ex_form)(const LaunchSet& ls, Prec pr, cudaStream_t st);
+  int (*ex_pcg)(const LaunchSet& ls, Prec pr, cudaStream_t st);
+  size_t (*ex_smem)(Prec pr, int C, int G, int nloc, int nres);   // shared memory of a solve by G CTAs
+  bool (*ex_grid_ok)(Prec pr, size_t smem);                       // a grid solve with that much can be launched
+  void (*ex_sizes)(Prec pr, size_t* row_bytes, int* per_cta_d);   // bytes of a camera row, diag items per CTA
   int (*backsub)(const LaunchSet& ls, Prec pr, cudaStream_t st);
   int (*retract)(const LaunchSet& ls, Prec pr, cudaStream_t st);
   int (*decide)(const LaunchSet& ls, Prec pr, cudaStream_t st);

@@ -20,11 +20,12 @@ using gpo::Scalars;
 enum KernelKind {
   KK_CAM_PREPARE, KK_COST, KK_COST_REDUCE, KK_LINEARIZE, KK_SCHUR, KK_CAM_FINALIZE, KK_SPMV,
   KK_CAM_APPLY, KK_PCG_UPDATE, KK_BACKSUB, KK_RETRACT, KK_DECIDE, KK_COMMIT, KK_PCG_CAMERA,
-  KK_FULL_INIT, KK_AUTODIFF, KK_COUNT
+  KK_FULL_INIT, KK_AUTODIFF, KK_EX_FORM, KK_EX_PCG, KK_COUNT
 };
 inline const char* const kKernelNames[KK_COUNT] = {
     "cam_prepare", "cost", "cost_reduce", "linearize", "schur_prepare", "cam_finalize", "spmv",
-    "cam_apply", "pcg_update", "backsub", "retract", "decide", "commit", "pcg_camera", "full_init", "autodiff"};
+    "cam_apply", "pcg_update", "backsub", "retract", "decide", "commit", "pcg_camera", "full_init", "autodiff",
+    "schur_form", "pcg_solve"};
 
 struct Profiler {
   bool on = false;
@@ -99,6 +100,8 @@ struct gpo_graph {
   size_t full_bytes = 0;
   DevBA dev{};
   gpo::LaunchSet ls{};             // one-problem launch set over `dev`
+  bool ex_cluster = false;         // explicit Schur complement: solved by a cluster (else a grid)
+  int4 ex_grid{0, 0, 0, 0};        // the solve's launch (problem, CTAs, shared memory)
   DevBA* dev_desc = nullptr;       // device copy of `dev` (ls.probs)
   Scalars* h_sc = nullptr;         // pinned
   int* h_flag = nullptr;           // pinned [2]
@@ -146,6 +149,9 @@ gpo_lm_params params_or_default(const gpo_lm_params* p);
 // One LM iteration's solve (linearise, Schur, PCG, back-substitution) over `ls`
 // on g's stream, counting launches in g's profiler.
 gpo_status solve_system(gpo_graph* g, const gpo::LaunchSet& ls, int max_it, bool force_lin);
+// Around the solves of a call: clear their flags; wait, and report a wait that gave up.
+gpo_status begin_solves(gpo_graph* g, const gpo::LaunchSet& ls);
+gpo_status end_solves(gpo_graph* g, const gpo::LaunchSet& ls);
 // Retraction, candidate cost, decision and commit over `ls`.
 gpo_status finish_iteration(gpo_graph* g, const gpo::LaunchSet& ls);
 // Camera render blocks, F(x) and its per-problem reduction over `ls` (no sync).

@@ -479,7 +479,7 @@ __global__ void __launch_bounds__(kThreads) k_schur_prepare(LaunchSet ls) {
   using R = SchurRec<Mo, AT>;
   constexpr int M = Mo::M, DC = Mo::DC, NJ = Mo::NJ, JP0 = Dm::JP0, RSY = R::RSY, RSG = R::RSG;
   GPO_BIND(ch, kl)
-  if (!d.sc->active) return;
+  if (!d.sc->active || (ls.ex && d.ex)) return;
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int next_slot;
   const int CH = d.ch_max;
@@ -586,6 +586,14 @@ __global__ void __launch_bounds__(kCamPerBlock * 32) k_cam_finalize(LaunchSet ls
   if (!d.sc->active) return;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int c = cbl * kCamPerBlock + warp;
+  const bool ex = ls.ex && d.ex;
+  if (ex) {   // no epoch of the coming PCG solve is posted yet
+    if (cbl == 0)
+      for (int i = threadIdx.x; i < 8 * kExMaxCtas + 1; i += blockDim.x) d.ex_red[i] = 0ull;
+    constexpr int ZC = DB * (int)(sizeof(AT) / 4);   // words of a camera's z
+    for (int i = threadIdx.x; i < kCamPerBlock * ZC; i += blockDim.x)
+      if (cbl * kCamPerBlock + i / ZC < d.C) d.ex_z[(size_t)cbl * kCamPerBlock * ZC + i] = 0ull;
+  }
   Scalars* sc = d.sc;
   const AT lam = (AT)sc->lambda;
   const AT* partA = reinterpret_cast<const AT*>(d.partA);
@@ -594,8 +602,17 @@ __global__ void __launch_bounds__(kCamPerBlock * 32) k_cam_finalize(LaunchSet ls
   if (c < d.C) {
     const int sa = d.cam_s_off[c], sb = d.cam_s_off[c + 1];
     // 2 NG groups of nine outputs; lanes stride over the camera's slots, then a fixed
-    // shuffle tree sums the lanes
-    for (int grp = 0; grp < 2 * NG; ++grp) {
+    // shuffle tree sums the lanes.  With the explicit Schur complement the second NG
+    // groups are the camera's diagonal partials, added in order
+    if (ex) {
+      const AT* dp = reinterpret_cast<const AT*>(d.ex_dpart);
+      for (int t = lane; t < NPA; t += 32) {
+        AT s = (AT)0;
+        for (int k = d.ex_doff[c]; k < d.ex_doff[c + 1]; ++k) s += dp[(size_t)k * NPA + t];
+        vals[warp][NPA + t] = s;
+      }
+    }
+    for (int grp = 0; grp < (ex ? NG : 2 * NG); ++grp) {
       const AT* base = (grp < NG ? partA : partB) + 9 * (grp % NG);
       AT acc[9];
 #pragma unroll
@@ -758,7 +775,7 @@ __global__ void __launch_bounds__(kCamPerBlock * 32) k_cam_finalize(LaunchSet ls
     sc->pcg_fail = (rr > 0.0 && (!(rz > 0.0) || !isfinite(rz))) ? 1 : 0;
     sc->pcg_breakdown = 0;
     sc->have_best = 0;
-    if (!sc->pcg_done) atomicAdd(ls.running, 1);
+    if (!sc->pcg_done && !ex) atomicAdd(ls.running, 1);
     sc->ticket = 0u;
   }
 }
@@ -1210,17 +1227,18 @@ __global__ void __launch_bounds__(kCamPerBlock * 32) k_pcg_update(LaunchSet ls) 
   pcg_update_body<Mo, AT>(ls, d, cbl, red, in);
 }
 
-__device__ __forceinline__ unsigned long long global_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+__device__ __forceinline__ long long sm_clock() {
+  long long t;
+  asm volatile("mov.u64 %0, %%clock64;" : "=l"(t));
   return t;
 }
-constexpr unsigned long long kWaitNs = 1000000000ull;   // bounded waits give up after 1 s
+// Bounded waits give up after this many clocks of the SM (about a second near 2.07 GHz).
+constexpr long long kWaitClocks = 2000000000ll;
 
 // Grid-wide barrier of the persistent camera kernel (every CTA resident; called after a
 // CTA barrier): thread 0 arrives with an acquire-release add, the last CTA to arrive
 // resets the count and advances the generation with a release add, and the others
-// wait for it with acquire loads.  The wait is bounded (kWaitNs of wall time); false if
+// wait for it with acquire loads.  The wait is bounded (kWaitClocks); false if
 // it gave up (the caller raises *ls.err).
 __device__ __forceinline__ bool grid_sync(int* count, int* gen, int ctas) {
   __shared__ int ok;
@@ -1233,9 +1251,9 @@ __device__ __forceinline__ bool grid_sync(int* count, int* gen, int ctas) {
       atomicExch(ucount, 0u);
       red_add_release(ugen, 1u);
     } else {
-      const unsigned long long t0 = global_ns();
+      const long long t0 = sm_clock();
       while (ld_acquire(ugen) == g0) {
-        if (global_ns() - t0 > kWaitNs) {
+        if (sm_clock() - t0 > kWaitClocks) {
           ok = 0;
           break;
         }
@@ -1595,6 +1613,7 @@ static void set_smem(const void* kernel, size_t bytes) {
 
 #include "schur_full.cuh"
 #include "autodiff.cuh"
+#include "schur_explicit.cuh"
 
 namespace gpo {
 
@@ -2018,6 +2037,102 @@ struct Launch {
     else launch_pdl(k_pcg_update<Mo, float>, ls.n_cb, kCamPerBlock * 32, 0, st, ls);
     return 1;
   }
+  // ---- explicit Schur complement
+  static void ex_sizes(Prec pr, size_t* row_bytes, int* per_cta_d) {
+    *row_bytes = 16 * (size_t)(pr == Prec::F64 ? ExRow<Mo, double>::Q : ExRow<Mo, float>::Q);
+    *per_cta_d = pr == Prec::F64 ? kExDiagWarps<double> : kExDiagWarps<float>;
+  }
+  static int ex_plan(const LaunchSet& ls, Prec, int C, int nb_max, int E, cudaStream_t st) {
+    // scratch: the camera rows' array, not in use yet
+    int* row_edge = static_cast<int*>(ls.ex_scratch);
+    int* e_row = row_edge + E;
+    launch_pdl(k_ex_rows, ls.n_ch, kThreads, 0, st, ls, row_edge, e_row);
+    const size_t sm = 9 * sizeof(int) * (size_t)nb_max;
+    set_smem(reinterpret_cast<const void*>(k_ex_pairs<false>), sm);
+    set_smem(reinterpret_cast<const void*>(k_ex_pairs<true>), sm);
+    k_ex_pairs<false><<<C, kThreads, sm, st>>>(ls, row_edge, e_row, nb_max);
+    k_ex_items<<<1, 1024, 0, st>>>(ls);
+    k_ex_pairs<true><<<C, kThreads, sm, st>>>(ls, row_edge, e_row, nb_max);
+    return 4;
+  }
+  template <class JT>
+  static void ex_form_t(const LaunchSet& ls, cudaStream_t st) {
+    using AT = typename AccOf<JT>::T;
+    const size_t sm = 9 * sizeof(AT) * (size_t)ls.np_max + sizeof(int) * (size_t)ls.ns_max;
+    set_smem(reinterpret_cast<const void*>(k_ex_prepare<Mo, JT>), sm);
+    launch_pdl(k_ex_prepare<Mo, JT>, ls.n_ch, kThreads, sm, st, ls);
+    launch_pdl(k_ex_diag<Mo, AT>, ls.n_xd, kExDiagWarps<AT> * 32, 0, st, ls);
+    if (ls.n_xf) {
+      launch_pdl(k_ex_form<Mo, AT>, ls.n_xf, 128, 0, st, ls);
+      launch_pdl(k_ex_merge<Mo, AT>, ls.n_xf, 128, 0, st, ls);
+    }
+  }
+  static int ex_form(const LaunchSet& ls, Prec pr, cudaStream_t st) {
+    if (pr == Prec::F64) ex_form_t<double>(ls, st);
+    else if (pr == Prec::F32) ex_form_t<float>(ls, st);
+    else ex_form_t<__nv_bfloat16>(ls, st);
+    return ls.n_xf ? 4 : 2;
+  }
+  static size_t ex_smem(Prec pr, int C, int G, int nloc, int nres) {
+    return pr == Prec::F64 ? ex_pcg_smem<Mo, double>(C, G, nloc, nres) : ex_pcg_smem<Mo, float>(C, G, nloc, nres);
+  }
+  template <class AT>
+  static bool ex_grid_ok_t(size_t sm) {
+    int dev = 0, n_sm = 0, occ = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+    set_smem(reinterpret_cast<const void*>(k_ex_pcg<Mo, AT, false, true>), sm);   // the form that uses more registers or memory
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_ex_pcg<Mo, AT, false, true>, kExThreads, sm) == cudaSuccess &&
+           occ * n_sm >= kExGrid;
+  }
+  static bool ex_grid_ok(Prec pr, size_t sm) {
+    return pr == Prec::F64 ? ex_grid_ok_t<double>(sm) : ex_grid_ok_t<float>(sm);
+  }
+  template <class AT>
+  static int ex_pcg_t(const LaunchSet& ls, cudaStream_t st) {
+    int n = 0;
+    if (ls.n_cl) {   // one cluster per problem
+      const size_t sm = (size_t)ls.cl_smem;
+      set_smem(reinterpret_cast<const void*>(k_ex_pcg<Mo, AT, true, true>), sm);
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3((unsigned)(ls.n_cl * kExCluster));
+      cfg.blockDim = dim3(kExThreads);
+      cfg.dynamicSmemBytes = sm;
+      cfg.stream = st;
+      cudaLaunchAttribute attr[2];
+      attr[0].id = cudaLaunchAttributeClusterDimension;
+      attr[0].val.clusterDim.x = kExCluster;
+      attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+      attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+      attr[1].val.programmaticStreamSerializationAllowed = 1;
+      cfg.attrs = attr;
+      cfg.numAttrs = 2;
+      if (cudaLaunchKernelEx(&cfg, k_ex_pcg<Mo, AT, true, true>, ls, 0) != cudaSuccess) return -1;
+      ++n;
+    }
+    for (int k = 0; k < ls.n_xg; ++k) {   // one whole (cooperative) grid per problem
+      const int G = ls.xg_host[k].y;
+      const size_t sm = (size_t)ls.xg_host[k].z;
+      auto kernel = ls.xg_host[k].w ? k_ex_pcg<Mo, AT, false, true> : k_ex_pcg<Mo, AT, false, false>;
+      set_smem(reinterpret_cast<const void*>(kernel), sm);
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3((unsigned)G);
+      cfg.blockDim = dim3(kExThreads);
+      cfg.dynamicSmemBytes = sm;
+      cfg.stream = st;
+      cudaLaunchAttribute attr[1];
+      attr[0].id = cudaLaunchAttributeCooperative;
+      attr[0].val.cooperative = 1;
+      cfg.attrs = attr;
+      cfg.numAttrs = 1;
+      if (cudaLaunchKernelEx(&cfg, kernel, ls, ls.xg_host[k].x) != cudaSuccess) return -1;
+      ++n;
+    }
+    return n;
+  }
+  static int ex_pcg(const LaunchSet& ls, Prec pr, cudaStream_t st) {
+    return pr == Prec::F64 ? ex_pcg_t<double>(ls, st) : ex_pcg_t<float>(ls, st);
+  }
   template <class JT, bool kDyn>
   static void backsub_k(const LaunchSet& ls, Prec pr, cudaStream_t st) {
     const size_t sm = backsub_smem(pr, ls.ch_max);
@@ -2080,6 +2195,12 @@ KernelSet make_kernel_set(ModelKind kind) {
   k.full_spmv = &L::full_spmv;
   k.full_update = &L::full_update;
   k.autodiff = &L::autodiff;
+  k.ex_plan = &L::ex_plan;
+  k.ex_form = &L::ex_form;
+  k.ex_pcg = &L::ex_pcg;
+  k.ex_smem = &L::ex_smem;
+  k.ex_grid_ok = &L::ex_grid_ok;
+  k.ex_sizes = &L::ex_sizes;
   k.backsub = &L::backsub;
   k.retract = &L::retract;
   k.decide = &L::decide;

@@ -15,12 +15,10 @@ import numpy as np
 from . import gpo
 
 
-# Schedule of served windows: a server step's launches cover hundreds of windows at once,
-# so the chunking and Schur product that suit a large problem serve them best (512-edge
-# chunks and the pipelined product gave 12 % more solves/s than the single-window tuning
-# of 256-edge chunks on a 2,000 requests/s stream).  The same knobs solve a window alone,
-# so served and lone results stay equal.
-SERVED_KNOBS = dict(chunk_edges=512, spmv_variant=3)
+# Schedule of served windows: the automatic product (explicit: one cluster of CTAs solves a
+# window's whole PCG) with 512-edge chunks.  The same knobs solve a window alone, so served
+# and lone results stay equal.
+SERVED_KNOBS = dict(chunk_edges=512, spmv_variant=0)
 
 
 def window_graph(p, precision: str, fix_first: bool = True, **kw) -> tuple:
