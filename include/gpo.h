@@ -125,9 +125,11 @@ typedef struct {
                                  one launch; it takes device memory for the blocks and
                                  for one row of 3 values per edge and camera coordinate,
                                  and is left out where the memory budget holds the graph
-                                 only without, a camera sees a point twice, or forming
-                                 the blocks costs more than it saves; then pipelined for
-                                 BF16 and FP32 storage, classic for FP64), 1 = staged
+                                 only without, a camera sees a point twice, forming the
+                                 blocks costs more than it saves, or for bundle
+                                 adjustment with BF16 storage, or FP32 and more than
+                                 65,536 points; then pipelined for BF16 and FP32
+                                 storage, classic for FP64), 1 = staged
                                  (persistent CTAs streaming chunks into shared memory
                                  with bulk copies), 2 = classic (one CTA per chunk),
                                  3 = pipelined (persistent CTAs prefetching the next

@@ -225,10 +225,24 @@ struct Prepared {
 
 void PrepDeleter::operator()(Prepared* p) const { delete p; }
 
+// Whether the automatic product may be the explicit one.  With FP32 or BF16 storage the
+// explicit blocks round in another order than the matrix-free product, and bundle
+// adjustment can magnify that: a step that takes a point next to a camera plane makes the
+// cost depend on the last bits of the camera step, and BF16 rows of the next linearisation
+// round the other way.  Of scenes with 250,000 points and more, one in five or eight had a
+// final cost that moved by more than 2e-5 (and BF16 windows single points by 1e-3), so
+// there those graphs keep the matrix-free product bit for bit.  Stereo points lie in front
+// of their cameras by their measured disparity (costs moved by 7e-7 at most).
+static bool explicit_allowed(const gpo_graph* g, const gpo::KernelSet& ks, int P) {
+  if (g->desc.spmv_variant != 0) return false;
+  if (g->prec == Prec::F64 || ks.model == gpo::ModelKind::STEREO) return true;
+  return g->prec == Prec::F32 && P <= 65536;
+}
+
 // Plans the explicit Schur complement: which camera pairs share points, the camera-major
-// rows and the work items.  Leaves R.ex false where the product stays matrix-free: a
-// product other than the automatic one was asked for, a camera sees a point twice, or
-// forming the blocks costs more than they save.
+// rows and the work items.  Leaves R.ex false where the product stays matrix-free: it is
+// not allowed (above), a camera sees a point twice, or forming the blocks costs more than
+// they save.
 //
 // The rule compares times on the GB300.  Forming: 0.014 ns per row pair in FP32 (about
 // four cycles per pair and SM), 0.46 ns in FP64 (243 FP64 multiply-adds per pair at the
@@ -237,7 +251,7 @@ void PrepDeleter::operator()(Prepared* p) const { delete p; }
 // TB/s and 6 us.  A solve is taken to have 16 iterations (solves to 1e-6 took 11 to 100).
 static void plan_explicit(gpo_graph* g, Prepared& R, const gpo::KernelSet& ks, int C, int P, int E, int NS) {
   R.ex = false;
-  if (g->desc.spmv_variant != 0 || E == 0 || C < 2 || C > 32768) return;
+  if (!explicit_allowed(g, ks, P) || E == 0 || C < 2 || C > 32768) return;
   int64_t pairs = 0;
   for (int p = 0; p < P; ++p) {
     const int64_t k = R.pt_off[p + 1] - R.pt_off[p];
@@ -428,11 +442,12 @@ static gpo_status prepare(gpo_graph* g) {
   if (!pp) return fail(g, GPO_ERR_OOM, "host allocation failed");
   Prepared& R = *pp;
 
-  // point order: by the smallest, then the largest camera index among the point's active
-  // edges (points without active edges last), ties by point index.  Consecutive points
-  // then share cameras, which keeps the per-chunk camera slot count small, and points with
-  // the same span of cameras are adjacent, which makes the rows that a pair of cameras
-  // shares (k_ex_form) runs of consecutive ones.
+  // point order: by the smallest camera index among the point's active edges (points
+  // without active edges last), ties by point index.  Consecutive points then share
+  // cameras, which keeps the per-chunk camera slot count small.  Where the explicit Schur
+  // complement may be used, ties go by the largest camera index first: points with the same
+  // span of cameras are then adjacent, which makes the rows that a pair of cameras shares
+  // (k_ex_form) runs of consecutive ones.
   std::vector<int32_t> key(P, C), last(P, 0);
   std::vector<int32_t> deg(P, 0);
   for (int64_t e = 0; e < Eall; ++e)
@@ -443,6 +458,7 @@ static gpo_status prepare(gpo_graph* g) {
       deg[p]++;
     }
   std::vector<int32_t> cnt(C + 2, 0), by_last(P);
+  if (!explicit_allowed(g, ks, P)) std::fill(last.begin(), last.end(), 0);
   for (int p = 0; p < P; ++p) cnt[last[p] + 1]++;
   for (int k = 0; k <= C; ++k) cnt[k + 1] += cnt[k];
   for (int p = 0; p < P; ++p) by_last[cnt[last[p]]++] = p;

@@ -434,12 +434,6 @@ __global__ void __launch_bounds__(128) k_ex_merge(LaunchSet ls) {
 
 // ---------------------------------------------------------------- the PCG solve
 
-// Scalars of a solve, the same in every lane of warp 0 of every CTA.
-struct ExState {
-  double rz, sigma, rnorm, rmin, tol_abs, ratio;
-  int pcg_it, max_it, normalize, restart_every, products, total;
-};
-
 __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
@@ -516,11 +510,30 @@ struct ExWait {
   __device__ __forceinline__ bool again() const { return sm_clock() - t0 < kWaitClocks; }
 };
 
-// Half the smallest power of two holding n lanes (at most a warp).
-__device__ __forceinline__ int tree_half(int n) {
-  int m = 1;
-  while (m < n && m < 32) m <<= 1;
-  return m >> 1;
+// Sum over a warp, the same in every lane.  FP64 additions take a sub-partition's pipe some 70 clocks each on this part, so the
+// values are added as 64-bit integers on the scale of the largest: a value's 53-bit
+// significand is shifted to leave room for n terms (bits below 2^-52 of the largest term and
+// less are cut, as roundings of a floating sum cut them), and the order does not matter.
+// Infinities, NaN and values near the smallest exponents are added as they are.
+// Here: the sum of the lanes' v, n values in all (the lanes past n hold zero).
+static __device__ __noinline__ double ex_warp_sum(double v, int n) {
+  constexpr unsigned full = 0xffffffffu;
+  const long long b = __double_as_longlong(v);
+  const int x = (int)(b >> 52) & 0x7ff, e = __reduce_max_sync(full, x);
+  if (e == 0x7ff || e < 128) {
+#pragma unroll 1
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(full, v, o);
+    return v;
+  }
+  const int room = 5 - (n > 1 ? 32 - __clz(n - 1) : 0) + 4;   // 2^53 terms n of them fit 62 bits when shifted by this
+  const int sh = e - x - room;                                // right shift
+  const long long m = (b & 0xfffffffffffffll) | 0x10000000000000ll;
+  long long q = x == 0 || sh > 62 ? 0ll : (sh >= 0 ? m >> sh : m << -sh);
+  if (b < 0) q = -q;
+#pragma unroll 1
+  for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(full, q, o);
+  // q 2^(e - 1023 - 52 - room)
+  return __ll2double_rn(q) * __hiloint2double((e - 52 - room) << 20, 0);
 }
 
 // Rows of a CTA: ceil(C / G) consecutive cameras; `wpr` warps share a row.
@@ -530,36 +543,122 @@ __host__ __device__ inline int ex_warps_per_row(int rpc) {
   while (w > 1 && w * rpc > kExThreads / 32) w >>= 1;
   return w;
 }
-// Shared memory of a solve: nloc cameras in a CTA's column set; nres: most blocks of a CTA's rows if they are kept in shared memory, else 0.
+// A camera's vector in shared memory: coordinate k of the first DC at (k mod 3) GS + k / 3, so
+// that a lane's coordinates of a block (columns k mod 3 = its column group) are one vector
+// load; the remaining coordinates after them.
+template <class Mo, class AT>
+struct ExVec {
+  static constexpr int DC = Mo::DC, DB = Mo::DB, ST = DC / 3, GS = ST == 3 ? 4 : 2;
+  static constexpr int VP = 16 / (int)sizeof(AT);
+  static constexpr int W = (3 * GS + DB - DC + VP - 1) / VP * VP;   // values of a camera
+  __device__ static __forceinline__ int at(int k) { return k < DC ? (k % 3) * GS + k / 3 : 3 * GS + k - DC; }
+  // the ST coordinates of column group cg
+  __device__ static __forceinline__ void group(const AT* v, int cg, AT (&o)[ST]) {
+    const AT* p = v + cg * GS;
+    if constexpr (sizeof(AT) == 4 && ST == 3) {
+      const float4 q = *reinterpret_cast<const float4*>(p);
+      o[0] = q.x; o[1] = q.y; o[2] = q.z;
+    } else if constexpr (sizeof(AT) == 4) {
+      const float2 q = *reinterpret_cast<const float2*>(p);
+      o[0] = q.x; o[1] = q.y;
+    } else {
+      const double2 q = *reinterpret_cast<const double2*>(p);
+      o[0] = q.x; o[1] = q.y;
+      if constexpr (ST == 3) o[2] = p[2];
+    }
+  }
+};
+// Shared memory of a solve: nloc cameras in a CTA's column set; nres: most blocks of a CTA's
+// rows if they are kept in shared memory, else 0.
 template <class Mo, class AT>
 __host__ __device__ inline size_t ex_pcg_smem(int C, int G, int nloc, int nres) {
   const int rpc = ex_rows_per_cta(C, G), PW = Mo::kExtra ? Mo::DB : Mo::DC;
-  return sizeof(double) * 2 * (size_t)rpc + sizeof(int) * (size_t)nres +
-         sizeof(AT) * (Mo::DC * Mo::DC * (size_t)nres + (size_t)rpc * Mo::DB * 5 + 2 * (size_t)nloc * Mo::DB + (size_t)rpc * ex_warps_per_row(rpc) * PW);
+  return sizeof(AT) * (2 * (size_t)nloc * ExVec<Mo, AT>::W + Mo::DC * Mo::DC * (size_t)nres +
+                       (size_t)rpc * Mo::DB * (7 + 2 * Mo::DB) + (size_t)rpc * ex_warps_per_row(rpc) * PW) +
+         sizeof(int) * (size_t)nres;
+}
+
+// The sum over a group of CTAs of each one's v[0 .. n-1], by one warp: value w (0 or 1) of the
+// reduction `epoch`; value 1 takes part in every second one.  slot_s: [2][kExCluster][4] words
+// in the CTA's shared memory (a cluster's slots); red: [2][kExMaxCtas][4] words and the two
+// counts of posts (a grid's).  n_slot: CTAs of the group.  Sets *lost on a wait that gave up.
+template <class AT, bool kCluster>
+__device__ __noinline__ double ex_group_sum(const AT* v, int n, int w, unsigned epoch, int rank, int n_slot,
+                                            unsigned long long* slot_s, unsigned long long* red, int* lost) {
+  constexpr unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31, par = epoch & 1;
+  double mine = 0.0;
+#pragma unroll 1
+  for (int i = lane; i < n; i += 32) mine += (double)v[i];
+  mine = ex_warp_sum(mine, 32);
+  ExWait wait;
+  bool ok = true;
+  if constexpr (kCluster) {
+    if (lane < kExCluster) ex_post_cluster(cluster_addr(slot_s + (par * kExCluster + rank) * 4 + 2 * w, lane), mine, epoch);
+    double u = 0.0;
+    if (lane < kExCluster)
+      while (!ex_poll_shared(slot_s + (par * kExCluster + lane) * 4 + 2 * w, u, epoch) && (ok = wait.again())) {}
+    if (!__all_sync(full, ok)) *lost = 1;
+    return ex_warp_sum(u, kExCluster);
+  } else {
+    constexpr int PS = (kExGrid + 32) / 32;   // slots per lane, one more than the grid's
+    unsigned long long* slots = red + (size_t)par * 4 * kExMaxCtas + 2 * w;
+    // one lane polls a count of the posts first: every CTA polling every slot while the last
+    // CTAs arrive keeps the few L2 lines of the slots so busy that the posts wait
+    if (lane == 0) {
+      unsigned* count = reinterpret_cast<unsigned*>(red + 8 * kExMaxCtas + w);
+      ex_post(slots + 4 * rank, mine, epoch);
+      asm volatile("red.relaxed.gpu.add.u32 [%0], %1;" ::"l"(count), "r"(1u) : "memory");
+      const unsigned want = (unsigned)n_slot * (w ? epoch / 2 : epoch);
+      unsigned c;
+      do asm volatile("ld.relaxed.gpu.u32 %0, [%1];" : "=r"(c) : "l"(count) : "memory");
+      while (c < want && (ok = wait.again()));
+    }
+    ok = __shfl_sync(full, (int)ok, 0);
+    double u[PS];
+    bool all;
+    do {
+      all = true;
+#pragma unroll
+      for (int k = 0; k < PS; ++k) {
+        u[k] = 0.0;
+        if (lane + 32 * k < n_slot) all = ex_poll(slots + 4 * (lane + 32 * k), u[k], epoch) && all;
+      }
+    } while (!__all_sync(full, all) && (ok = __all_sync(full, ok && wait.again())));
+    if (!ok) *lost = 1;
+#pragma unroll
+    for (int k = 1; k < PS; ++k) u[0] += u[k];
+    return ex_warp_sum(u[0], 32);
+  }
 }
 
 // The whole solve of one problem by a group of CTAs: a cluster of kExCluster (small
 // problems; several in one launch) or a grid of up to kExGrid (cooperative launch).  A CTA
 // owns consecutive block rows and keeps the search direction p of every camera its rows
-// touch (its column set) in shared memory, updated there as p = (z + beta p) / n, so that a
-// product reads only blocks (from L1 after the first iteration, where they fit) and shared
-// memory.  Two group reductions per iteration, p^T S p and then r^T M r with |r|^2, and one
-// exchange of z.  Both travel as words that carry their epoch, which a cluster writes into
-// every CTA's shared memory and a grid into global memory that every CTA polls; a value is
+// touch (its column set) in shared memory, updated there as p = (z + beta p) / n, and its
+// rows' blocks as well where they fit.  Two group reductions per iteration, p^T S p and then
+// r^T M r with |r|^2 (a warp each), and one exchange of z, which the other warps receive
+// while the reduction runs.  Both travel as words that carry their epoch, the partial sums
+// of a cluster into every CTA's shared memory, all else through global memory; a value is
 // overwritten only after a later reduction has shown that every CTA has read it.  Every CTA
-// sums the partials in rank order and so forms the same scalars; rank 0 writes them back.
-// The recurrences, guards and stopping rules are those of k_cam_apply and k_pcg_update.
+// sums the partials in the same way and so forms the same scalars; rank 0 writes them back.
+// The recurrences, guards and stopping rules are those of k_cam_apply and k_pcg_update; the
+// inner products are sums of AT products, added exactly to FP64's precision.
 template <class Mo, class AT, bool kCluster, bool kRes>
 __global__ void __launch_bounds__(kExThreads, 1) k_ex_pcg(LaunchSet ls, int prob0) {
+  using V = ExVec<Mo, AT>;
   constexpr int DC = Mo::DC, DB = Mo::DB, TB = Dims<Mo>::TB, EL = DC * DC, NW = kExThreads / 32;
   constexpr int CG = 3, LN = CG * DC, ST = DC / CG;   // columns per step, lanes in use, steps per block
   constexpr int PW = Mo::kExtra ? DB : DC;
+  constexpr int ZW = sizeof(AT) / 4;                  // words of a value
+  constexpr int ZT = kExThreads - 64, ZK = 4;         // threads that receive z, values each keeps in registers
   constexpr unsigned full = 0xffffffffu;
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ DevBA d;
   __shared__ unsigned long long slot_s[2][kExCluster][4];
-  __shared__ AT co[5];       // alpha, sigma alpha, 1 / n (of the update), beta, 1 / n (of the direction)
-  __shared__ int fl[4];      // stop, restart, save best, barrier gave up
+  __shared__ double is_s;
+  __shared__ AT co[4];       // alpha, sigma alpha, 1 / n, beta
+  __shared__ int fl[5];      // stop, restart, save best, a wait gave up, r^T M r not positive
   const int G = kCluster ? kExCluster : (int)gridDim.x, rank = (int)blockIdx.x % G;
   const int q = kCluster ? ls.cl_prob[blockIdx.x / kExCluster] : prob0;
   bind_problem(d, ls.probs + q);
@@ -567,186 +666,143 @@ __global__ void __launch_bounds__(kExThreads, 1) k_ex_pcg(LaunchSet ls, int prob
   Scalars* sc = d.sc;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (!sc->active || sc->pcg_done) return;   // the same for every CTA of the group
-  if (!kCluster && *reinterpret_cast<volatile int*>(ls.err)) return;   // an earlier solve's barrier gave up
+  if (!kCluster && *reinterpret_cast<volatile int*>(ls.err)) return;   // an earlier solve's wait gave up
   const int rpc = ex_rows_per_cta(d.C, G), wpr = ex_warps_per_row(rpc), rpp = NW / wpr;
   const int c0 = min(rank * rpc, d.C), nr = min(c0 + rpc, d.C) - c0;
   const int* lcol = d.ex_lcol + d.ex_loff[rank];
   const int nloc = d.ex_loff[rank + 1] - d.ex_loff[rank];
-  double* dot = reinterpret_cast<double*>(smem);                 // [rpc][2]
-  AT* xs = reinterpret_cast<AT*>(dot + 2 * (size_t)rpc);         // [rpc][DB]: x, r, y, g, best x
+  const int b0 = d.ex_row[c0], nb = d.ex_row[c0 + nr] - b0;
+  AT* pl = reinterpret_cast<AT*>(smem);                          // [nloc][V::W] direction
+  AT* xl = pl + (size_t)nloc * V::W;                             // [nloc][V::W] x, with restarts
+  AT* xs = xl + (size_t)nloc * V::W;                             // [rpc][DB]: x, r, y, g, best x, terms of the sums
   AT* rs = xs + (size_t)rpc * DB;
   AT* ys = rs + (size_t)rpc * DB;
   AT* gs = ys + (size_t)rpc * DB;
   AT* bs = gs + (size_t)rpc * DB;
-  AT* part = bs + (size_t)rpc * DB;                              // [rpc][wpr][PW]
-  AT* pl = part + (size_t)rpc * wpr * PW;                        // [nloc][DB] direction
-  AT* xl = pl + (size_t)nloc * DB;                               // [nloc][DB] x, with restarts
-  AT* Sr = xl + (size_t)nloc * DB;                               // the rows' blocks (kRes) ...
-  constexpr int ZW = sizeof(AT) / 4;                             // words of a value
-  unsigned long long* zw = d.ex_z;                               // z as words
+  AT* da = bs + (size_t)rpc * DB;
+  AT* db = da + (size_t)rpc * DB;
+  AT* Ss = db + (size_t)rpc * DB;                                // [rpc][DB][DB] diagonal blocks, preconditioner
+  AT* Ms = Ss + (size_t)rpc * DB * DB;
+  AT* part = Ms + (size_t)rpc * DB * DB;                         // [rpc][wpr][PW]
+  AT* Sr = part + (size_t)rpc * wpr * PW;                        // the rows' blocks (kRes) ...
+  int* li_s = reinterpret_cast<int*>(Sr + (size_t)nb * EL);      // ... and their columns in the set
+  unsigned long long* zw = d.ex_z;
   AT* gx = reinterpret_cast<AT*>(d.x);
   const AT* gz = reinterpret_cast<const AT*>(d.z);
   const AT* Sx = reinterpret_cast<const AT*>(d.ex_S);
-  const AT* Sd = reinterpret_cast<const AT*>(d.S);
-  const AT* Mi = reinterpret_cast<const AT*>(d.Minv);
   const AT* xH = reinterpret_cast<const AT*>(d.xe_H);
+  // The loops of the solve are kept rolled where they are not the work itself: unrolled, the
+  // kernel is 95 KB of instructions, which an iteration fetches anew, and each CTA in turn
+  // is late by the misses (12 us instead of 5 an iteration of a small problem)
+#pragma unroll 1
   for (int i = tid; i < nr * DB; i += kExThreads) {
     xs[i] = bs[i] = (AT)0;
     rs[i] = gs[i] = reinterpret_cast<const AT*>(d.g)[(size_t)c0 * DB + i];
   }
-  for (int i = tid; i < nloc * DB; i += kExThreads) {
-    pl[i] = xl[i] = (AT)0;
+#pragma unroll 1
+  for (int i = tid; i < nr * DB * DB; i += kExThreads) {
+    const int c = c0 + i / (DB * DB), a = i % (DB * DB) / DB, b = i % DB;
+    const size_t o = (size_t)c * TB + sym_idx(DB, a, b);
+    Ss[i] = reinterpret_cast<const AT*>(d.S)[o];
+    Ms[i] = reinterpret_cast<const AT*>(d.Minv)[o];
   }
+#pragma unroll 1
+  for (int i = tid; i < nloc * V::W; i += kExThreads) pl[i] = xl[i] = (AT)0;
   if (kCluster && tid < 2 * kExCluster * 4) (&slot_s[0][0][0])[tid] = 0ull;
-  const int b0 = d.ex_row[c0], nb = d.ex_row[c0 + nr] - b0;
-  int* li_s = reinterpret_cast<int*>(Sr + (size_t)nb * EL);      // ... and their columns in the set
   if constexpr (kRes) {
     const AT* src = Sx + (size_t)b0 * EL;
     const int n = nb * EL;
+#pragma unroll 1
     for (int i = tid; i < nb; i += kExThreads) li_s[i] = __ldg(d.ex_lidx + b0 + i);
-#pragma unroll 8
+#pragma unroll 4
     for (int i = tid; i < n; i += kExThreads) Sr[i] = __ldg(src + i);
   }
-  ExState st;
-  st.rz = sc->rz;
-  st.sigma = 1.0;
-  st.rnorm = sc->rnorm;
-  st.rmin = sc->rmin;
-  st.tol_abs = sc->tol_abs;
-  st.ratio = sc->ratio;
-  st.max_it = sc->max_it;
-  st.normalize = sc->normalize;
-  st.restart_every = sc->restart_every;
-  st.total = sc->pcg_total;
-  st.pcg_it = st.products = 0;
-  if (tid == 0) {
-    co[2] = co[4] = (AT)1;
-    co[3] = (AT)0;
-    fl[0] = fl[1] = fl[2] = fl[3] = 0;
+  // the z values this thread receives: entries zi of the column set, their place in z
+  const int nz = nloc * DB, z0 = tid - 64;
+  AT zr[ZK];
+  int zo[ZK];
+#pragma unroll
+  for (int k = 0; k < ZK; ++k) {
+    const int i = z0 + k * ZT;
+    zo[k] = z0 >= 0 && i < nz ? lcol[i / DB] * DB + i % DB : -1;
+    zr[k] = zo[k] >= 0 ? gz[zo[k]] : (AT)0;
   }
+  // scalars of the solve: warp 0 keeps those of r^T M r, warp 1 those of |r|
+  const double tol_abs = sc->tol_abs, ratio = sc->ratio;
+  const int max_it = sc->max_it, normalize = sc->normalize, restart_every = sc->restart_every;
+  double s_rz = sc->rz, s_sigma = 1.0, s_rnorm = sc->rnorm, s_rmin = sc->rmin;
+  int pcg_it = 0, products = 0;
+  if (tid == 0) {
+    co[2] = (AT)1;
+    co[3] = (AT)0;
+    fl[0] = fl[1] = fl[2] = fl[3] = fl[4] = 0;
+    is_s = 1.0;
+  }
+  __shared__ double sigma_s;
+  if (tid == 0) sigma_s = 1.0;
   int fail = 0, breakdown = 0, use_best = 0, have_best = 0, saved = 0;
   unsigned epoch = 0;   // of the group reductions
   if constexpr (kCluster) cluster_sync();   // every CTA has started before its shared memory is written
   else __syncthreads();
 
-  // The group's sums of the rows' partial pairs, in warp 0 (called by every thread after a
-  // barrier).  The other warps wait at the caller's next barrier.  On a wait that gave up
-  // fl[3] is set.
-  auto group_sum = [&](double& a, double& b) {
-    ++epoch;
-    if (warp != 0) return;
-    a = b = 0.0;
-    for (int i = lane; i < nr; i += 32) {
-      a += dot[2 * i];
-      b += dot[2 * i + 1];
-    }
-    for (int o = tree_half(nr); o > 0; o >>= 1) {
-      a += __shfl_xor_sync(full, a, o);
-      b += __shfl_xor_sync(full, b, o);
-    }
-    a = __shfl_sync(full, a, 0);
-    b = __shfl_sync(full, b, 0);
-    constexpr int PS = kCluster ? 1 : (kExGrid + 32) / 32;   // slots per lane (a grid: one more than its CTAs)
-    const int par = epoch & 1, n = kCluster ? kExCluster : G + ls.debug_wait;
-    unsigned long long* slots = d.ex_red + (size_t)par * 4 * kExMaxCtas;
-    if constexpr (kCluster) {
-      if (lane < kExCluster) {
-        const unsigned at = cluster_addr(&slot_s[par][rank][0], lane);
-        ex_post_cluster(at, a, epoch);
-        ex_post_cluster(at + 16, b, epoch);
-      }
-    }
-    double u[PS], v[PS];
-    ExWait wait;
-    bool ok = true;
-    if constexpr (!kCluster) {
-      // one lane polls a count of the posts first: every CTA polling every slot while the
-      // last CTAs arrive keeps the few L2 lines of the slots so busy that the posts wait
-      unsigned* count = reinterpret_cast<unsigned*>(d.ex_red + 8 * kExMaxCtas);
-      if (lane == 0) {
-        ex_post(slots + 4 * rank, a, epoch);
-        ex_post(slots + 4 * rank + 2, b, epoch);
-        asm volatile("red.relaxed.gpu.add.u32 [%0], %1;" ::"l"(count), "r"(1u) : "memory");
-        unsigned c;
-        do asm volatile("ld.relaxed.gpu.u32 %0, [%1];" : "=r"(c) : "l"(count) : "memory");
-        while (c < (unsigned)n * epoch && (ok = wait.again()));
-      }
-      ok = __shfl_sync(full, (int)ok, 0);
-    }
-    do {
-      bool all = true;
-#pragma unroll
-      for (int k = 0; k < PS; ++k) {
-        u[k] = v[k] = 0.0;
-        const int i = lane + 32 * k;
-        if (i < n) {
-          if constexpr (kCluster) all = ex_poll_shared(&slot_s[par][i][0], u[k], epoch) & ex_poll_shared(&slot_s[par][i][2], v[k], epoch);
-          else all = (ex_poll(slots + 4 * i, u[k], epoch) & ex_poll(slots + 4 * i + 2, v[k], epoch)) && all;
-        }
-      }
-      if (all) break;
-      ok = ok && wait.again();
-    } while (ok);
-    a = u[0];
-    b = v[0];
-#pragma unroll
-    for (int k = 1; k < PS; ++k) {
-      a += u[k];
-      b += v[k];
-    }
-    ok = __all_sync(full, ok);
-    if (!ok && lane == 0) fl[3] = 1;
-    for (int o = tree_half(kCluster ? kExCluster : n); o > 0; o >>= 1) {
-      a += __shfl_xor_sync(full, a, o);
-      b += __shfl_xor_sync(full, b, o);
-    }
-    a = __shfl_sync(full, a, 0);
-    b = __shfl_sync(full, b, 0);
+  auto group_sum = [&](const AT* v, int w) -> double {
+    return ex_group_sum<AT, kCluster>(v, nr * DB, w, epoch, rank, G + (kCluster ? 0 : ls.debug_wait),
+                                      &slot_s[0][0][0], d.ex_red, &fl[3]);
   };
   auto gave_up = [&] {   // leaves the kernel (a cluster's CTAs together: their shared memory is shared)
     if (tid == 0) atomicExch(ls.err, 1);
     if constexpr (kCluster) cluster_sync();
   };
+  auto receive_z = [&](int o, AT& z) {
+    ExWait wait;
+    bool ok = true;
+    while (!ex_poll(zw + (size_t)o * ZW, z, epoch) && (ok = wait.again())) {}
+    if (!ok) fl[3] = 1;
+  };
 
   for (;;) {
     const int restart = fl[1];
-    if (!restart) {   // the direction of every camera of the column set, from the z of the last reduction's epoch
-      const AT beta = co[3], inv_n = co[4];
-      for (int i = tid; i < nloc * DB; i += kExThreads) {
-        const size_t o = (size_t)__ldg(lcol + i / DB) * DB + i % DB;
-        AT z;
-        if (epoch == 0) {
-          z = gz[o];
-        } else {
-          ExWait wait;
-          bool ok;
-          do ok = ex_poll(zw + o * ZW, z, epoch);
-          while (!ok && wait.again());
-          if (!ok) fl[3] = 1;
+    if (!restart && z0 >= 0) {   // the direction of every camera of the column set
+      const AT beta = co[3], inv_n = co[2];
+#pragma unroll
+      for (int k = 0; k < ZK; ++k) {
+        const int i = z0 + k * ZT;
+        if (i < nz) {
+          AT* p = pl + i / DB * V::W + V::at(i % DB);
+          *p = (zr[k] + beta * *p) * inv_n;
         }
-        pl[i] = (z + beta * pl[i]) * inv_n;
+      }
+#pragma unroll 1
+      for (int i = z0 + ZK * ZT; i < nz; i += ZT) {
+        const int o = __ldg(lcol + i / DB) * DB + i % DB;
+        AT* p = pl + i / DB * V::W + V::at(i % DB);
+        AT z = (AT)0;
+        if (epoch == 0) z = gz[o];
+        else receive_z(o, z);
+        *p = (z + beta * *p) * inv_n;
       }
     }
     const AT* vec = restart ? xl : pl;   // a restart's product is of the current solution
     __syncthreads();
+#pragma unroll 1
     for (int r = warp / wpr; r < nr; r += rpp) {
-      const int sub = warp % wpr, c = c0 + r;
+      const int sub = warp % wpr, c = c0 + r, cg = lane < LN ? lane / DC : 0;
       AT acc = (AT)0;
       const int b1 = __ldg(d.ex_row + c + 1);
       int b = __ldg(d.ex_row + c) + sub;
       if constexpr (kRes) {
 #pragma unroll 4
         for (; b < b1; b += wpr) {
-          const AT* v = vec + li_s[b - b0] * DB + lane / DC;
-          const AT* Sb = Sr + (size_t)(b - b0) * EL + lane;
-          if (lane < LN) {
+          AT v[ST];
+          V::group(vec + li_s[b - b0] * V::W, cg, v);
+          const AT* Sb = Sr + (size_t)(b - b0) * EL + (lane < LN ? lane : 0);
 #pragma unroll
-            for (int s = 0; s < ST; ++s) acc = fma(Sb[s * LN], v[s * CG], acc);
-          }
+          for (int s = 0; s < ST; ++s) acc = fma(Sb[s * LN], v[s], acc);
         }
       } else {
         // blocks from the L2 cache: UB blocks of a warp are in flight
         constexpr int UB = 8;
+#pragma unroll 1
         for (; b < b1; b += UB * wpr) {
           AT w[UB][ST];
           int li[UB];
@@ -760,67 +816,74 @@ __global__ void __launch_bounds__(kExThreads, 1) k_ex_pcg(LaunchSet ls, int prob
           }
 #pragma unroll
           for (int k = 0; k < UB; ++k) {
-            const AT* v = vec + li[k] * DB + (lane < LN ? lane / DC : 0);
+            AT v[ST];
+            V::group(vec + li[k] * V::W, cg, v);
 #pragma unroll
-            for (int s = 0; s < ST; ++s) acc = fma(w[k][s], v[s * CG], acc);
+            for (int s = 0; s < ST; ++s) acc = fma(w[k][s], v[s], acc);
           }
         }
       }
       const AT a1 = __shfl_down_sync(full, acc, DC), a2 = __shfl_down_sync(full, acc, 2 * DC);
       AT y = lane < DC ? (acc + a1) + a2 : (AT)0;
       if constexpr (Mo::kExtra) {
-        // products with the camera-side edges' off-diagonal blocks, dealt over the row's warps
+        // products with the camera-side edges' off-diagonal blocks, dealt over the row's
+        // warps; two lanes per row of the block, half of its columns each
+        constexpr int H0 = (DB + 1) / 2;
+        const int half = lane / DB, a = lane % DB;
+        AT t = (AT)0;
+#pragma unroll 1
         for (int u = __ldg(d.xk_off + c) + sub; u < __ldg(d.xk_off + c + 1); u += wpr) {
           const int o = __ldg(d.ex_xl + u);
           if (o < 0) continue;   // unary edge: diagonal only
           const int code = __ldg(d.xk_list + u), side = code & 1;
           const AT* H = xH + (size_t)(code >> 1) * DB * DB;
-          if (lane < DB) {
+          const int step = side ? DB : 1, base = side ? a : a * DB;
+          if (half < 2) {
 #pragma unroll
-            for (int j = 0; j < DB; ++j) y += (side ? __ldg(H + j * DB + lane) : __ldg(H + lane * DB + j)) * vec[o * DB + j];
+            for (int j = 0; j < H0; ++j) {
+              const int k = half * H0 + j;
+              if (k < DB) t += __ldg(H + base + k * step) * vec[o * V::W + V::at(k)];
+            }
           }
         }
+        t += __shfl_down_sync(full, t, DB);
+        y += t;
       }
       if (lane < PW) part[((size_t)r * wpr + sub) * PW + lane] = y;
     }
     __syncthreads();
+#pragma unroll 1
     for (int r = warp; r < nr; r += NW) {
       const int c = c0 + r;
-      const AT* v = vec + __ldg(d.ex_lown + c) * DB;
-      AT dt = (AT)0;
+      const AT* v = vec + __ldg(d.ex_lown + c) * V::W;
       if (lane < DB) {
         AT yi = (AT)0;
 #pragma unroll
-        for (int j = 0; j < DB; ++j) yi += __ldg(Sd + (size_t)c * TB + sym_idx(DB, lane, j)) * v[j];
+        for (int j = 0; j < DB; ++j) yi += Ss[(r * DB + lane) * DB + j] * v[V::at(j)];
         if (lane < PW)
+#pragma unroll 1
           for (int s = 0; s < wpr; ++s) yi += part[((size_t)r * wpr + s) * PW + lane];
         ys[r * DB + lane] = yi;
-        dt = v[lane] * yi;
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) dt += __shfl_down_sync(full, dt, o);
-      if (lane == 0) {
-        dot[2 * r] = (double)dt;
-        dot[2 * r + 1] = 0.0;
+        da[r * DB + lane] = v[V::at(lane)] * yi;
       }
     }
     __syncthreads();
-    double s0, s1;
-    group_sum(s0, s1);
+    ++epoch;
     if (warp == 0) {
+      const double pAp = group_sum(da, 0);
       int bad = 0;
       double al = 0.0;
       if (!restart) {
-        bad = !(s0 > 0.0) || !isfinite(s0);
-        al = bad ? 0.0 : st.rz / s0;
+        bad = !(pAp > 0.0) || !isfinite(pAp);
+        al = bad ? 0.0 : s_rz / pAp;
         if (bad) {   // p^T S p not positive: S is not positive definite at this damping
-          if (st.pcg_it == 0) fail = 1;
+          if (pcg_it == 0) fail = 1;
           else breakdown = 1;
         }
       }
       if (lane == 0) {
         co[0] = (AT)al;
-        co[1] = (AT)(st.sigma * al);
+        co[1] = (AT)(sigma_s * al);
         fl[0] = bad;
       }
     }
@@ -828,109 +891,119 @@ __global__ void __launch_bounds__(kExThreads, 1) k_ex_pcg(LaunchSet ls, int prob
     if (fl[3]) return gave_up();
     if (fl[0]) break;
     const AT alpha = co[0], sa = co[1], sn = co[2];
-    if (st.restart_every > 0 && !restart)
-      for (int i = tid; i < nloc * DB; i += kExThreads) xl[i] += sa * pl[i];
+    if (restart_every > 0 && !restart)
+#pragma unroll 1
+      for (int i = tid; i < nloc * V::W; i += kExThreads) xl[i] += sa * pl[i];
+#pragma unroll 1
     for (int r = warp; r < nr; r += NW) {
       const int c = c0 + r, k = r * DB + lane;
-      AT ri = (AT)0, zi = (AT)0, a = (AT)0, b = (AT)0;
+      AT ri = (AT)0;
       if (lane < DB) {
         if (restart) {
           ri = gs[k] - ys[k];
         } else {
-          xs[k] += sa * pl[__ldg(d.ex_lown + c) * DB + lane];
+          xs[k] += sa * pl[__ldg(d.ex_lown + c) * V::W + V::at(lane)];
           ri = rs[k] * sn - alpha * ys[k];
         }
         rs[k] = ri;
       }
       __syncwarp();
       if (lane < DB) {
+        AT zi = (AT)0;
 #pragma unroll
-        for (int j = 0; j < DB; ++j) zi += __ldg(Mi + (size_t)c * TB + sym_idx(DB, lane, j)) * rs[r * DB + j];
+        for (int j = 0; j < DB; ++j) zi += Ms[(r * DB + lane) * DB + j] * rs[r * DB + j];
         ex_post(zw + ((size_t)c * DB + lane) * ZW, zi, epoch + 1);
-        a = ri * zi;
-        b = ri * ri;
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        a += __shfl_down_sync(full, a, o);
-        b += __shfl_down_sync(full, b, o);
-      }
-      if (lane == 0) {
-        dot[2 * r] = (double)a;
-        dot[2 * r + 1] = (double)b;
+        da[k] = ri * zi;
+        db[k] = ri * ri;
       }
     }
     __syncthreads();
-    group_sum(s0, s1);
-    if (warp == 0) {   // stopping rules, beta and the normalisation (as pcg_update_finish)
-      const double rz = s0, rr = s1;
-      // one division and one inverse square root, independent of each other: FP64 operations
-      // in sequence are the longest part of the iteration's end
-      const double quo = rz / st.rz, is = rr > 0.0 ? rsqrt(rr) : 0.0, n = rr > 0.0 ? rr * is : rr;
-      const double be = restart ? 0.0 : quo;
-      if (restart) st.sigma = 1.0;
-      const double rtrue = st.sigma * n;
-      if (!restart) st.pcg_it += 1;
+    ++epoch;
+    pcg_it += restart ? 0 : 1;
+    products += 1;
+    // stopping rules, beta and the normalisation (as pcg_update_finish): warp 0 from
+    // r^T M r, warp 1 from |r|^2, while the others receive z
+    if (warp == 0) {
+      const double rz = group_sum(da, 0);
+      const double be = restart ? 0.0 : rz / s_rz;
+      s_rz = rz;
+      if (lane == 0) {
+        co[3] = (AT)be;
+        fl[4] = !(rz > 0.0);
+      }
+    } else if (warp == 1) {
+      const double rr = group_sum(db, 1);
+      const double is = rr > 0.0 ? rsqrt(rr) : 0.0, n = rr > 0.0 ? rr * is : rr;
+      if (restart) s_sigma = 1.0;
+      const double rtrue = s_sigma * n;
       int done = 0, save = 0;
-      if (st.ratio > 0.0) {
-        if (rtrue < st.rmin) {
-          st.rmin = rtrue;
+      if (ratio > 0.0) {
+        if (rtrue < s_rmin) {
+          s_rmin = rtrue;
           save = 1;
           have_best = 1;
-        } else if (rtrue > st.ratio * st.rmin) {
+        } else if (rtrue > ratio * s_rmin) {
           done = 1;
           use_best = 1;
         }
       }
-      if (rtrue <= st.tol_abs || st.pcg_it >= st.max_it || !isfinite(rtrue) || !(rz > 0.0)) {
-        done = 1;
-        if (!isfinite(rtrue)) use_best = 1;
-        if (!(rz > 0.0) && !(rtrue <= st.tol_abs)) breakdown = 1;
-      }
+      const bool tol = rtrue <= tol_abs, fin = isfinite(rtrue);
+      if (tol || pcg_it >= max_it || !fin) done = 1;
+      if (!fin) use_best = 1;
+      s_rnorm = rtrue;
       double in = 1.0;
-      st.rz = rz;
-      if (st.normalize && n > 0.0) {
+      if (normalize && n > 0.0) {
         in = is;
-        st.sigma *= n;
-        st.rz = rz * is * is;
+        s_sigma *= n;
       }
-      st.rnorm = rtrue;
-      st.products += 1;
-      st.total += 1;
       if (lane == 0) {
-        co[2] = co[4] = (AT)in;
-        co[3] = (AT)be;
-        fl[0] = done;
-        fl[1] = (!done && !restart && st.restart_every > 0 && st.pcg_it % st.restart_every == 0) ? 1 : 0;
+        co[2] = (AT)in;
+        is_s = in;
+        sigma_s = s_sigma;
+        fl[0] = done | (tol ? 2 : 0);
+        fl[1] = (!restart && restart_every > 0 && pcg_it % restart_every == 0) ? 1 : 0;
         fl[2] = save;
       }
+    } else {
+#pragma unroll
+      for (int k = 0; k < ZK; ++k)
+        if (zo[k] >= 0) receive_z(zo[k], zr[k]);
     }
     __syncthreads();
     if (fl[3]) return gave_up();
+    if (warp == 0) s_rz = s_rz * is_s * is_s;
+    // r^T M r not positive before the tolerance is met: the preconditioned system is not
+    // positive definite at this damping (after at least one step)
+    if (fl[4] && !(fl[0] & 2)) breakdown = 1;
     if (fl[2]) {
       saved = 1;
+#pragma unroll 1
       for (int i = tid; i < nr * DB; i += kExThreads) bs[i] = xs[i];
     }
-    if (fl[0]) break;
+    if (fl[0] || fl[4]) break;
   }
   if constexpr (kCluster) cluster_sync();   // no CTA's shared memory is written any more
+#pragma unroll 1
   for (int i = tid; i < nr * DB; i += kExThreads) {
     gx[(size_t)c0 * DB + i] = xs[i];
     if (saved) reinterpret_cast<AT*>(d.xbest)[(size_t)c0 * DB + i] = bs[i];
   }
-  if (tid == 0 && rank == 0) {
-    sc->rz = st.rz;
-    sc->sigma = st.sigma;
-    sc->rnorm = st.rnorm;
-    sc->rmin = st.rmin;
-    sc->pcg_it = st.pcg_it;
-    sc->pcg_products = st.products;
-    sc->pcg_total = st.total;
+  if (rank != 0) return;
+  if (tid == 0) {
+    sc->rz = s_rz;
+    sc->pcg_it = pcg_it;
+    sc->pcg_products = products;
+    sc->pcg_total += products;
     if (fail) sc->pcg_fail = 1;
     if (breakdown) sc->pcg_breakdown = 1;
+    sc->pcg_done = 1;
+  }
+  if (tid == 32) {
+    sc->sigma = s_sigma;
+    sc->rnorm = s_rnorm;
+    sc->rmin = s_rmin;
     if (use_best) sc->use_best = 1;
     if (have_best) sc->have_best = 1;
-    sc->pcg_done = 1;
   }
 }
 

@@ -589,7 +589,7 @@ __global__ void __launch_bounds__(kCamPerBlock * 32) k_cam_finalize(LaunchSet ls
   const bool ex = ls.ex && d.ex;
   if (ex) {   // no epoch of the coming PCG solve is posted yet
     if (cbl == 0)
-      for (int i = threadIdx.x; i < 8 * kExMaxCtas + 1; i += blockDim.x) d.ex_red[i] = 0ull;
+      for (int i = threadIdx.x; i < 8 * kExMaxCtas + 2; i += blockDim.x) d.ex_red[i] = 0ull;
     constexpr int ZC = DB * (int)(sizeof(AT) / 4);   // words of a camera's z
     for (int i = threadIdx.x; i < kCamPerBlock * ZC; i += blockDim.x)
       if (cbl * kCamPerBlock + i / ZC < d.C) d.ex_z[(size_t)cbl * kCamPerBlock * ZC + i] = 0ull;

@@ -45,7 +45,8 @@ def test_step_matches_the_matrix_free_product(gpo, scene, prec):
     p = SCENES[scene]()
     steps = []
     # in FP64, forming 2,415 pairs per point costs more than the products of a solve: not planned
-    auto = 2 if (scene, prec) == ("long_tracks", "fp64") else 7
+    # and BF16 bundle adjustment keeps the matrix-free product (pipelined)
+    auto = 3 if prec == "bf16" else 2 if (scene, prec) == ("long_tracks", "fp64") else 7
     for variant in (2, 0):
         g, _, _ = _ba(gpo, p, prec, variant)
         dx, its = g.debug_step(1e-2, 9 * p.n_cams + 3 * p.n_pts, gpo.default_params(pcg_max_iters=3, pcg_tol=0.0))
@@ -56,7 +57,7 @@ def test_step_matches_the_matrix_free_product(gpo, scene, prec):
     assert np.max(np.abs(steps[1] - steps[0])) <= tol * np.max(np.abs(steps[0]))
 
 
-@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+@pytest.mark.parametrize("prec", ["fp64", "fp32", "bf16"])
 @pytest.mark.parametrize("kfs", [3, 20, 150])
 def test_vi_step_matches_the_matrix_free_product(gpo, kfs, prec):
     p = synth.vi_problem(5, kfs, 60 * kfs)
@@ -154,6 +155,7 @@ def test_memory_budget_without_room_for_the_blocks_stays_matrix_free(gpo):
         sizes[variant] = g.plan()
         g.close()
     assert sizes[0] > sizes[2]
-    g, _, _ = _ba(gpo, p, "fp32", 0, memory_budget=(sizes[0] + sizes[2]) // 2)
+    budget = (sizes[0] + sizes[2]) // 2
+    g, _, _ = _ba(gpo, p, "fp32", 0, memory_budget=budget)
     g.optimize(1)
-    assert g.info()["spmv_kernel"] != 7 and g.footprint() == sizes[2]
+    assert g.info()["spmv_kernel"] != 7 and g.footprint() <= budget
