@@ -133,9 +133,9 @@ cudaError_t up(T* dst, const std::vector<T>& src, cudaStream_t st) {
 // that a warp's accesses to the caller's buffer -- often page-locked host memory read
 // or written in place over the host link -- form one contiguous 256-byte span.  (Two
 // values per thread as 16-byte accesses measured no faster.)
-// dst rows (through idx) = src rows; *changed = 1 if any value's bits differ (one store
-// per CTA at most)
-__global__ void k_assign_rows(double* dst, const double* src, const int32_t* idx, int n, int w, int* changed) {
+// dst rows (through idx) = src rows; if any value's bits differ, *dev = *host = call
+__global__ void k_assign_rows(double* dst, const double* src, const int32_t* idx, int n, int w, int* dev, int* host,
+                              int call) {
   const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   int diff = 0;
   if (e < (size_t)n * w) {
@@ -146,7 +146,8 @@ __global__ void k_assign_rows(double* dst, const double* src, const int32_t* idx
     diff = __double_as_longlong(*p) != __double_as_longlong(v);
     *p = v;
   }
-  if (__syncthreads_or(diff) && threadIdx.x == 0) *changed = 1;
+  if (__syncthreads_or(diff) && threadIdx.x == 0 && atomicExch(dev, call) != call)
+    *reinterpret_cast<volatile int*>(host) = call;
 }
 // dst rows = src rows through idx (the caller's row i is the graph's row idx[i])
 __global__ void k_gather_rows(double* dst, const double* src, const int32_t* idx, int n, int w) {
@@ -957,10 +958,11 @@ void gpo_host::fill_scalars(gpo_graph* g, const gpo_lm_params& p, double lambda,
 
 gpo_status gpo_host::upload_scalars(gpo_graph* g, const Scalars& s) {
   if (gpo_status st = ensure_runtime(g); st != GPO_OK) return st;
-  *g->h_sc = s;
-  GPO_CUDA(g, cudaMemcpyAsync(g->dev.sc, g->h_sc, sizeof(Scalars), cudaMemcpyHostToDevice, g->stream));
-  // the pinned staging buffer is reused: make sure the copy has been consumed
-  GPO_CUDA(g, cudaStreamSynchronize(g->stream));
+  // the pinned staging buffer is reused: make sure an earlier copy has been consumed
+  if (g->up_busy) GPO_CUDA(g, cudaStreamSynchronize(g->stream));
+  *g->h_up = s;
+  g->up_busy = true;
+  GPO_CUDA(g, cudaMemcpyAsync(g->dev.sc, g->h_up, sizeof(Scalars), cudaMemcpyHostToDevice, g->stream));
   return GPO_OK;
 }
 
@@ -1158,6 +1160,7 @@ gpo_status gpo_host::begin_solves(gpo_graph* g, const gpo::LaunchSet& ls) {
 gpo_status gpo_host::end_solves(gpo_graph* g, const gpo::LaunchSet& ls) {
   if (ls.n_xg) GPO_CUDA(g, cudaMemcpyAsync(g->h_flag, ls.running, 2 * sizeof(int), cudaMemcpyDeviceToHost, g->stream));
   GPO_CUDA(g, cudaStreamSynchronize(g->stream));
+  g->up_busy = false;
   if (ls.n_xg && g->h_flag[1]) return fail(g, GPO_ERR_TIMEOUT, "a bounded device wait in the PCG solve gave up");
   return GPO_OK;
 }
@@ -1184,6 +1187,7 @@ static gpo_status compute_cost(gpo_graph* g, double* out) {
   if (s != GPO_OK) return s;
   GPO_CUDA(g, cudaMemcpyAsync(g->h_sc, g->dev.sc, sizeof(Scalars), cudaMemcpyDeviceToHost, g->stream));
   GPO_CUDA(g, cudaStreamSynchronize(g->stream));
+  g->up_busy = false;
   *out = g->h_sc->cost;
   return GPO_OK;
 }
@@ -1234,6 +1238,9 @@ gpo_status gpo_host::ensure_runtime(gpo_graph* g) {
   GPO_CUDA(g, cudaMallocHost(&g->h_flag, 4 * sizeof(int)));
   GPO_CUDA(g, cudaMallocHost(&g->h_changed, sizeof(int)));
   GPO_CUDA(g, cudaMalloc(&g->d_changed, sizeof(int)));
+  GPO_CUDA(g, cudaMemsetAsync(g->d_changed, 0, sizeof(int), g->stream));
+  *g->h_changed = 0;
+  GPO_CUDA(g, cudaMallocHost(&g->h_up, sizeof(Scalars)));
   GPO_CUDA(g, cudaEventCreateWithFlags(&g->ev[0], cudaEventDisableTiming));
   GPO_CUDA(g, cudaEventCreateWithFlags(&g->ev[1], cudaEventDisableTiming));
   GPO_CUDA(g, cudaMallocHost(&g->h_sc, sizeof(Scalars)));   // last: marks the runtime as ready
@@ -1315,6 +1322,7 @@ gpo_status gpo_graph_destroy(gpo_graph* g) {
   if (g->stream) cudaStreamSynchronize(g->stream);
   release_device(g);
   if (g->h_sc) cudaFreeHost(g->h_sc);
+  if (g->h_up) cudaFreeHost(g->h_up);
   if (g->h_flag) cudaFreeHost(g->h_flag);
   if (g->h_changed) cudaFreeHost(g->h_changed);
   if (g->d_changed) cudaFree(g->d_changed);
@@ -1340,6 +1348,7 @@ gpo_status gpo_add_vertices(gpo_graph* g, int32_t kind, int32_t block_size, int6
   const int64_t id0 = (int64_t)g->v_kind.size();
   const int64_t loc0 = is_camera(kind) ? (int64_t)g->cam_fixed.size() : (int64_t)g->pt_fixed.size();
   if (loc0 + n > INT32_MAX / 16) return fail(g, GPO_ERR_UNSUPPORTED, "too many vertices of kind %d", kind);
+  if (n > 0 && (g->v_runs.empty() || g->v_runs.back().kind != kind)) g->v_runs.push_back({id0, (int8_t)kind});
   g->v_kind.insert(g->v_kind.end(), n, (int8_t)kind);
   for (int64_t i = 0; i < n; ++i) g->v_local.push_back(loc0 + i);
   if (is_camera(kind)) {
@@ -1578,8 +1587,10 @@ static gpo_status check_range(gpo_graph* g, int64_t first, int64_t n, int* kind_
     return fail(g, GPO_ERR_ARG, "vertex range [%lld, %lld) out of bounds", (long long)first, (long long)(first + n));
   if (n == 0) { *kind_out = -1; return GPO_OK; }
   const int k = g->v_kind[first];
-  for (int64_t i = 1; i < n; ++i)
-    if (g->v_kind[first + i] != k) return fail(g, GPO_ERR_ARG, "vertex range mixes kinds");
+  // the run after the one that holds `first` begins behind the range
+  auto next = std::upper_bound(g->v_runs.begin(), g->v_runs.end(), first,
+                               [](int64_t id, const gpo_graph::VRun& r) { return id < r.first; });
+  if (next != g->v_runs.end() && next->first < first + n) return fail(g, GPO_ERR_ARG, "vertex range mixes kinds");
   // the range must also be contiguous in the kind's local numbering
   if (g->v_local[first + n - 1] - g->v_local[first] != n - 1)
     return fail(g, GPO_ERR_ARG, "vertex range is not contiguous within its kind");
@@ -1624,7 +1635,6 @@ gpo_status gpo_set_initial(gpo_graph* g, int64_t first, int64_t n, const double*
   // memory directly (pageable memory through a device copy) and flags any value whose
   // bits change; points live on the device in sorted order (the id -> row map is
   // resident)
-  GPO_CUDA(g, cudaMemsetAsync(g->d_changed, 0, sizeof(int), st));
   const double* src = on_device ? state : mapped_host(state);
   double* tmp = nullptr;
   if (!src) {
@@ -1634,12 +1644,13 @@ gpo_status gpo_set_initial(gpo_graph* g, int64_t first, int64_t n, const double*
   }
   double* dst = is_camera(kind) ? g->dev.cam + loc * w : g->dev.pt;
   const int32_t* idx = is_camera(kind) ? nullptr : g->pt_old2new_d + loc;
-  k_assign_rows<<<(int)((n * w + 255) / 256), 256, 0, st>>>(dst, src, idx, (int)n, w, g->d_changed);
+  const int call = ++g->set_calls;
+  k_assign_rows<<<(int)((n * w + 255) / 256), 256, 0, st>>>(dst, src, idx, (int)n, w, g->d_changed, g->h_changed, call);
   GPO_CUDA(g, cudaGetLastError());
   if (tmp) GPO_CUDA(g, cudaFreeAsync(tmp, st));
-  GPO_CUDA(g, cudaMemcpyAsync(g->h_changed, g->d_changed, sizeof(int), cudaMemcpyDeviceToHost, st));
   GPO_CUDA(g, cudaStreamSynchronize(st));
-  if (*g->h_changed) {
+  g->up_busy = false;
+  if (*reinterpret_cast<volatile int*>(g->h_changed) == call) {
     g->cost_valid = false;
     g->state_same = false;
   }
@@ -1701,10 +1712,9 @@ gpo_status gpo_optimize(gpo_graph* g, int32_t max_iters, const gpo_lm_params* pa
     sc.cost = g->last_cost;
   }
   if ((s = upload_scalars(g, sc)) != GPO_OK) return s;
-  double F0;
-  if (cont) F0 = g->last_cost;
-  else if ((s = compute_cost(g, &F0)) != GPO_OK) return s;
-  if (!std::isfinite(F0)) return fail(g, GPO_ERR_NUMERIC, "initial cost is not finite (%g)", F0);
+  // the iterations follow without a look at the cost: one that is not finite switches them
+  // off on the device
+  if (!cont && (s = launch_initial_cost(g, g->ls)) != GPO_OK) return s;
   if ((s = begin_solves(g, g->ls)) != GPO_OK) return s;
   for (int it = 0; it < max_iters; ++it) {
     g->cur_lm_iter = it;
@@ -1714,11 +1724,14 @@ gpo_status gpo_optimize(gpo_graph* g, int32_t max_iters, const gpo_lm_params* pa
   g->cur_lm_iter = -1;
   GPO_CUDA(g, cudaMemcpyAsync(g->h_sc, g->dev.sc, sizeof(Scalars), cudaMemcpyDeviceToHost, g->stream));
   const int nh = std::min(max_iters, gpo::kMaxHistory);
-  g->hist.resize(nh);
+  std::vector<gpo::IterRecord> hist(nh);
   if (nh)
-    GPO_CUDA(g, cudaMemcpyAsync(g->hist.data(), g->dev.hist, nh * sizeof(gpo::IterRecord),
+    GPO_CUDA(g, cudaMemcpyAsync(hist.data(), g->dev.hist, nh * sizeof(gpo::IterRecord),
                                 cudaMemcpyDeviceToHost, g->stream));
   if ((s = end_solves(g, g->ls)) != GPO_OK) return s;
+  const double F0 = cont ? g->last_cost : g->h_sc->cost0;
+  if (!std::isfinite(F0)) return fail(g, GPO_ERR_NUMERIC, "initial cost is not finite (%g)", F0);
+  g->hist = std::move(hist);
   if (g->prof.on) prof_resolve(g);
   g->last_cost = g->h_sc->cost;
   g->cost_valid = true;

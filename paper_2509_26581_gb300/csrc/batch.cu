@@ -88,39 +88,28 @@ gpo_status build_set(gpo_graph* owner, const std::vector<gpo_graph*>& gs, BatchS
   cudaStream_t st = owner->stream;
   char* mem = nullptr;
   GPO_CUDA(owner, cudaMallocAsync(reinterpret_cast<void**>(&mem), total, st));
-  char* p = mem;
-  auto take = [&](size_t b) { char* r = p; p += b; return r; };
-  DevBA* probs_d = reinterpret_cast<DevBA*>(take(b_probs));
-  Scalars* stage_d = reinterpret_cast<Scalars*>(take(b_stage));
-  int* ch_d = reinterpret_cast<int*>(take(b_ch));
-  int* cb_d = reinterpret_cast<int*>(take(b_cb));
-  int* pb_d = reinterpret_cast<int*>(take(b_pb));
-  int* chb_d = reinterpret_cast<int*>(take(b_base));
-  int* cbb_d = reinterpret_cast<int*>(take(b_base));
-  int* pbb_d = reinterpret_cast<int*>(take(b_base));
-  int* running_d = reinterpret_cast<int*>(take(256));
-  int* xf_d = reinterpret_cast<int*>(take(b_xf));
-  int* xd_d = reinterpret_cast<int*>(take(b_xd));
-  int* xfb_d = reinterpret_cast<int*>(take(b_base));
-  int* xdb_d = reinterpret_cast<int*>(take(b_base));
-  int* cl_d = reinterpret_cast<int*>(take(b_base));
-  if (!xf_prob.empty()) GPO_CUDA(owner, cudaMemcpyAsync(xf_d, xf_prob.data(), xf_prob.size() * 4, cudaMemcpyHostToDevice, st));
-  if (!xd_prob.empty()) GPO_CUDA(owner, cudaMemcpyAsync(xd_d, xd_prob.data(), xd_prob.size() * 4, cudaMemcpyHostToDevice, st));
-  if (!cl_prob.empty()) GPO_CUDA(owner, cudaMemcpyAsync(cl_d, cl_prob.data(), cl_prob.size() * 4, cudaMemcpyHostToDevice, st));
-  if (ex) {
-    GPO_CUDA(owner, cudaMemcpyAsync(xfb_d, xf_base.data(), n * 4, cudaMemcpyHostToDevice, st));
-    GPO_CUDA(owner, cudaMemcpyAsync(xdb_d, xd_base.data(), n * 4, cudaMemcpyHostToDevice, st));
-  }
-  GPO_CUDA(owner, cudaMemcpyAsync(probs_d, probs.data(), n * sizeof(DevBA), cudaMemcpyHostToDevice, st));
-  if (!ch_prob.empty()) GPO_CUDA(owner, cudaMemcpyAsync(ch_d, ch_prob.data(), ch_prob.size() * 4, cudaMemcpyHostToDevice, st));
-  if (!cb_prob.empty()) GPO_CUDA(owner, cudaMemcpyAsync(cb_d, cb_prob.data(), cb_prob.size() * 4, cudaMemcpyHostToDevice, st));
-  if (!pb_prob.empty()) GPO_CUDA(owner, cudaMemcpyAsync(pb_d, pb_prob.data(), pb_prob.size() * 4, cudaMemcpyHostToDevice, st));
-  GPO_CUDA(owner, cudaMemcpyAsync(chb_d, ch_base.data(), n * 4, cudaMemcpyHostToDevice, st));
-  GPO_CUDA(owner, cudaMemcpyAsync(cbb_d, cb_base.data(), n * 4, cudaMemcpyHostToDevice, st));
-  GPO_CUDA(owner, cudaMemcpyAsync(pbb_d, pb_base.data(), n * 4, cudaMemcpyHostToDevice, st));
-  GPO_CUDA(owner, cudaMemsetAsync(running_d, 0, 32, st));
-  // the host vectors go out of scope: wait for the copies
-  GPO_CUDA(owner, cudaStreamSynchronize(st));
+  // one host image, one copy (staged before the call returns: the memory is pageable)
+  std::vector<char> img(total, 0);
+  size_t at = 0;
+  auto take = [&](size_t b) {
+    const size_t r = at;
+    at += b;
+    return r;
+  };
+  auto put = [&](size_t b, const void* src, size_t n_bytes) {
+    const size_t r = take(b);
+    if (n_bytes) std::memcpy(img.data() + r, src, n_bytes);
+    return mem + r;
+  };
+  auto put_i = [&](size_t b, const std::vector<int>& v) { return reinterpret_cast<int*>(put(b, v.data(), v.size() * 4)); };
+  DevBA* probs_d = reinterpret_cast<DevBA*>(put(b_probs, probs.data(), n * sizeof(DevBA)));
+  Scalars* stage_d = reinterpret_cast<Scalars*>(mem + take(b_stage));
+  int *ch_d = put_i(b_ch, ch_prob), *cb_d = put_i(b_cb, cb_prob), *pb_d = put_i(b_pb, pb_prob);
+  int *chb_d = put_i(b_base, ch_base), *cbb_d = put_i(b_base, cb_base), *pbb_d = put_i(b_base, pb_base);
+  int* running_d = reinterpret_cast<int*>(mem + take(256));
+  int *xf_d = put_i(b_xf, xf_prob), *xd_d = put_i(b_xd, xd_prob);
+  int *xfb_d = put_i(b_base, xf_base), *xdb_d = put_i(b_base, xd_base), *cl_d = put_i(b_base, cl_prob);
+  GPO_CUDA(owner, cudaMemcpyAsync(mem, img.data(), total, cudaMemcpyHostToDevice, st));
   gpo::LaunchSet ls{};
   ls.probs = probs_d;
   ls.ch_prob = ch_d; ls.ch_base = chb_d;
@@ -156,10 +145,9 @@ gpo_status build_set(gpo_graph* owner, const std::vector<gpo_graph*>& gs, BatchS
 
 gpo_status put_scalars(gpo_graph* owner, BatchSet& bs, const std::vector<Scalars>& sc) {
   GPO_CUDA(owner, cudaMemcpyAsync(bs.staging, sc.data(), sc.size() * sizeof(Scalars),
-                                  cudaMemcpyHostToDevice, owner->stream));
+                                  cudaMemcpyHostToDevice, owner->stream));   // pageable: staged before the call returns
   k_put_scalars<<<(bs.n + 127) / 128, 128, 0, owner->stream>>>(bs.ls.probs, bs.staging, bs.n);
   GPO_CUDA(owner, cudaGetLastError());
-  GPO_CUDA(owner, cudaStreamSynchronize(owner->stream));
   return GPO_OK;
 }
 

@@ -59,6 +59,7 @@ __host__ __device__ inline int pad8(int n) { return (n + 7) & ~7; }
 struct Scalars {
   // LM
   double lambda, nu, cost, cand_cost, model_dec, rho;
+  double cost0;          // F at the start of the call
   double lambda_min, lambda_max, diag_min, diag_max;
   int damping_mode, need_lin, accepted, n_accepted, iter, pcg_total;
   // PCG

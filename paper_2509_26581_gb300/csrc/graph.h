@@ -57,6 +57,8 @@ struct gpo_graph {
   int cam_kind = -1;
   std::vector<int8_t> v_kind;
   std::vector<int64_t> v_local;
+  struct VRun { int64_t first; int8_t kind; };
+  std::vector<VRun> v_runs;        // runs of consecutive ids of one kind
   std::vector<double> cam_state;   // [C][SS] (host copy until finalize)
   std::vector<double> pt_state;    // [P][3]
   std::vector<uint8_t> cam_fixed, pt_fixed;
@@ -103,7 +105,9 @@ struct gpo_graph {
   bool ex_cluster = false;         // explicit Schur complement: solved by a cluster (else a grid)
   int4 ex_grid{0, 0, 0, 0};        // the solve's launch (problem, CTAs, shared memory)
   DevBA* dev_desc = nullptr;       // device copy of `dev` (ls.probs)
-  Scalars* h_sc = nullptr;         // pinned
+  Scalars* h_sc = nullptr;         // pinned, read back into
+  Scalars* h_up = nullptr;         // pinned, uploaded from
+  bool up_busy = false;            // an upload from h_up may still be in flight
   int* h_flag = nullptr;           // pinned [2]
   cudaEvent_t ev[2] = {nullptr, nullptr};
   std::vector<gpo::IterRecord> hist;
@@ -115,8 +119,11 @@ struct gpo_graph {
   bool state_same = false;
   int last_need_lin = 1;           // the run's need_lin at its end (0: rows at the state)
   int32_t last_solver = -1;
-  int* d_changed = nullptr;        // device flag: gpo_set_initial changed a value
-  int* h_changed = nullptr;        // pinned
+  // gpo_set_initial's kernel stores the call's number when it changes a value: in device
+  // memory (so that one store per call crosses to the host), and in pinned host memory
+  int* d_changed = nullptr;
+  int* h_changed = nullptr;
+  int set_calls = 0;
   Profiler prof;
   int cur_lm_iter = -1;
   int cur_pcg_k = 0;

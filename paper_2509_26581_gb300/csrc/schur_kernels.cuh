@@ -184,7 +184,10 @@ __global__ void k_cost_init(LaunchSet ls) {
   if constexpr (Mo::kExtra)
     for (int x = threadIdx.x; x < d.NX; x += kThreads) acc += d.xe_cost[x];
   const double s = block_sum(acc, red);
-  if (threadIdx.x == 0) d.sc->cost = s;
+  if (threadIdx.x == 0) {
+    d.sc->cost = d.sc->cost0 = s;
+    if (!isfinite(s)) d.sc->active = 0;   // the call reports it; no iteration runs
+  }
 }
 
 // ---------------------------------------------------------------- per-edge records and slot rows
