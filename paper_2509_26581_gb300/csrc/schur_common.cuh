@@ -11,6 +11,7 @@
 #include <cmath>
 #include <type_traits>
 
+#include "fp64.cuh"
 #include "gpo_internal.h"
 
 namespace gpo {
@@ -404,11 +405,6 @@ __device__ __forceinline__ double huber_weight(double s, double delta) {
     return sqrt(delta / sqrt(s));
   }
 }
-// Huber value rho(s) (FP64): s inside delta^2, 2 delta sqrt(s) - delta^2 outside.
-__device__ __forceinline__ double huber_rho(double s, double delta) {
-  if (delta > 0.0 && s > delta * delta) return 2.0 * delta * sqrt(s) - delta * delta;
-  return s;
-}
 
 // ---------------------------------------------------------------- BA model
 
@@ -467,13 +463,23 @@ struct ModelBA {
     r[1] = r1;
   }
 
-  // 1/2 rho of an edge (cost only).
+  // rho of an edge (cost only; the caller halves the sum).  Written for few FP64 operations,
+  // which bound the cost kernel: 28 and 8 more outside the Huber threshold.
   __device__ static double cost(const DevBA& d, int e, const double* rb, const double* X) {
-    Geom g;
-    geom(rb, X, g);
-    double r[M];
-    residual(d, e, g, r);
-    return 0.5 * huber_rho(r[0] * r[0] + r[1] * r[1], __ldg(d.e_delta + e));
+    double P[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+      P[i] = fma(rb[3 * i], X[0], fma(rb[3 * i + 1], X[1], fma(rb[3 * i + 2], X[2], rb[9 + i])));
+    const double iz = -rcp_newton(P[2]), p0 = P[0] * iz, p1 = P[1] * iz;
+    const double r2 = fma(p0, p0, p1 * p1), fd = rb[12] * fma(r2, fma(r2, rb[14], rb[13]), 1.0);
+    const double2 z = __ldg(reinterpret_cast<const double2*>(d.obs) + e);
+    double r0 = fma(fd, p0, -z.x), r1 = fma(fd, p1, -z.y);
+    if (d.e_sqinfo) {
+      const double* U = d.e_sqinfo + NQ * (size_t)e;
+      r0 = U[0] * r0 + U[1] * r1;
+      r1 = U[2] * r1;
+    }
+    return huber_value(fma(r0, r0, r1 * r1), __ldg(d.e_delta + e));
   }
 
   // Whitened residual, Huber, and the whitened, sqrt(rho')-scaled Jacobian rows on the
@@ -702,12 +708,35 @@ struct ModelStereo {
     r[0] = e0; r[1] = e1; r[2] = e2;
   }
 
+  // rho of an edge (cost only; the caller halves the sum), pinhole rigs with few FP64
+  // operations.
   __device__ static double cost(const DevBA& d, int e, const double* rb, const double* X) {
-    Geom g;
-    geom(d, rb, X, g);
     double r[M];
-    residual(d, e, g, r);
-    return 0.5 * huber_rho(r[0] * r[0] + r[1] * r[1] + r[2] * r[2], __ldg(d.e_delta + e));
+    if (d.camk[17] != 0.0) {
+      Geom g;
+      geom(d, rb, X, g);
+      residual(d, e, g, r);
+    } else {
+      const double a0 = X[0] - rb[9], a1 = X[1] - rb[10], a2 = X[2] - rb[11];
+      const double* Rc = d.camk + 5;
+      double b[3], c[3];
+#pragma unroll
+      for (int i = 0; i < 3; ++i) b[i] = fma(rb[i], a0, fma(rb[3 + i], a1, rb[6 + i] * a2));   // R^T (X - p)
+#pragma unroll
+      for (int i = 0; i < 3; ++i) c[i] = fma(Rc[3 * i], b[0], fma(Rc[3 * i + 1], b[1], fma(Rc[3 * i + 2], b[2], d.camk[14 + i])));
+      const double iz = rcp_newton(c[2]), fx = d.camk[0] * iz;
+      const double* z = d.obs + 3 * (size_t)e;
+      const double e0 = fma(fx, c[0], d.camk[2] - z[0]), e1 = fma(d.camk[1] * iz, c[1], d.camk[3] - z[1]);
+      const double e2 = fma(fx, c[0] - d.camk[4], d.camk[2] - z[2]);
+      r[0] = e0; r[1] = e1; r[2] = e2;
+      if (d.e_sqinfo) {
+        const double* U = d.e_sqinfo + NQ * (size_t)e;
+        r[0] = U[0] * e0 + U[1] * e1 + U[2] * e2;
+        r[1] = U[3] * e1 + U[4] * e2;
+        r[2] = U[5] * e2;
+      }
+    }
+    return huber_value(fma(r[0], r[0], fma(r[1], r[1], r[2] * r[2])), __ldg(d.e_delta + e));
   }
 
   // dr/dX_c rows: [fx/Z, 0, -fx X/Z^2], [0, fy/Z, -fy Y/Z^2], [fx/Z, 0, -fx (X-b)/Z^2];

@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(kThreads) k_cost(LaunchSet ls, int candidate) 
     const double X[3] = {Xp[0], Xp[1], Xp[2]};
     acc += Mo::cost(d, e, rb, X);
   }
-  const double s = block_sum(acc, red);
+  const double s = 0.5 * block_sum(acc, red);
   if (threadIdx.x == 0) d.cost_part[kl] = s;
 }
 

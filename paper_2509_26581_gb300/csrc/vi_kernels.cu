@@ -317,7 +317,7 @@ __global__ void __launch_bounds__(kCamPerBlock * 32) k_extra_eval(LaunchSet ls, 
       }
       for (int p = 0; p < kXRows; ++p) d.xe_r[(size_t)x * kXRows + p] = r[p];
     } else {
-      d.xe_cost[x] = 0.5 * huber_rho(s, delta);
+      d.xe_cost[x] = 0.5 * huber_value(s, delta);
     }
   }
 }
