@@ -740,7 +740,7 @@ static gpo_status prepare(gpo_graph* g) {
   pl.add_raw(&d.y, (size_t)DB * C * sA); pl.add_raw(&d.xbest, (size_t)DB * C * sA);
   pl.add_raw(&d.p2, (size_t)DB * C * sA);
   pl.add(&d.cost_part, std::max(NCH, 1)); pl.add(&d.md_part, std::max(NCH, 1));
-  pl.add(&d.cblk_part, 2 * 5 * (size_t)d.ncblk);   // four camera-half CTAs per camera block, then the update's
+  pl.add(&d.cblk_part, 2 * 12 * (size_t)d.ncblk);   // four camera-half CTAs per camera block, then the update's (per camera in the resident PCG)
   pl.add(&d.hist, gpo::kMaxHistory);
   pl.add(&R.desc_d, 1);
   R.bytes = pl.total();
@@ -855,6 +855,7 @@ gpo_status gpo_host::finalize(gpo_graph* g, size_t* plan_bytes) {
     g->ks->ex_plan(ls, g->prec, d.C, R.ex_nb_max, d.E, st);
     ls.ex_scratch = nullptr;
   }
+  if (ls.mf && ls.n_ch && ls.n_cb) gpo_host::plan_resident(*g->ks, g->prec, {make_int2(ls.n_ch, ls.n_cb)}, ls);
   g->ls = ls;
   g->dev_desc = R.desc_d;
   g->ch_max = R.ch;
@@ -1008,12 +1009,20 @@ static void capture_pcg_group(gpo_graph* g, const gpo::LaunchSet& ls) {
   if (graph) cudaGraphDestroy(graph);
 }
 
+// The resident PCG (profiling times the launches of an iteration apart).
+static bool resident(const gpo_graph* g, const gpo::LaunchSet& ls) { return ls.res_m > 0 && !g->pcg_full && !g->prof.on; }
+
 // PCG iterations with early exit: iterations are launched in groups; after each
 // group the done flag is copied back, and the flag of the previous group decides
 // whether to launch more (one group of look-ahead keeps the GPU busy).  Full groups
 // replay a captured CUDA graph unless profiling is on (which times every launch).
 static gpo_status pcg_solve(gpo_graph* g, const gpo::LaunchSet& ls, int max_it) {
   if (gpo_status s = gpo_host::ensure_runtime(g); s != GPO_OK) return s;
+  if (resident(g, ls)) {
+    int n = 0;
+    run(g, KK_EX_PCG, [&] { n = g->ks->pcg_resident(ls, g->prec, max_it + max_it / 4 + 1, g->stream); return std::max(n, 0); });
+    return n < 0 ? fail(g, GPO_ERR_CUDA, "the launch of the PCG solve was refused") : GPO_OK;
+  }
   const int kGroup = kPcgGroup;
   int launched = 0, slot = 0, pending = -1;
   // restart iterations (at most one per four PCG iterations) are launched on top of
@@ -1108,6 +1117,21 @@ static gpo_status ensure_full(gpo_graph* g) {
   return GPO_OK;
 }
 
+// Plans the resident PCG of a launch set: the fewest chunks per CTA at which the CTAs fit the
+// device at once (probs: chunks and camera blocks per problem).
+void gpo_host::plan_resident(const gpo::KernelSet& ks, Prec pr, const std::vector<int2>& probs, gpo::LaunchSet& ls) {
+  for (ls.res_m = 1; ls.res_m <= gpo::kResChunks; ++ls.res_m) {
+    const int slots = ks.res_slots(ls, pr);
+    ls.res_ctas = 0;
+    for (const int2& p : probs) ls.res_ctas += gpo::resident_ctas(p.x, p.y, ls.res_m);
+    for (const int2& p : probs)   // the block sums of the residual norms fit the passes' scratch
+      if (16 * (size_t)p.y > (size_t)ks.DC * (ls.ch_max + 1) * sizeof(float)) ls.res_ctas = slots + 1;
+    if (slots <= 0) break;
+    if (ls.res_ctas <= slots) return;
+  }
+  ls.res_m = ls.res_ctas = 0;
+}
+
 static gpo_status solve_matrix_free(gpo_graph* g, const gpo::LaunchSet& ls, int max_it);
 
 gpo_status gpo_host::solve_system(gpo_graph* g, const gpo::LaunchSet& ls, int max_it, bool force_lin) {
@@ -1118,7 +1142,7 @@ gpo_status gpo_host::solve_system(gpo_graph* g, const gpo::LaunchSet& ls, int ma
   if (ls.ex && !g->pcg_full) {   // explicit Schur complement (of the problems that have one planned)
     if (ls.mf) run(g, KK_SCHUR, [&] { return g->ks->schur_prepare(ls, g->prec, g->stream); });
     run(g, KK_EX_FORM, [&] { return g->ks->ex_form(ls, g->prec, g->stream); });
-    if (ls.mf) GPO_CUDA(g, cudaMemsetAsync(ls.running, 0, 6 * sizeof(int), g->stream));
+    if (ls.mf && !resident(g, ls)) GPO_CUDA(g, cudaMemsetAsync(ls.running, 0, 6 * sizeof(int), g->stream));
     run(g, KK_CAM_FINALIZE, [&] { return g->ks->cam_finalize(ls, g->prec, g->stream); });
     int n = 0;
     run(g, KK_EX_PCG, [&] { n = g->ks->ex_pcg(ls, g->prec, g->stream); return std::max(n, 0); });
@@ -1139,7 +1163,7 @@ gpo_status gpo_host::solve_system(gpo_graph* g, const gpo::LaunchSet& ls, int ma
 
 static gpo_status solve_matrix_free(gpo_graph* g, const gpo::LaunchSet& ls, int max_it) {
   run(g, KK_SCHUR, [&] { return g->ks->schur_prepare(ls, g->prec, g->stream); });
-  GPO_CUDA(g, cudaMemsetAsync(ls.running, 0, 6 * sizeof(int), g->stream));   // flags and work counters
+  if (!resident(g, ls)) GPO_CUDA(g, cudaMemsetAsync(ls.running, 0, 6 * sizeof(int), g->stream));   // flags and work counters
   if (g->pcg_full) run(g, KK_FULL_INIT, [&] { return g->ks->full_init(ls, g->prec, g->stream); });
   run(g, KK_CAM_FINALIZE, [&] { return g->ks->cam_finalize(ls, g->prec, g->stream); });
   GPO_CUDA(g, cudaGetLastError());
@@ -1154,14 +1178,15 @@ static gpo_status solve_matrix_free(gpo_graph* g, const gpo::LaunchSet& ls, int 
 // The flags and counters of the whole-grid PCG solves start at zero; end_solves waits for
 // the stream and reports a solve whose grid barrier gave up.
 gpo_status gpo_host::begin_solves(gpo_graph* g, const gpo::LaunchSet& ls) {
-  if (ls.ex) GPO_CUDA(g, cudaMemsetAsync(ls.running, 0, 6 * sizeof(int), g->stream));
+  if (ls.ex || resident(g, ls)) GPO_CUDA(g, cudaMemsetAsync(ls.running, 0, 6 * sizeof(int), g->stream));
   return GPO_OK;
 }
 gpo_status gpo_host::end_solves(gpo_graph* g, const gpo::LaunchSet& ls) {
-  if (ls.n_xg) GPO_CUDA(g, cudaMemcpyAsync(g->h_flag, ls.running, 2 * sizeof(int), cudaMemcpyDeviceToHost, g->stream));
+  const bool flag = ls.n_xg || resident(g, ls);
+  if (flag) GPO_CUDA(g, cudaMemcpyAsync(g->h_flag, ls.running, 2 * sizeof(int), cudaMemcpyDeviceToHost, g->stream));
   GPO_CUDA(g, cudaStreamSynchronize(g->stream));
   g->up_busy = false;
-  if (ls.n_xg && g->h_flag[1]) return fail(g, GPO_ERR_TIMEOUT, "a bounded device wait in the PCG solve gave up");
+  if (flag && g->h_flag[1]) return fail(g, GPO_ERR_TIMEOUT, "a bounded device wait in the PCG solve gave up");
   return GPO_OK;
 }
 
@@ -2110,6 +2135,16 @@ gpo_status gpo_debug_wait_timeout(gpo_graph* g) {
   GPO_CUDA(g, cudaStreamSynchronize(g->stream));
   GPO_CUDA(g, cudaMemsetAsync(g->ls.running, 0, 6 * sizeof(int), g->stream));   // leave clean counters
   GPO_CUDA(g, cudaStreamSynchronize(g->stream));
+  if (ls.res_m && flags[1]) {   // the resident solve's wait as well
+    ls.debug_wait = 0;
+    g->ks->cam_finalize(ls, g->prec, g->stream);
+    ls.debug_wait = 1;
+    if (g->ks->pcg_resident(ls, g->prec, 1, g->stream) < 0) return fail(g, GPO_ERR_CUDA, "the launch of the PCG solve was refused");
+    GPO_CUDA(g, cudaMemcpyAsync(flags, ls.running, sizeof(flags), cudaMemcpyDeviceToHost, g->stream));
+    GPO_CUDA(g, cudaStreamSynchronize(g->stream));
+    GPO_CUDA(g, cudaMemsetAsync(g->ls.running, 0, 6 * sizeof(int), g->stream));
+    GPO_CUDA(g, cudaStreamSynchronize(g->stream));
+  }
   if (!fused) return fail(g, GPO_ERR_UNSUPPORTED, "the camera blocks do not fit one resident wave");
   if (flags[1]) return fail(g, GPO_ERR_TIMEOUT, "the PCG kernel's grid barrier gave up");
   return fail(g, GPO_ERR_STATE, "the grid barrier did not give up");

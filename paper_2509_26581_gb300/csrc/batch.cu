@@ -136,6 +136,9 @@ gpo_status build_set(gpo_graph* owner, const std::vector<gpo_graph*>& gs, BatchS
   ls.n_cl = (int)cl_prob.size();
   ls.n_xg = (int)out.grids.size();
   ls.cl_smem = cl_smem;
+  std::vector<int2> sizes;
+  for (const gpo_graph* g : gs) sizes.push_back(make_int2(g->ls.n_ch, g->ls.n_cb));
+  if (mf && !cb_prob.empty()) plan_resident(*gs[0]->ks, owner->prec, sizes, ls);
   out.ls = ls;
   out.mem = mem;
   out.staging = stage_d;
@@ -486,7 +489,7 @@ gpo_status gpo_server_step(gpo_server* sv, int32_t* n_resident, int32_t* n_queue
     gpo_status s = begin_solves(owner, sv->set.ls);
     if (s == GPO_OK) s = solve_system(owner, sv->set.ls, max_it, false);
     if (s == GPO_OK) s = finish_iteration(owner, sv->set.ls);
-    if (s == GPO_OK && sv->set.ls.n_xg) s = end_solves(owner, sv->set.ls);
+    if (s == GPO_OK && (sv->set.ls.n_xg || sv->set.ls.res_m)) s = end_solves(owner, sv->set.ls);
     if (s != GPO_OK) return s;
     ++sv->steps;
     // 3. retirement of graphs that ran all their iterations

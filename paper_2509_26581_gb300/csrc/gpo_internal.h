@@ -30,6 +30,7 @@ constexpr int kGroupEdges = 64;     // edges of a warp group (two per lane) of a
 constexpr int kMaxGroups = 16;      // warp groups per chunk
 constexpr int kMaxHistory = 4096;
 // explicit Schur complement (schur_explicit.cuh)
+constexpr int kResChunks = 2;      // chunks per CTA of the resident PCG at most
 constexpr int kExThreads = 512;     // CTA size of the PCG solve
 constexpr int kExCluster = 8;       // CTAs of a small problem's solve (a cluster)
 constexpr int kExGrid = 152;        // CTAs of a larger one's (one per SM)
@@ -94,6 +95,8 @@ struct Scalars {
   float beta_f, inv_n_f; // beta and inv_n rounded to FP32 once, where they are set (the
                          // FP32 kernels read these: a conversion from FP64 per thread
                          // would occupy the part's small FP64 pipe)
+  unsigned int bar[4];   // the resident PCG: arrivals of a solve after the products, the
+                         // camera halves and the updates, and whether it broke down
 };
 
 struct IterRecord {       // mirrors gpo_iter_record
@@ -224,6 +227,13 @@ struct DevBA {
 
 enum class Prec { F64 = 0, F32 = 1, BF16 = 2 };
 
+constexpr int kApplySplit = 4;      // CTAs per camera block in the camera half (two cameras each)
+// CTAs of a problem: its chunks dealt res_m each, at least one per unit of the camera half.
+__host__ __device__ inline int resident_ctas(int chunks, int cam_blocks, int m) {
+  const int a = (chunks + m - 1) / m, b = cam_blocks * kApplySplit;
+  return a > b ? a : b;
+}
+
 // A launch over several independent problems (one problem for a plain graph).
 // Every CTA finds its problem through a schedule table and binds that problem's
 // DevBA (device copy) in shared memory:
@@ -249,6 +259,8 @@ struct LaunchSet {
                          // waits for this many CTAs more than the grid, so that its
                          // bounded wait gives up
   int nprob, n_ch, n_cb, n_pb;
+  int res_m, res_ctas;   // the whole PCG in one launch on the matrix-free product: chunks per
+                         // CTA (0: the launches of an iteration) and CTAs
   int ch_max;            // largest chunk over the problems (shared-memory sizing)
   int ns_max, np_max;    // most slots / points in one chunk over the problems
   // explicit Schur complement: problems that use it (DevBA::ex; 0: none of the launch
@@ -290,6 +302,8 @@ struct KernelSet {
   // launch was refused)
   int (*ex_plan)(const LaunchSet& ls, Prec pr, int C, int nb_max, int E, cudaStream_t st);
   int (*ex_form)(const LaunchSet& ls, Prec pr, cudaStream_t st);
+  int (*res_slots)(const LaunchSet& ls, Prec pr);   // CTAs of the resident PCG that fit at once with ls.res_m chunks each (0: not for it)
+  int (*pcg_resident)(const LaunchSet& ls, Prec pr, int max_launch, cudaStream_t st);   // the whole PCG, < 0: refused
   int (*ex_pcg)(const LaunchSet& ls, Prec pr, cudaStream_t st);
   size_t (*ex_smem)(Prec pr, int C, int G, int nloc, int nres);   // shared memory of a solve by G CTAs
   bool (*ex_grid_ok)(Prec pr, size_t smem);                       // a grid solve with that much can be launched

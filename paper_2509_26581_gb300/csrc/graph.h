@@ -157,6 +157,7 @@ gpo_lm_params params_or_default(const gpo_lm_params* p);
 // on g's stream, counting launches in g's profiler.
 gpo_status solve_system(gpo_graph* g, const gpo::LaunchSet& ls, int max_it, bool force_lin);
 // Around the solves of a call: clear their flags; wait, and report a wait that gave up.
+void plan_resident(const gpo::KernelSet& ks, Prec pr, const std::vector<int2>& probs, gpo::LaunchSet& ls);
 gpo_status begin_solves(gpo_graph* g, const gpo::LaunchSet& ls);
 gpo_status end_solves(gpo_graph* g, const gpo::LaunchSet& ls);
 // Retraction, candidate cost, decision and commit over `ls`.

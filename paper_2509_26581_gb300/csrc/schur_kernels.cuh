@@ -766,6 +766,7 @@ __global__ void __launch_bounds__(kCamPerBlock * 32) k_cam_finalize(LaunchSet ls
     sc->inv_n_f = 1.0f;
     sc->beta_f = 0.0f;
     sc->pidx = 0;
+    sc->bar[0] = sc->bar[1] = sc->bar[2] = sc->bar[3] = 0u;
     sc->pcg_it = 0;
     sc->pcg_products = 0;
     sc->restart = 0;
@@ -790,7 +791,6 @@ __global__ void __launch_bounds__(kCamPerBlock * 32) k_cam_finalize(LaunchSet ls
 // partials and of its camera-side edges; the quarters are added in a fixed order).  The CTAs of camera block b
 // are 4b .. 4b + 3, two cameras each.  The last CTA of the problem reduces p^T y and
 // sets alpha = r^T z / p^T y.
-constexpr int kApplySplit = 4;
 template <class Mo, class AT>
 struct ApplyShared {
   double red[kCamPerBlock];
@@ -1009,21 +1009,12 @@ __device__ __forceinline__ void pcg_update_load(const DevBA& d, int cbl, UpdateI
   }
 }
 
-// The end of a PCG update, reached by every CTA of the update after writing its
-// partial (r^T z, |r|^2): the last one of the problem sums the camera blocks' partials
-// (and, in the full-system form, the point blocks' after them), applies the stopping
-// rules (tolerance, rejection ratio, iteration cap) and computes beta and the
-// normalisation factor.
-__device__ inline void pcg_update_finish(const LaunchSet& ls, const DevBA& d, int restart) {
-  Scalars* sc = d.sc;
-  const int full = sc->full;
-  const int npb = full ? update_point_blocks(d.P) : 0;   // the update's point CTAs
-  if (!last_cta(&sc->ticket, d.ncblk + npb)) return;
-  // the solve's state, read by thread 0 in one batch while the partials are summed (read
-  // one at a time between the writes below, they were a chain of dependent round trips)
-  double sigma = 0.0, rmin = 0.0, ratio = 0.0, tol_abs = 0.0, rz_old = 0.0;
-  int pcg_it = 0, max_it = 0, normalize = 0, restart_every = 0, pidx = 0, pcg_total = 0, pcg_products = 0;
-  if (threadIdx.x == 0) {
+// The solve's state that the stopping rules read (read one at a time between the rules'
+// writes, these were a chain of dependent round trips).
+struct SolveState {
+  double sigma, rmin, ratio, tol_abs, rz_old;
+  int pcg_it, max_it, normalize, restart_every, pidx, pcg_total, pcg_products;
+  __device__ __forceinline__ void load(const Scalars* sc) {
     sigma = sc->sigma;
     rmin = sc->rmin;
     ratio = sc->ratio;
@@ -1037,6 +1028,79 @@ __device__ inline void pcg_update_finish(const LaunchSet& ls, const DevBA& d, in
     pcg_total = sc->pcg_total;
     pcg_products = sc->pcg_products;
   }
+};
+
+// The stopping rules on the new residual's r^T z and |r|^2, beta and the normalisation
+// factor (one thread); returns whether the solve has ended.
+__device__ __forceinline__ int pcg_rules(Scalars* sc, const SolveState& st, double rz, double rr, int restart) {
+  double sigma = st.sigma, rmin = st.rmin;
+  int pcg_it = st.pcg_it;
+  const double n = sqrt(rr);
+  if (restart) sigma = 1.0;                // r is now the true residual
+  const double rtrue = sigma * n;
+  if (!restart) pcg_it += 1;               // a restart is an extra product, not an iteration
+  int done = 0, save_best = 0, have_best = 0, use_best = 0, breakdown = 0;
+  if (st.ratio > 0.0) {
+    if (rtrue < rmin) {
+      rmin = rtrue;
+      save_best = 1;
+      have_best = 1;
+    } else if (rtrue > st.ratio * rmin) {
+      done = 1;
+      use_best = 1;
+    }
+  }
+  if (rtrue <= st.tol_abs || pcg_it >= st.max_it || !isfinite(rtrue) || !(rz > 0.0)) {
+    done = 1;
+    if (!isfinite(rtrue)) use_best = 1;
+    // r^T M r not positive before the tolerance is met: the preconditioned system is
+    // not positive definite at this damping (after at least one step)
+    if (!(rz > 0.0) && !(rtrue <= st.tol_abs)) breakdown = 1;
+  }
+  const double beta = restart ? 0.0 : rz / st.rz_old;   // a restart starts the direction from z
+  double inv_n, rz_new;
+  if (st.normalize && n > 0.0) {
+    inv_n = 1.0 / n;
+    sigma *= n;
+    rz_new = rz / (n * n);
+  } else {
+    inv_n = 1.0;
+    rz_new = rz;
+  }
+  sc->sigma = sigma;
+  sc->pcg_it = pcg_it;
+  sc->pcg_total = st.pcg_total + 1;
+  sc->pcg_products = st.pcg_products + 1;
+  sc->rnorm = rtrue;
+  sc->rmin = rmin;
+  sc->save_best = save_best;
+  if (have_best) sc->have_best = 1;
+  if (use_best) sc->use_best = 1;
+  if (breakdown) sc->pcg_breakdown = 1;
+  sc->beta = beta;
+  sc->inv_n = inv_n;
+  sc->rz = rz_new;
+  sc->beta_f = (float)beta;
+  sc->inv_n_f = (float)inv_n;
+  if (!restart) sc->pidx = st.pidx ^ 1;       // a restart wrote no new direction
+  sc->restart = (!done && !restart && st.restart_every > 0 && pcg_it % st.restart_every == 0) ? 1 : 0;
+  sc->pcg_done = done;
+  return done;
+}
+
+// The end of a PCG update, reached by every CTA of the update after writing its
+// partial (r^T z, |r|^2): the last one of the problem sums the camera blocks' partials
+// (and, in the full-system form, the point blocks' after them), applies the stopping
+// rules (tolerance, rejection ratio, iteration cap) and computes beta and the
+// normalisation factor.
+__device__ inline void pcg_update_finish(const LaunchSet& ls, const DevBA& d, int restart) {
+  Scalars* sc = d.sc;
+  const int full = sc->full;
+  const int npb = full ? update_point_blocks(d.P) : 0;   // the update's point CTAs
+  if (!last_cta(&sc->ticket, d.ncblk + npb)) return;
+  // the solve's state, read by thread 0 in one batch while the partials are summed
+  SolveState st;
+  if (threadIdx.x == 0) st.load(sc);
   double rz, rr;
   sum_partials(d.cblk_part + 2 * kApplySplit * (size_t)d.ncblk, d.ncblk, rz, rr);
   if (full) {
@@ -1047,56 +1111,7 @@ __device__ inline void pcg_update_finish(const LaunchSet& ls, const DevBA& d, in
     rr += rrq;
   }
   if (threadIdx.x == 0) {
-    const double n = sqrt(rr);
-    if (restart) sigma = 1.0;                // r is now the true residual
-    const double rtrue = sigma * n;
-    if (!restart) pcg_it += 1;               // a restart is an extra product, not an iteration
-    int done = 0, save_best = 0, have_best = 0, use_best = 0, breakdown = 0;
-    if (ratio > 0.0) {
-      if (rtrue < rmin) {
-        rmin = rtrue;
-        save_best = 1;
-        have_best = 1;
-      } else if (rtrue > ratio * rmin) {
-        done = 1;
-        use_best = 1;
-      }
-    }
-    if (rtrue <= tol_abs || pcg_it >= max_it || !isfinite(rtrue) || !(rz > 0.0)) {
-      done = 1;
-      if (!isfinite(rtrue)) use_best = 1;
-      // r^T M r not positive before the tolerance is met: the preconditioned system is
-      // not positive definite at this damping (after at least one step)
-      if (!(rz > 0.0) && !(rtrue <= tol_abs)) breakdown = 1;
-    }
-    const double beta = restart ? 0.0 : rz / rz_old;   // a restart starts the direction from z
-    double inv_n, rz_new;
-    if (normalize && n > 0.0) {
-      inv_n = 1.0 / n;
-      sigma *= n;
-      rz_new = rz / (n * n);
-    } else {
-      inv_n = 1.0;
-      rz_new = rz;
-    }
-    sc->sigma = sigma;
-    sc->pcg_it = pcg_it;
-    sc->pcg_total = pcg_total + 1;
-    sc->pcg_products = pcg_products + 1;
-    sc->rnorm = rtrue;
-    sc->rmin = rmin;
-    sc->save_best = save_best;
-    if (have_best) sc->have_best = 1;
-    if (use_best) sc->use_best = 1;
-    if (breakdown) sc->pcg_breakdown = 1;
-    sc->beta = beta;
-    sc->inv_n = inv_n;
-    sc->rz = rz_new;
-    sc->beta_f = (float)beta;
-    sc->inv_n_f = (float)inv_n;
-    if (!restart) sc->pidx = pidx ^ 1;       // a restart wrote no new direction
-    sc->restart = (!done && !restart && restart_every > 0 && pcg_it % restart_every == 0) ? 1 : 0;
-    sc->pcg_done = done;
+    const int done = pcg_rules(sc, st, rz, rr, restart);
     if (done) atomicSub(ls.running, 1);
     sc->ticket = 0u;
   }
@@ -1616,6 +1631,7 @@ static void set_smem(const void* kernel, size_t bytes) {
 
 #include "schur_full.cuh"
 #include "autodiff.cuh"
+#include "schur_resident.cuh"
 #include "schur_explicit.cuh"
 
 namespace gpo {
@@ -1796,6 +1812,46 @@ struct Launch {
     }
     const int grid = std::max(1, std::min(ls.n_ch, n_sm * std::max(occ, 1)));
     launch_pdl(k_spmv_ws<Mo, JT>, grid, kWsThreads, sm, st, ls);
+  }
+  // The resident PCG: BF16 and FP32 storage, chunks of at most 512 edges.
+  template <class JT>
+  static int res_slots_t(const LaunchSet& ls) {
+    const size_t sm = resident_layout<Mo>(sizeof(typename AccOf<JT>::T), ls.ch_max, ls.np_max, ls.ns_max, ls.res_m).size;
+    if (sm > 200 * 1024) return 0;
+    int dev = 0, n_sm = 0, occ = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+    set_smem(reinterpret_cast<const void*>(k_pcg_resident<Mo, JT, 2>), sm);
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_pcg_resident<Mo, JT, 2>, kThreads, sm) != cudaSuccess) {
+      cudaGetLastError();
+      return 0;
+    }
+    return occ * n_sm;
+  }
+  static int res_slots(const LaunchSet& ls, Prec pr) {
+    if constexpr (Mo::kExtra) return 0;
+    else if (pr == Prec::F64 || ls.spmv_variant != 0 || ls.ch_max > 2 * kThreads || ls.nprob > 256) return 0;
+    else return pr == Prec::F32 ? res_slots_t<float>(ls) : res_slots_t<__nv_bfloat16>(ls);
+  }
+  template <class JT>
+  static int pcg_resident_t(const LaunchSet& ls, int max_launch, cudaStream_t st) {
+    const size_t sm = resident_layout<Mo>(sizeof(typename AccOf<JT>::T), ls.ch_max, ls.np_max, ls.ns_max, ls.res_m).size;
+    set_smem(reinterpret_cast<const void*>(k_pcg_resident<Mo, JT, 2>), sm);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)ls.res_ctas);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = sm;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_pcg_resident<Mo, JT, 2>, ls, max_launch) == cudaSuccess ? 1 : -1;
+  }
+  static int pcg_resident(const LaunchSet& ls, Prec pr, int max_launch, cudaStream_t st) {
+    if constexpr (Mo::kExtra) return -1;
+    else return pr == Prec::F32 ? pcg_resident_t<float>(ls, max_launch, st) : pcg_resident_t<__nv_bfloat16>(ls, max_launch, st);
   }
   static size_t pp_smem(Prec pr, const LaunchSet& ls) {
     return pipe_layout<Mo>(sA(pr), ls.ch_max, ls.np_max, ls.ns_max).size;
@@ -2202,6 +2258,8 @@ KernelSet make_kernel_set(ModelKind kind) {
   k.ex_form = &L::ex_form;
   k.ex_pcg = &L::ex_pcg;
   k.ex_smem = &L::ex_smem;
+  k.res_slots = &L::res_slots;
+  k.pcg_resident = &L::pcg_resident;
   k.ex_grid_ok = &L::ex_grid_ok;
   k.ex_sizes = &L::ex_sizes;
   k.backsub = &L::backsub;
