@@ -1030,62 +1030,58 @@ struct SolveState {
   }
 };
 
-// The stopping rules on the new residual's r^T z and |r|^2, beta and the normalisation
-// factor (one thread); returns whether the solve has ended.
-__device__ __forceinline__ int pcg_rules(Scalars* sc, const SolveState& st, double rz, double rr, int restart) {
-  double sigma = st.sigma, rmin = st.rmin;
-  int pcg_it = st.pcg_it;
-  const double n = sqrt(rr);
-  if (restart) sigma = 1.0;                // r is now the true residual
-  const double rtrue = sigma * n;
-  if (!restart) pcg_it += 1;               // a restart is an extra product, not an iteration
-  int done = 0, save_best = 0, have_best = 0, use_best = 0, breakdown = 0;
+// The stopping rules on the new residual's r^T z and norm n (one thread): what they decide,
+// and its record with beta, the normalisation factor 1 / n (if set) and the scaled r^T z.
+struct RuleFlags {
+  double rtrue, rmin;
+  int pcg_it, done, save_best, have_best, use_best, breakdown;
+};
+__device__ __forceinline__ RuleFlags pcg_flags(const SolveState& st, double rz, double n, int restart) {
+  RuleFlags f;
+  f.rmin = st.rmin;
+  f.pcg_it = st.pcg_it;
+  const double rtrue = f.rtrue = (restart ? 1.0 : st.sigma) * n;   // after a restart r is the true residual
+  if (!restart) f.pcg_it += 1;             // a restart is an extra product, not an iteration
+  f.done = f.save_best = f.have_best = f.use_best = f.breakdown = 0;
   if (st.ratio > 0.0) {
-    if (rtrue < rmin) {
-      rmin = rtrue;
-      save_best = 1;
-      have_best = 1;
-    } else if (rtrue > st.ratio * rmin) {
-      done = 1;
-      use_best = 1;
+    if (rtrue < f.rmin) {
+      f.rmin = rtrue;
+      f.save_best = 1;
+      f.have_best = 1;
+    } else if (rtrue > st.ratio * f.rmin) {
+      f.done = 1;
+      f.use_best = 1;
     }
   }
-  if (rtrue <= st.tol_abs || pcg_it >= st.max_it || !isfinite(rtrue) || !(rz > 0.0)) {
-    done = 1;
-    if (!isfinite(rtrue)) use_best = 1;
+  if (rtrue <= st.tol_abs || f.pcg_it >= st.max_it || !isfinite(rtrue) || !(rz > 0.0)) {
+    f.done = 1;
+    if (!isfinite(rtrue)) f.use_best = 1;
     // r^T M r not positive before the tolerance is met: the preconditioned system is
     // not positive definite at this damping (after at least one step)
-    if (!(rz > 0.0) && !(rtrue <= st.tol_abs)) breakdown = 1;
+    if (!(rz > 0.0) && !(rtrue <= st.tol_abs)) f.breakdown = 1;
   }
-  const double beta = restart ? 0.0 : rz / st.rz_old;   // a restart starts the direction from z
-  double inv_n, rz_new;
-  if (st.normalize && n > 0.0) {
-    inv_n = 1.0 / n;
-    sigma *= n;
-    rz_new = rz / (n * n);
-  } else {
-    inv_n = 1.0;
-    rz_new = rz;
-  }
+  return f;
+}
+__device__ __forceinline__ void pcg_record(Scalars* sc, const SolveState& st, const RuleFlags& f, double beta,
+                                           double inv_n, double sigma, double rz, int restart) {
   sc->sigma = sigma;
-  sc->pcg_it = pcg_it;
+  sc->pcg_it = f.pcg_it;
   sc->pcg_total = st.pcg_total + 1;
   sc->pcg_products = st.pcg_products + 1;
-  sc->rnorm = rtrue;
-  sc->rmin = rmin;
-  sc->save_best = save_best;
-  if (have_best) sc->have_best = 1;
-  if (use_best) sc->use_best = 1;
-  if (breakdown) sc->pcg_breakdown = 1;
+  sc->rnorm = f.rtrue;
+  sc->rmin = f.rmin;
+  sc->save_best = f.save_best;
+  if (f.have_best) sc->have_best = 1;
+  if (f.use_best) sc->use_best = 1;
+  if (f.breakdown) sc->pcg_breakdown = 1;
   sc->beta = beta;
   sc->inv_n = inv_n;
-  sc->rz = rz_new;
+  sc->rz = rz;
   sc->beta_f = (float)beta;
   sc->inv_n_f = (float)inv_n;
   if (!restart) sc->pidx = st.pidx ^ 1;       // a restart wrote no new direction
-  sc->restart = (!done && !restart && st.restart_every > 0 && pcg_it % st.restart_every == 0) ? 1 : 0;
-  sc->pcg_done = done;
-  return done;
+  sc->restart = (!f.done && !restart && st.restart_every > 0 && f.pcg_it % st.restart_every == 0) ? 1 : 0;
+  sc->pcg_done = f.done;
 }
 
 // The end of a PCG update, reached by every CTA of the update after writing its
@@ -1111,8 +1107,17 @@ __device__ inline void pcg_update_finish(const LaunchSet& ls, const DevBA& d, in
     rr += rrq;
   }
   if (threadIdx.x == 0) {
-    const int done = pcg_rules(sc, st, rz, rr, restart);
-    if (done) atomicSub(ls.running, 1);
+    const double n = sqrt(rr);
+    const RuleFlags f = pcg_flags(st, rz, n, restart);
+    const double beta = restart ? 0.0 : rz / st.rz_old;   // a restart starts the direction from z
+    double inv_n = 1.0, sigma = restart ? 1.0 : st.sigma, rz_new = rz;
+    if (st.normalize && n > 0.0) {
+      inv_n = 1.0 / n;
+      sigma *= n;
+      rz_new = rz / (n * n);
+    }
+    pcg_record(sc, st, f, beta, inv_n, sigma, rz_new, restart);
+    if (f.done) atomicSub(ls.running, 1);
     sc->ticket = 0u;
   }
 }
