@@ -136,11 +136,11 @@ __device__ __forceinline__ int xrows(int kind) { return kind == XK_IMU ? 9 : 6; 
 // ---------------------------------------------------------------- camera render blocks
 
 template <class Mo>
-__global__ void __launch_bounds__(kCamPerBlock * 32) k_cam_prepare(LaunchSet ls, int candidate) {
+__global__ void __launch_bounds__(32) k_cam_prepare(LaunchSet ls, int candidate) {
   GPO_BIND(cb, cbl)
   if (!d.sc->active) return;
-  const int c = cbl * kCamPerBlock + (threadIdx.x >> 5);
-  if (c >= d.C || (threadIdx.x & 31) != 0) return;
+  const int c = cbl * kCamPerBlock + threadIdx.x;   // a lane per camera: see k_retract_cams
+  if (c >= d.C || threadIdx.x >= kCamPerBlock) return;
   const double* cam = (candidate ? d.cam_cand : d.cam) + Mo::SS * (size_t)c;
   double* rb = (candidate ? d.camrb_cand : d.camrb) + 16 * (size_t)c;
   float* rbf = (candidate ? d.camrbf_cand : d.camrbf) + 16 * (size_t)c;
@@ -1454,13 +1454,17 @@ __global__ void __launch_bounds__(kThreads) k_backsub(LaunchSet ls) {
 
 // ---------------------------------------------------------------- retraction (FP64)
 
+// A lane per camera, one warp per camera block: bound by FP64 issue (one warp instruction
+// holds a sub-partition some 70 clocks whatever its active lanes), so a warp per camera
+// made a sub-partition take every instruction of two cameras in turn.  With the points'
+// kernel, 20 cameras 31 -> 21 us, 4,000 cameras 117 -> 39; k_cam_prepare of 4,000 35 -> 14.
 template <class Mo, class AT>
-__global__ void __launch_bounds__(kCamPerBlock * 32) k_retract_cams(LaunchSet ls) {
+__global__ void __launch_bounds__(32) k_retract_cams(LaunchSet ls) {
   constexpr int SS = Mo::SS, DB = Mo::DB;
   GPO_BIND(cb, cbl)
   if (!d.sc->active) return;
-  const int c = cbl * kCamPerBlock + (threadIdx.x >> 5);
-  if (c >= d.C || (threadIdx.x & 31) != 0) return;
+  const int c = cbl * kCamPerBlock + threadIdx.x;
+  if (c >= d.C || threadIdx.x >= kCamPerBlock) return;
   const double* cur = d.cam + SS * (size_t)c;
   double* nxt = d.cam_cand + SS * (size_t)c;
   double* rb = d.camrb_cand + 16 * (size_t)c;
@@ -1709,7 +1713,7 @@ struct Launch {
 
   static int cam_prepare(const LaunchSet& ls, bool candidate, cudaStream_t st) {
     if (ls.n_cb == 0) return 0;
-    launch_pdl(k_cam_prepare<Mo>, ls.n_cb, kCamPerBlock * 32, 0, st, ls, candidate ? 1 : 0);
+    launch_pdl(k_cam_prepare<Mo>, ls.n_cb, 32, 0, st, ls, candidate ? 1 : 0);
     return 1;
   }
   static int cost(const LaunchSet& ls, bool candidate, cudaStream_t st) {
@@ -2218,10 +2222,10 @@ struct Launch {
   static int retract(const LaunchSet& ls, Prec pr, cudaStream_t st) {
     int n = 0;
     if (pr == Prec::F64) {
-      if (ls.n_cb) { launch_pdl(k_retract_cams<Mo, double>, ls.n_cb, kCamPerBlock * 32, 0, st, ls); ++n; }
+      if (ls.n_cb) { launch_pdl(k_retract_cams<Mo, double>, ls.n_cb, 32, 0, st, ls); ++n; }
       if (ls.n_pb) { launch_pdl(k_retract_pts<Mo, double>, ls.n_pb, 256, 0, st, ls); ++n; }
     } else {
-      if (ls.n_cb) { launch_pdl(k_retract_cams<Mo, float>, ls.n_cb, kCamPerBlock * 32, 0, st, ls); ++n; }
+      if (ls.n_cb) { launch_pdl(k_retract_cams<Mo, float>, ls.n_cb, 32, 0, st, ls); ++n; }
       if (ls.n_pb) { launch_pdl(k_retract_pts<Mo, float>, ls.n_pb, 256, 0, st, ls); ++n; }
     }
     return n;
