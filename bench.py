@@ -238,7 +238,7 @@ def load_peaks() -> tuple[float, str]:
 # DRAM bytes (read + write) per Schur-product launch on the medium workload, counted by
 # ncu, keyed by (precision, kernel, hash of the kernel sources): stale once the sources
 # change.
-MEASURED_TRAFFIC = {("bf16", "k_spmv_pp", "7fc91d8044b4"): 179.2e6}
+MEASURED_TRAFFIC = {("bf16", "k_spmv_pp", "5dffd4067dfb"): 181.3e6}
 SPMV_VARIANTS = {"auto": 0, "staged": 1, "classic": 2, "pipelined": 3, "dynamic": 4, "warpgroup": 5,
                  "warpgroup_staged": 6}
 KERNEL_SOURCES = ("schur_common.cuh", "schur_spmv.cuh")
@@ -269,7 +269,25 @@ def spmv_kernel(precision: str, knobs: dict, ch_max: int) -> str:
     return "k_spmv"
 
 
-KERNEL_LABEL = {"k_spmv_wgs": "k_spmv_wgs (PCG Schur product, warp groups fed through shared-memory stages)",
+def product_kernel(g, precision: str) -> str:
+    """The kernel that takes the graph's Schur products (the explicit complement's PCG solve
+    when the graph has one planned)."""
+    info = g.info()
+    return "k_ex_pcg" if info["spmv_kernel"] == 7 else spmv_kernel(precision, g.knobs, info["chunk_edges"])
+
+
+def product_rate(prof: dict, algorithmic_bytes: float):
+    """(ms per Schur product, GB/s) of the profiled launches; (None, 0) where the products
+    are not launches of their own."""
+    sp = prof["spmv"]
+    if not sp["active"]:
+        return None, 0.0
+    ms = sp["active_ms"] / sp["active"]
+    return ms, algorithmic_bytes / (ms * 1e-3) / 1e9
+
+
+KERNEL_LABEL = {"k_ex_pcg": "k_ex_pcg (PCG solve on the explicit Schur complement; no launch per product)",
+                "k_spmv_wgs": "k_spmv_wgs (PCG Schur product, warp groups fed through shared-memory stages)",
                 "k_spmv_wg": "k_spmv_wg (PCG Schur product, warp groups)",
                 "k_spmv_pp": "k_spmv_pp (PCG Schur product, pipelined persistent)",
                 "k_spmv_ws": "k_spmv_ws (PCG Schur product, staged)",
@@ -525,10 +543,7 @@ def extra_vi(dev, stream, iters: int = 10) -> dict:
         g.set_profiling(True)
         g.optimize(iters, params)
         prof = g.profile()
-        sp = prof["spmv"]
-        spmv_ms = sp["active_ms"] / sp["active"] if sp["active"] else float("nan")
-        alg = spmv_algorithmic_bytes_vi(p.n_edges, p.n_pts, prec)
-        gbs = alg / (spmv_ms * 1e-3) / 1e9 if sp["active"] else 0.0
+        spmv_ms, gbs = product_rate(prof, spmv_algorithmic_bytes_vi(p.n_edges, p.n_pts, prec))
         costs[prec] = rep.final_cost
         out[prec] = dict(lm_iter_per_s=iters / (ms / 1e3), initial_cost=rep.initial_cost,
                          final_cost=rep.final_cost, accepted=rep.accepted,
@@ -602,19 +617,16 @@ def extra_large(dev, stream, iters: int = 20) -> dict:
         g.set_profiling(True)
         g.optimize(3, params)
         prof = g.profile()
-        sp = prof["spmv"]
-        spmv_ms = sp["active_ms"] / sp["active"] if sp["active"] else float("nan")
         acc_ms = sum(prof[k]["active_ms"] / max(1, prof[k]["active"]) for k in ("linearize", "schur_prepare"))
-        alg_s = spmv_algorithmic_bytes(p.n_edges, p.n_pts, prec)
+        spmv_ms, gbs = product_rate(prof, spmv_algorithmic_bytes(p.n_edges, p.n_pts, prec))
         alg_a = accumulation_bytes(p.n_edges, p.n_pts, info["slots"], prec)
         out[prec] = dict(lm_iter_per_s=iters / (ms / 1e3), initial_cost=rep.initial_cost,
                          final_cost=rep.final_cost, accepted=rep.accepted,
                          first_accepted_iter=next((k for k, r in enumerate(h) if r["accepted"]), None),
                          pcg_failed=int(sum(r["pcg_failed"] for r in h)), pcg_iters=rep.pcg_iters_total,
                          footprint_bytes=g.footprint(), schedule=g.knobs,
-                         spmv=dict(kernel=spmv_kernel(prec, g.knobs, info["chunk_edges"]), avg_ms=spmv_ms,
-                                   achieved_gbs=alg_s / (spmv_ms * 1e-3) / 1e9,
-                                   frac=alg_s / (spmv_ms * 1e-3) / 1e9 / peak),
+                         spmv=dict(kernel=product_kernel(g, prec), avg_ms=spmv_ms, achieved_gbs=gbs,
+                                   frac=gbs / peak),
                          accumulation=dict(avg_ms=acc_ms, achieved_gbs=alg_a / (acc_ms * 1e-3) / 1e9,
                                            frac=alg_a / (acc_ms * 1e-3) / 1e9 / peak))
         g.close()
@@ -738,11 +750,9 @@ def run_vi(args, dev, stream, world: int) -> dict:
     g.set_profiling(True)
     g.optimize(args.steps, params)
     prof = g.profile()
-    sp = prof["spmv"]
     peak, peak_kind = load_peaks()
     alg = spmv_algorithmic_bytes_vi(p.n_edges, p.n_pts, args.precision)
-    spmv_ms = sp["active_ms"] / sp["active"] if sp["active"] else float("nan")
-    achieved = alg / (spmv_ms * 1e-3) / 1e9 if sp["active"] else 0.0
+    spmv_ms, achieved = product_rate(prof, alg)
     return dict(
         metric=METRIC, value=world * args.steps / (ms / 1e3), unit="LM iter/s", n_gpus=world,
         steps=args.steps, warmup=args.warmup, ms_per_step=ms / args.steps, higher_is_better=True,
@@ -754,7 +764,7 @@ def run_vi(args, dev, stream, world: int) -> dict:
                     parallelism=f"replicas x{world}"),
         gpu_launches=launches,
         roofline=dict(bound="hbm", achieved=achieved, peak=peak, unit="GB/s", frac=achieved / peak, traffic=None,
-                      kernel=KERNEL_LABEL[spmv_kernel(args.precision, g.knobs, g.info()["chunk_edges"])],
+                      kernel=KERNEL_LABEL[product_kernel(g, args.precision)],
                       peak_source=peak_kind, algorithmic_bytes=alg, avg_ms=spmv_ms),
         clocks=clk, final_cost=rep.final_cost,
         kernels_ms={k: round(v["active_ms"], 3) for k, v in prof.items()},
@@ -840,15 +850,13 @@ def run_ours(args, rank: int, world: int, dist) -> dict | None:
     e2e_s = max_over_ranks(e2e_s, dist)
     if rank != 0:
         return None
-    sp = prof["spmv"]
     peak, peak_kind = load_peaks()
-    kern = spmv_kernel(args.precision, g.knobs, g.info()["chunk_edges"])
+    kern = product_kernel(g, args.precision)
     alg = spmv_algorithmic_bytes(p.n_edges, p.n_pts, args.precision)
     if args.solver == "full":   # the full-system product instead of the Schur product
         kern = "k_full_spmv"
         alg = full_algorithmic_bytes(p.n_edges, p.n_pts, args.precision)
-    spmv_ms = sp["active_ms"] / sp["active"] if sp["active"] else float("nan")
-    achieved = alg / (spmv_ms * 1e-3) / 1e9 if sp["active"] else 0.0
+    spmv_ms, achieved = product_rate(prof, alg)
     state_bytes = (p.n_cams * 9 + p.n_pts * 3) * 8
     pcg_iters = [h["pcg_iters"] for h in hist]
     line = dict(

@@ -129,7 +129,9 @@ typedef struct {
                                  blocks costs more than it saves, or for bundle
                                  adjustment with BF16 storage, or FP32 and more than
                                  65,536 points; then pipelined for BF16 and FP32
-                                 storage, classic for FP64), 1 = staged
+                                 storage, the whole PCG in one launch with the same
+                                 bits where the chunks fit the device at once; classic
+                                 for FP64), 1 = staged
                                  (persistent CTAs streaming chunks into shared memory
                                  with bulk copies), 2 = classic (one CTA per chunk),
                                  3 = pipelined (persistent CTAs prefetching the next

@@ -8,6 +8,9 @@ Two knobs of `gpo_graph_desc` change how the kernels walk a problem, not the met
                     1 = staged (persistent CTAs, warp-specialised bulk-copy pipeline),
                     3 = pipelined (persistent CTAs prefetching the next chunk's
                     indices); all give bit-identical results (see the variant tests).
+                    0 = the library's own choice, which besides these may form the Schur
+                    complement or run the whole PCG in one launch; timed at each chunk
+                    size too and taken unless another is faster by more than 1 %.
 The best choice depends on the problem's size (how many chunks fill the GPU, how many
 slots a chunk has) and on the storage precision.  `tune` times every candidate on a
 representative problem of a size class -- a few LM iterations after a warm-up, wall
@@ -31,6 +34,7 @@ TABLE = os.path.join(HERE, "tuning.json")
 SIZE_CLASSES = [(20_000, "window"), (300_000, "small"), (8_000_000, "medium"), (math.inf, "large")]
 CANDIDATES = [dict(chunk_edges=c, spmv_variant=v) for c in (256, 512, 1024) for v in (2, 1, 3)]
 DEFAULT = dict(chunk_edges=512, spmv_variant=0)
+AUTOMATIC = [dict(DEFAULT, chunk_edges=c) for c in (256, 512, 1024)]
 
 
 def size_class(n_edges: int) -> str:
@@ -77,7 +81,7 @@ def choose(n_edges: int, precision: str, model: str = "ba", table: dict | None =
     return dict(entry["best"]) if entry else dict(DEFAULT)
 
 
-def tune(build, candidates=CANDIDATES, iters: int = 3, warmup: int = 1, repeats: int = 2) -> dict:
+def tune(build, candidates=CANDIDATES + AUTOMATIC, iters: int = 3, warmup: int = 1, repeats: int = 2) -> dict:
     """Times build(**knobs).optimize(iters) for every candidate (after `warmup` LM
     iterations on the same graph, state reset in between); returns the fastest and all
     timings (seconds per LM iteration, best of `repeats`)."""
@@ -96,7 +100,7 @@ def tune(build, candidates=CANDIDATES, iters: int = 3, warmup: int = 1, repeats:
             best = min(best, (time.perf_counter() - t0) / iters)
         g.close()
         timings.append(dict(knobs=knobs, s_per_iter=best))
-    fastest = min(timings, key=lambda t: t["s_per_iter"])
+    fastest = min(timings, key=lambda t: t["s_per_iter"] * (1.0 if t["knobs"].get("spmv_variant") == 0 else 1.01))
     return dict(best=fastest["knobs"], timings=timings)
 
 

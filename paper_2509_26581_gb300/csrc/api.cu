@@ -245,11 +245,14 @@ static bool explicit_allowed(const gpo_graph* g, const gpo::KernelSet& ks, int P
 // not allowed (above), a camera sees a point twice, or forming the blocks costs more than
 // they save.
 //
-// The rule compares times on the GB300.  Forming: 0.014 ns per row pair in FP32 (about
-// four cycles per pair and SM), 0.46 ns in FP64 (243 FP64 multiply-adds per pair at the
+// The rule compares times on the GB300.  Forming: 0.024 ns per row pair in FP32 (18.5
+// million pairs of 1,000 cameras in 437 us), 0.46 ns in FP64 (243 FP64 multiply-adds per pair at the
 // pipe's rate).  A matrix-free iteration: 0.026 ns per edge in FP32 and BF16 storage, 0.21
 // ns in FP64, and 20 us of launches and barriers; an explicit one: the blocks' bytes at 6
-// TB/s and 6 us.  A solve is taken to have 16 iterations (solves to 1e-6 took 11 to 100).
+// TB/s and 6 us (5.3 to 9.7 measured with on-chip blocks).  A solve is taken to have 16
+// iterations (solves to 1e-6 took 11 to 100).  Both sides measured: 10 cameras FP64 6,587
+// -> 3,031 us, 20 keyframes FP64 7,178 -> 2,449, 1,000 keyframes BF16 4,030 -> 1,917, 100
+// cameras FP32 2,664 -> 1,478, 300 cameras FP64 4,707 -> 3,780.
 static void plan_explicit(gpo_graph* g, Prepared& R, const gpo::KernelSet& ks, int C, int P, int E, int NS) {
   R.ex = false;
   if (!explicit_allowed(g, ks, P) || E == 0 || C < 2 || C > 32768) return;
@@ -259,7 +262,7 @@ static void plan_explicit(gpo_graph* g, Prepared& R, const gpo::KernelSet& ks, i
     pairs += k * (k - 1) / 2;
   }
   const bool f64 = g->prec == Prec::F64;
-  const double form = pairs * (f64 ? 4.6e-10 : 1.4e-11), free_it = E * (f64 ? 2.1e-10 : 2.6e-11) + 20e-6;
+  const double form = pairs * (f64 ? 4.6e-10 : 2.4e-11), free_it = E * (f64 ? 2.1e-10 : 2.6e-11) + 20e-6;
   const int EL = ks.DC * ks.DC;
   const size_t sA = at_size(g->prec);
   auto pays = [&](size_t nb) { return form + 16 * ((double)nb * EL * sA / 6e12 + 6e-6) < 16 * free_it; };
