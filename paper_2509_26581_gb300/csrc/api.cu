@@ -462,11 +462,14 @@ static gpo_status prepare(gpo_graph* g) {
       deg[p]++;
     }
   std::vector<int32_t> cnt(C + 2, 0), by_last(P);
-  if (!explicit_allowed(g, ks, P)) std::fill(last.begin(), last.end(), 0);
-  for (int p = 0; p < P; ++p) cnt[last[p] + 1]++;
-  for (int k = 0; k <= C; ++k) cnt[k + 1] += cnt[k];
-  for (int p = 0; p < P; ++p) by_last[cnt[last[p]]++] = p;
-  std::fill(cnt.begin(), cnt.end(), 0);
+  if (explicit_allowed(g, ks, P)) {
+    for (int p = 0; p < P; ++p) cnt[last[p] + 1]++;
+    for (int k = 0; k <= C; ++k) cnt[k + 1] += cnt[k];
+    for (int p = 0; p < P; ++p) by_last[cnt[last[p]]++] = p;
+    std::fill(cnt.begin(), cnt.end(), 0);
+  } else {
+    for (int p = 0; p < P; ++p) by_last[p] = p;
+  }
   for (int p = 0; p < P; ++p) cnt[key[p] + 1]++;
   for (int k = 0; k <= C; ++k) cnt[k + 1] += cnt[k];
   R.pt_new2old.assign(P, 0);
@@ -748,7 +751,7 @@ static gpo_status prepare(gpo_graph* g) {
   pl.add(&R.desc_d, 1);
   R.bytes = pl.total();
   // the explicit Schur complement, unless the memory budget holds the graph only without
-  {
+  if (explicit_allowed(g, ks, P)) {
     Plan plain = pl;
     plan_explicit(g, R, ks, C, P, E, NS);
     if (R.ex && g->desc.memory_budget && pl.total() > g->desc.memory_budget) R.ex = false;
@@ -1129,7 +1132,6 @@ void gpo_host::plan_resident(const gpo::KernelSet& ks, Prec pr, const std::vecto
     for (const int2& p : probs) ls.res_ctas += gpo::resident_ctas(p.x, p.y, ls.res_m);
     for (const int2& p : probs)   // the block sums of the residual norms fit the passes' scratch
       if (16 * (size_t)p.y > (size_t)ks.DC * (ls.ch_max + 1) * sizeof(float)) ls.res_ctas = slots + 1;
-    if (slots <= 0) break;
     if (ls.res_ctas <= slots) return;
   }
   ls.res_m = ls.res_ctas = 0;
@@ -1263,12 +1265,13 @@ gpo_status gpo_host::ensure_stream(gpo_graph* g) {
 gpo_status gpo_host::ensure_runtime(gpo_graph* g) {
   if (g->h_sc) return GPO_OK;
   if (gpo_status s = ensure_stream(g); s != GPO_OK) return s;
-  GPO_CUDA(g, cudaMallocHost(&g->h_flag, 4 * sizeof(int)));
-  GPO_CUDA(g, cudaMallocHost(&g->h_changed, sizeof(int)));
+  // one pinned block: the scalars uploaded, the flags, the range check's call number
+  GPO_CUDA(g, cudaMallocHost(&g->h_up, sizeof(Scalars) + 8 * sizeof(int)));
+  g->h_flag = reinterpret_cast<int*>(g->h_up + 1);
+  g->h_changed = g->h_flag + 4;
   GPO_CUDA(g, cudaMalloc(&g->d_changed, sizeof(int)));
   GPO_CUDA(g, cudaMemsetAsync(g->d_changed, 0, sizeof(int), g->stream));
   *g->h_changed = 0;
-  GPO_CUDA(g, cudaMallocHost(&g->h_up, sizeof(Scalars)));
   GPO_CUDA(g, cudaEventCreateWithFlags(&g->ev[0], cudaEventDisableTiming));
   GPO_CUDA(g, cudaEventCreateWithFlags(&g->ev[1], cudaEventDisableTiming));
   GPO_CUDA(g, cudaMallocHost(&g->h_sc, sizeof(Scalars)));   // last: marks the runtime as ready
@@ -1351,8 +1354,6 @@ gpo_status gpo_graph_destroy(gpo_graph* g) {
   release_device(g);
   if (g->h_sc) cudaFreeHost(g->h_sc);
   if (g->h_up) cudaFreeHost(g->h_up);
-  if (g->h_flag) cudaFreeHost(g->h_flag);
-  if (g->h_changed) cudaFreeHost(g->h_changed);
   if (g->d_changed) cudaFree(g->d_changed);
   for (auto& ev : g->prof.pool)
     if (ev) cudaEventDestroy(ev);

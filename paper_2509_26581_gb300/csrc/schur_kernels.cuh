@@ -1830,6 +1830,9 @@ struct Launch {
     int dev = 0, n_sm = 0, occ = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+    // the register bound alone: a set that does not fit by it needs no occupancy query (a
+    // server plans a set at every admission)
+    if (ls.n_ch > ls.res_m * n_sm * (sizeof(JT) == 2 ? 4 : 3)) return 0;
     set_smem(reinterpret_cast<const void*>(k_pcg_resident<Mo, JT, 2>), sm);
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_pcg_resident<Mo, JT, 2>, kThreads, sm) != cudaSuccess) {
       cudaGetLastError();
