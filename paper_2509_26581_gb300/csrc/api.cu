@@ -177,6 +177,7 @@ void gpo_host::release_device(gpo_graph* g) {
   g->arena = nullptr;
   g->arena_bytes = 0;
   g->finalized = false;
+  g->uploading = false;
   g->state_same = false;
 }
 
@@ -874,9 +875,28 @@ gpo_status gpo_host::finalize(gpo_graph* g, size_t* plan_bytes) {
   g->x_sorted = std::move(R.x_sorted);
   g->dev = d;
   g->finalized = true;
+  g->uploading = true;
   g->prep.reset();
   g->state_same = false;
   GPO_CUDA(g, cudaGetLastError());
+  return GPO_OK;
+}
+
+// A graph that a batch or a server finalizes uploads on its own stream and is then solved on
+// the owner's: the kernels there wait for an event behind the upload.  (One event serves all
+// graphs: a wait is for the record before it.)
+gpo_status gpo_host::join_uploads(gpo_graph* owner, const std::vector<gpo_graph*>& graphs) {
+  cudaEvent_t ev = nullptr;
+  cudaError_t e = cudaSuccess;
+  for (gpo_graph* g : graphs) {
+    if (!g->uploading || g->stream == owner->stream) continue;
+    if (!ev) e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventRecord(ev, g->stream);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(owner->stream, ev, 0);
+    if (e != cudaSuccess) break;
+  }
+  if (ev) cudaEventDestroy(ev);
+  GPO_CUDA(owner, e);
   return GPO_OK;
 }
 
@@ -1190,7 +1210,7 @@ gpo_status gpo_host::end_solves(gpo_graph* g, const gpo::LaunchSet& ls) {
   const bool flag = ls.n_xg || resident(g, ls);
   if (flag) GPO_CUDA(g, cudaMemcpyAsync(g->h_flag, ls.running, 2 * sizeof(int), cudaMemcpyDeviceToHost, g->stream));
   GPO_CUDA(g, cudaStreamSynchronize(g->stream));
-  g->up_busy = false;
+  g->up_busy = g->uploading = false;
   if (flag && g->h_flag[1]) return fail(g, GPO_ERR_TIMEOUT, "a bounded device wait in the PCG solve gave up");
   return GPO_OK;
 }
@@ -1217,7 +1237,7 @@ static gpo_status compute_cost(gpo_graph* g, double* out) {
   if (s != GPO_OK) return s;
   GPO_CUDA(g, cudaMemcpyAsync(g->h_sc, g->dev.sc, sizeof(Scalars), cudaMemcpyDeviceToHost, g->stream));
   GPO_CUDA(g, cudaStreamSynchronize(g->stream));
-  g->up_busy = false;
+  g->up_busy = g->uploading = false;
   *out = g->h_sc->cost;
   return GPO_OK;
 }
@@ -1678,7 +1698,7 @@ gpo_status gpo_set_initial(gpo_graph* g, int64_t first, int64_t n, const double*
   GPO_CUDA(g, cudaGetLastError());
   if (tmp) GPO_CUDA(g, cudaFreeAsync(tmp, st));
   GPO_CUDA(g, cudaStreamSynchronize(st));
-  g->up_busy = false;
+  g->up_busy = g->uploading = false;
   if (*reinterpret_cast<volatile int*>(g->h_changed) == call) {
     g->cost_valid = false;
     g->state_same = false;

@@ -281,7 +281,8 @@ gpo_status gpo_optimize_batch(gpo_graph* const* graphs, int32_t n, int32_t max_i
   if (!(prm.initial_damping > 0.0)) return fail(owner, GPO_ERR_ARG, "initial damping must be positive");
   std::vector<gpo_graph*> gs(graphs, graphs + n);
   BatchSet bs;
-  gpo_status s = build_set(owner, gs, bs);
+  gpo_status s = join_uploads(owner, gs);
+  if (s == GPO_OK) s = build_set(owner, gs, bs);
   if (s != GPO_OK) return s;
   std::vector<Scalars> sc(n);
   for (int i = 0; i < n; ++i) {
@@ -323,7 +324,8 @@ gpo_status gpo_optimize_batch(gpo_graph* const* graphs, int32_t n, int32_t max_i
     prof_resolve(owner);
   }
   bs.release(owner->stream);
-  cudaStreamSynchronize(owner->stream);
+  if (cudaStreamSynchronize(owner->stream) == cudaSuccess)
+    for (int i = 0; i < n; ++i) graphs[i]->uploading = false;
   return s;
 }
 
@@ -448,7 +450,8 @@ gpo_status gpo_server_step(gpo_server* sv, int32_t* n_resident, int32_t* n_queue
     std::vector<gpo_graph*> gs;
     for (auto& r : adm) gs.push_back(r.g);
     BatchSet bs;
-    gpo_status s = build_set(owner, gs, bs);
+    gpo_status s = join_uploads(owner, gs);
+    if (s == GPO_OK) s = build_set(owner, gs, bs);
     if (s != GPO_OK) return s;
     std::vector<Scalars> sc(adm.size());
     for (size_t i = 0; i < adm.size(); ++i) {

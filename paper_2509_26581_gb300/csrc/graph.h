@@ -86,6 +86,7 @@ struct gpo_graph {
   // finalized topology
   std::unique_ptr<Prepared, PrepDeleter> prep;   // planned, not yet uploaded
   bool finalized = false;
+  bool uploading = false;          // finalize's copies and kernels may still run on `stream`
   const gpo::KernelSet* ks = nullptr;
   int ch_max = 0;
   std::vector<int64_t> sorted_edge;   // sorted position -> observation edge index
@@ -156,8 +157,11 @@ gpo_lm_params params_or_default(const gpo_lm_params* p);
 // One LM iteration's solve (linearise, Schur, PCG, back-substitution) over `ls`
 // on g's stream, counting launches in g's profiler.
 gpo_status solve_system(gpo_graph* g, const gpo::LaunchSet& ls, int max_it, bool force_lin);
-// Around the solves of a call: clear their flags; wait, and report a wait that gave up.
+// Orders owner's stream after the uploads that are still running on the graphs' own streams.
+gpo_status join_uploads(gpo_graph* owner, const std::vector<gpo_graph*>& graphs);
+// Plans the one-launch matrix-free PCG of a launch set (probs: chunks and camera blocks).
 void plan_resident(const gpo::KernelSet& ks, Prec pr, const std::vector<int2>& probs, gpo::LaunchSet& ls);
+// Around the solves of a call: clear their flags; wait, and report a wait that gave up.
 gpo_status begin_solves(gpo_graph* g, const gpo::LaunchSet& ls);
 gpo_status end_solves(gpo_graph* g, const gpo::LaunchSet& ls);
 // Retraction, candidate cost, decision and commit over `ls`.
