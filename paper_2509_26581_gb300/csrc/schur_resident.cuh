@@ -343,7 +343,9 @@ __global__ void __launch_bounds__(kThreads, sizeof(JT) == 2 ? 4 : 3) k_pcg_resid
           }
         }
       }
-      // ---- alpha from all units' p^T y (a restart's product needs none)
+      // ---- alpha from all units' p^T y (a restart's product needs none, but its arrivals
+      // count: they show that every unit has read the last update's norms in upart, which
+      // the update below overwrites; units without chunks arrive nowhere else before it)
       if (!restart) {
         AT dot = lead ? pi * yi : (AT)0;
 #pragma unroll
@@ -355,8 +357,10 @@ __global__ void __launch_bounds__(kThreads, sizeof(JT) == 2 ? 4 : 3) k_pcg_resid
           for (int w = 0; w < kCamPerBlock; w += kApplySplit) a += dots[w];   // the other warps' are zero
           d.cblk_part[2 * rank] = a;
         }
-        res_arrive(bar + 1);
-        if (!(ok = res_wait(bar + 1, (unsigned)units * (unsigned)(s.pcg_it + 1)))) break;
+      }
+      res_arrive(bar + 1);
+      if (!(ok = res_wait(bar + 1, (unsigned)units * (unsigned)(it + 1)))) break;
+      if (!restart) {
         double pAp = 0.0;   // by two warps, for the two coefficients
         if (units > 32) pAp = sum_partials_first(d.cblk_part, units);
         else if (warp < 2) pAp = res_tree(lane < units ? d.cblk_part[2 * lane] : 0.0, units);
