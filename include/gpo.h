@@ -584,15 +584,22 @@ gpo_status gpo_debug_schur(gpo_graph* g, double lambda, const gpo_lm_params* par
                            double* S_out, double* g_out);
 
 /* Failure-detection test of the bounded device waits: prepares one PCG solve and
- * launches the fused camera kernel (camera half of the Schur product and PCG update)
- * with its grid barrier waiting for one CTA more than the grid, so that nothing can
- * complete it.  The barrier's bounded wait (1 s) gives up, the kernel raises the
- * error flag and returns.  Returns GPO_ERR_TIMEOUT when that happened (the expected
+ * launches the fused camera kernel (camera half of the Schur product and PCG update) or
+ * the whole-grid solve of an explicit Schur complement, then the graph's other one-launch
+ * solve if it has one, each waiting for one CTA more than there are, so that nothing can
+ * complete the wait.  The bounded wait (1 s) gives up, the kernel raises the error flag
+ * and returns.  Returns GPO_ERR_TIMEOUT when that happened (the expected
  * result), GPO_ERR_UNSUPPORTED when the graph's camera blocks do not fit one resident
  * wave (the fused kernel is then not used), GPO_ERR_STATE otherwise.  The graph's
  * device counters are left clean and the context usable: a later gpo_optimize runs
  * as if this call had not been made. */
 gpo_status gpo_debug_wait_timeout(gpo_graph* g);
+
+/* Test hook for the same waits inside solves: while `on`, the solves of this graph, and of
+ * batches and server steps that hold it (a server's from the graph's admission on), wait for
+ * an arrival that does not come, and so end with GPO_ERR_TIMEOUT after about a second where
+ * the PCG runs in one launch or in the fused camera kernel. */
+gpo_status gpo_debug_hold_waits(gpo_graph* g, int32_t on);
 
 #ifdef __cplusplus
 }

@@ -840,6 +840,7 @@ gpo_status gpo_host::finalize(gpo_graph* g, size_t* plan_bytes) {
   ls.work = R.running_d + 2;
   ls.spmv_variant = g->desc.spmv_variant;
   ls.nprob = 1; ls.n_ch = R.NCH; ls.n_cb = d.C > 0 ? d.ncblk : 0; ls.n_pb = d.P > 0 ? R.npb : 0;
+  ls.debug_wait = g->debug_wait;
   ls.ch_max = R.ch;
   ls.ns_max = d.ns_max;
   ls.np_max = d.np_max;
@@ -1200,14 +1201,14 @@ static gpo_status solve_matrix_free(gpo_graph* g, const gpo::LaunchSet& ls, int 
   return GPO_OK;
 }
 
-// The flags and counters of the whole-grid PCG solves start at zero; end_solves waits for
-// the stream and reports a solve whose grid barrier gave up.
+// The flags and counters of the one-launch PCG solves start at zero; end_solves waits for
+// the stream and reports a solve one of whose waits gave up.
 gpo_status gpo_host::begin_solves(gpo_graph* g, const gpo::LaunchSet& ls) {
   if (ls.ex || resident(g, ls)) GPO_CUDA(g, cudaMemsetAsync(ls.running, 0, 6 * sizeof(int), g->stream));
   return GPO_OK;
 }
 gpo_status gpo_host::end_solves(gpo_graph* g, const gpo::LaunchSet& ls) {
-  const bool flag = ls.n_xg || resident(g, ls);
+  const bool flag = ls.ex || resident(g, ls);
   if (flag) GPO_CUDA(g, cudaMemcpyAsync(g->h_flag, ls.running, 2 * sizeof(int), cudaMemcpyDeviceToHost, g->stream));
   GPO_CUDA(g, cudaStreamSynchronize(g->stream));
   g->up_busy = g->uploading = false;
@@ -2146,7 +2147,7 @@ gpo_status gpo_debug_wait_timeout(gpo_graph* g) {
   g->ks->cam_prepare(g->ls, false, g->stream);
   g->ks->linearize(g->ls, g->prec, true, g->stream);
   gpo::LaunchSet ls = g->ls;
-  if (!ls.n_xg) ls.ex = 0;   // a cluster's solve has no such wait: the matrix-free camera kernel's
+  if (!ls.n_xg) ls.ex = 0;   // a cluster's solve, below, and the matrix-free camera kernel
   if (ls.ex) g->ks->ex_form(ls, g->prec, g->stream);
   else g->ks->schur_prepare(ls, g->prec, g->stream);
   GPO_CUDA(g, cudaMemsetAsync(g->ls.running, 0, 6 * sizeof(int), g->stream));
@@ -2169,9 +2170,27 @@ gpo_status gpo_debug_wait_timeout(gpo_graph* g) {
     GPO_CUDA(g, cudaMemsetAsync(g->ls.running, 0, 6 * sizeof(int), g->stream));
     GPO_CUDA(g, cudaStreamSynchronize(g->stream));
   }
+  if (g->ls.n_cl && (flags[1] || !fused)) {   // a cluster's wait
+    ls = g->ls;
+    ls.debug_wait = 1;
+    g->ks->ex_form(ls, g->prec, g->stream);
+    g->ks->cam_finalize(ls, g->prec, g->stream);
+    if (g->ks->ex_pcg(ls, g->prec, g->stream) < 0) return fail(g, GPO_ERR_CUDA, "the launch of the PCG solve was refused");
+    GPO_CUDA(g, cudaMemcpyAsync(flags, ls.running, sizeof(flags), cudaMemcpyDeviceToHost, g->stream));
+    GPO_CUDA(g, cudaStreamSynchronize(g->stream));
+    GPO_CUDA(g, cudaMemsetAsync(ls.running, 0, 6 * sizeof(int), g->stream));
+    GPO_CUDA(g, cudaStreamSynchronize(g->stream));
+    if (!flags[1]) return fail(g, GPO_ERR_STATE, "the cluster's wait did not give up");
+  }
   if (!fused) return fail(g, GPO_ERR_UNSUPPORTED, "the camera blocks do not fit one resident wave");
   if (flags[1]) return fail(g, GPO_ERR_TIMEOUT, "the PCG kernel's grid barrier gave up");
   return fail(g, GPO_ERR_STATE, "the grid barrier did not give up");
+}
+
+gpo_status gpo_debug_hold_waits(gpo_graph* g, int32_t on) {
+  if (!g) return GPO_ERR_ARG;
+  g->ls.debug_wait = g->debug_wait = on ? 1 : 0;
+  return GPO_OK;
 }
 
 gpo_status gpo_debug_schur(gpo_graph* g, double lambda, const gpo_lm_params* params, double* S_out, double* g_out) {

@@ -35,7 +35,7 @@ struct BatchSet {
   char* mem = nullptr;
   Scalars* staging = nullptr;    // device [n]
   std::vector<int4> grids;       // problems whose PCG takes a whole grid (ls.xg_host)
-  int n = 0;
+  int n = 0, debug_wait = 0;
 
   void release(cudaStream_t st) {
     if (mem) cudaFreeAsync(mem, st);
@@ -51,6 +51,7 @@ gpo_status build_set(gpo_graph* owner, const std::vector<gpo_graph*>& gs, BatchS
   std::vector<int> xf_prob, xd_prob, cl_prob, xf_base(n), xd_base(n);   // explicit Schur complement
   int ch_max = 32, ns_max = 1, np_max = 1, mf = 0, ex = 0, cl_smem = 0;
   out.grids.clear();
+  out.debug_wait = 0;
   for (int q = 0; q < n; ++q) {
     const gpo_graph* g = gs[q];
     probs[q] = g->dev;
@@ -60,6 +61,7 @@ gpo_status build_set(gpo_graph* owner, const std::vector<gpo_graph*>& gs, BatchS
     ch_prob.insert(ch_prob.end(), g->ls.n_ch, q);
     cb_prob.insert(cb_prob.end(), g->ls.n_cb, q);
     pb_prob.insert(pb_prob.end(), g->ls.n_pb, q);
+    out.debug_wait |= g->debug_wait;
     ch_max = std::max(ch_max, g->ls.ch_max);
     ns_max = std::max(ns_max, g->ls.ns_max);
     np_max = std::max(np_max, g->ls.np_max);
@@ -119,6 +121,7 @@ gpo_status build_set(gpo_graph* owner, const std::vector<gpo_graph*>& gs, BatchS
   ls.err = running_d + 1;
   ls.work = running_d + 2;
   ls.spmv_variant = owner->desc.spmv_variant;
+  ls.debug_wait = out.debug_wait;
   ls.nprob = n;
   ls.n_ch = (int)ch_prob.size();
   ls.n_cb = (int)cb_prob.size();
@@ -492,7 +495,7 @@ gpo_status gpo_server_step(gpo_server* sv, int32_t* n_resident, int32_t* n_queue
     gpo_status s = begin_solves(owner, sv->set.ls);
     if (s == GPO_OK) s = solve_system(owner, sv->set.ls, max_it, false);
     if (s == GPO_OK) s = finish_iteration(owner, sv->set.ls);
-    if (s == GPO_OK && (sv->set.ls.n_xg || sv->set.ls.res_m)) s = end_solves(owner, sv->set.ls);
+    if (s == GPO_OK && (sv->set.ls.ex || sv->set.ls.res_m)) s = end_solves(owner, sv->set.ls);
     if (s != GPO_OK) return s;
     ++sv->steps;
     // 3. retirement of graphs that ran all their iterations

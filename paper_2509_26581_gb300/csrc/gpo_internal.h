@@ -255,9 +255,9 @@ struct LaunchSet {
                          // grid barrier (back to 0 at every barrier), [3] its generation
   int spmv_variant;      // Schur-product kernel: 0 auto, 1 staged (bulk copies), 2 classic,
                          // 3 pipelined, 4 dynamic Jacobians
-  int debug_wait;        // test hook, 0 in production: the camera kernel's grid barrier
-                         // waits for this many CTAs more than the grid, so that its
-                         // bounded wait gives up
+  int debug_wait;        // test hook, 0 in production: the waits of the camera kernel and
+                         // of the one-launch solves are for this many CTAs more than
+                         // there are, so that they give up
   int nprob, n_ch, n_cb, n_pb;
   int res_m, res_ctas;   // the whole PCG in one launch on the matrix-free product: chunks per
                          // CTA (0: the launches of an iteration) and CTAs

@@ -105,6 +105,7 @@ struct gpo_graph {
   gpo::LaunchSet ls{};             // one-problem launch set over `dev`
   bool ex_cluster = false;         // explicit Schur complement: solved by a cluster (else a grid)
   int4 ex_grid{0, 0, 0, 0};        // the solve's launch (problem, CTAs, shared memory)
+  int debug_wait = 0;              // LaunchSet::debug_wait of the graph's solves
   DevBA* dev_desc = nullptr;       // device copy of `dev` (ls.probs)
   Scalars* h_sc = nullptr;         // pinned, read back into
   Scalars* h_up = nullptr;         // pinned, uploaded from

@@ -585,7 +585,9 @@ __host__ __device__ inline size_t ex_pcg_smem(int C, int G, int nloc, int nres) 
 // The sum over a group of CTAs of each one's v[0 .. n-1], by one warp: value w (0 or 1) of the
 // reduction `epoch`; value 1 takes part in every second one.  slot_s: [2][kExCluster][4] words
 // in the CTA's shared memory (a cluster's slots); red: [2][kExMaxCtas][4] words and the two
-// counts of posts (a grid's).  n_slot: CTAs of the group.  Sets *lost on a wait that gave up.
+// counts of posts (a grid's).  n_slot: CTAs of the group (the test hook adds one that posts
+// nothing: a grid waits for its slot, a cluster for an epoch that does not come).  Sets *lost
+// on a wait that gave up.
 template <class AT, bool kCluster>
 __device__ __noinline__ double ex_group_sum(const AT* v, int n, int w, unsigned epoch, int rank, int n_slot,
                                             unsigned long long* slot_s, unsigned long long* red, int* lost) {
@@ -600,8 +602,9 @@ __device__ __noinline__ double ex_group_sum(const AT* v, int n, int w, unsigned 
   if constexpr (kCluster) {
     if (lane < kExCluster) ex_post_cluster(cluster_addr(slot_s + (par * kExCluster + rank) * 4 + 2 * w, lane), mine, epoch);
     double u = 0.0;
+    const unsigned want = epoch + (unsigned)(n_slot - kExCluster);
     if (lane < kExCluster)
-      while (!ex_poll_shared(slot_s + (par * kExCluster + lane) * 4 + 2 * w, u, epoch) && (ok = wait.again())) {}
+      while (!ex_poll_shared(slot_s + (par * kExCluster + lane) * 4 + 2 * w, u, want) && (ok = wait.again())) {}
     if (!__all_sync(full, ok)) *lost = 1;
     return ex_warp_sum(u, kExCluster);
   } else {
@@ -751,7 +754,7 @@ __global__ void __launch_bounds__(kExThreads, 1) k_ex_pcg(LaunchSet ls, int prob
   else __syncthreads();
 
   auto group_sum = [&](const AT* v, int w) -> double {
-    return ex_group_sum<AT, kCluster>(v, nr * DB, w, epoch, rank, G + (kCluster ? 0 : ls.debug_wait),
+    return ex_group_sum<AT, kCluster>(v, nr * DB, w, epoch, rank, G + ls.debug_wait,
                                       &slot_s[0][0][0], d.ex_red, &fl[3]);
   };
   auto gave_up = [&] {   // leaves the kernel (a cluster's CTAs together: their shared memory is shared)

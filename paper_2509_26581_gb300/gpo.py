@@ -123,6 +123,7 @@ _SIGS = {
     "gpo_debug_step": (C.c_int, [_P, C.c_double, C.POINTER(gpo_lm_params), _P, C.POINTER(C.c_int32)]),
     "gpo_debug_schur": (C.c_int, [_P, C.c_double, C.POINTER(gpo_lm_params), _P, _P]),
     "gpo_debug_wait_timeout": (C.c_int, [_P]),
+    "gpo_debug_hold_waits": (C.c_int, [_P, C.c_int32]),
     "gpo_debug_autodiff_edges": (C.c_int, [_P, _P, C.c_int64, _P, _P]),
     "gpo_fp64_fma_probe": (C.c_int, [_P, C.c_int32, C.c_int32, _P]),
     "gpo_generic_create": (C.c_int, [C.c_int32, C.c_int64, _P, C.c_int32, _P, C.POINTER(_P)]),
@@ -355,6 +356,10 @@ class Graph:
     def debug_wait_timeout(self) -> int:
         """gpo_debug_wait_timeout: the status it returns (GPO_ERR_TIMEOUT expected)."""
         return int(lib.gpo_debug_wait_timeout(self.h))
+
+    def debug_hold_waits(self, on: bool) -> None:
+        """gpo_debug_hold_waits: makes the bounded waits of this graph's solves give up."""
+        _check(lib.gpo_debug_hold_waits(self.h, int(on)), self.h)
 
     def debug_schur(self, lam: float, n_cams: int, params: gpo_lm_params | None = None, db: int = 9):
         S = np.zeros((n_cams, db, db))
