@@ -334,7 +334,9 @@ gpo_status gpo_set_initial(gpo_graph* g, int64_t first_id, int64_t n, const doub
  * linearisation is kept: the values a fresh evaluation gives, without the kernels.
  * Errors: GPO_ERR_ARG, GPO_ERR_OOM, GPO_ERR_NUMERIC (non-finite initial cost),
  *         GPO_ERR_UNSUPPORTED (a point seen more than the supported maximum of
- *         times), GPO_ERR_CUDA. */
+ *         times), GPO_ERR_CUDA, GPO_ERR_TIMEOUT (a bounded device wait gave up: no step
+ *         was taken from the solve that was lost, the state is the one before it, and
+ *         the next call evaluates it afresh; so too in a batch). */
 gpo_status gpo_optimize(gpo_graph* g, int32_t max_iters, const gpo_lm_params* params,
                         gpo_report* out);
 
@@ -455,7 +457,9 @@ gpo_status gpo_server_destroy(gpo_server* sv);
 gpo_status gpo_server_submit(gpo_server* sv, gpo_graph* g, int32_t max_iters,
                              const gpo_lm_params* params, int64_t* ticket);
 /* Admission, one LM iteration of the resident graphs, retirement.  Outputs (optional):
- * graphs resident after the step, still queued, and retired by this step. */
+ * graphs resident after the step, still queued, and retired by this step.
+ * GPO_ERR_TIMEOUT: a bounded device wait gave up; the graphs whose solve was lost keep their
+ * state and make the iteration in the next step, the others are as after any step. */
 gpo_status gpo_server_step(gpo_server* sv, int32_t* n_resident, int32_t* n_queued,
                            int32_t* n_finished);
 /* *done = 1 and the report once the ticket's graph has been retired (each ticket is
@@ -595,11 +599,11 @@ gpo_status gpo_debug_schur(gpo_graph* g, double lambda, const gpo_lm_params* par
  * as if this call had not been made. */
 gpo_status gpo_debug_wait_timeout(gpo_graph* g);
 
-/* Test hook for the same waits inside solves: while `on`, the solves of this graph, and of
- * batches and server steps that hold it (a server's from the graph's admission on), wait for
- * an arrival that does not come, and so end with GPO_ERR_TIMEOUT after about a second where
- * the PCG runs in one launch or in the fused camera kernel. */
-gpo_status gpo_debug_hold_waits(gpo_graph* g, int32_t on);
+/* Test hook for the same waits inside solves: from the given LM iteration of a call on (1:
+ * the first; 0: the hook is off), the solves of this graph, and of batches and server steps
+ * that hold it, wait for an arrival that does not come, and so end with GPO_ERR_TIMEOUT
+ * after about a second where the PCG runs in one launch or in the fused camera kernel. */
+gpo_status gpo_debug_hold_waits(gpo_graph* g, int32_t from_iteration);
 
 #ifdef __cplusplus
 }

@@ -840,7 +840,6 @@ gpo_status gpo_host::finalize(gpo_graph* g, size_t* plan_bytes) {
   ls.work = R.running_d + 2;
   ls.spmv_variant = g->desc.spmv_variant;
   ls.nprob = 1; ls.n_ch = R.NCH; ls.n_cb = d.C > 0 ? d.ncblk : 0; ls.n_pb = d.P > 0 ? R.npb : 0;
-  ls.debug_wait = g->debug_wait;
   ls.ch_max = R.ch;
   ls.ns_max = d.ns_max;
   ls.np_max = d.np_max;
@@ -1202,7 +1201,8 @@ static gpo_status solve_matrix_free(gpo_graph* g, const gpo::LaunchSet& ls, int 
 }
 
 // The flags and counters of the one-launch PCG solves start at zero; end_solves waits for
-// the stream and reports a solve one of whose waits gave up.
+// the stream and reports a solve one of whose waits gave up.  Such a solve has switched its
+// problem off, so no step was taken from it.
 gpo_status gpo_host::begin_solves(gpo_graph* g, const gpo::LaunchSet& ls) {
   if (ls.ex || resident(g, ls)) GPO_CUDA(g, cudaMemsetAsync(ls.running, 0, 6 * sizeof(int), g->stream));
   return GPO_OK;
@@ -1213,6 +1213,19 @@ gpo_status gpo_host::end_solves(gpo_graph* g, const gpo::LaunchSet& ls) {
   GPO_CUDA(g, cudaStreamSynchronize(g->stream));
   g->up_busy = g->uploading = false;
   if (flag && g->h_flag[1]) return fail(g, GPO_ERR_TIMEOUT, "a bounded device wait in the PCG solve gave up");
+  return GPO_OK;
+}
+
+gpo_status gpo_host::post_flags(gpo_graph* g, const gpo::LaunchSet& ls) {
+  if (!ls.ex && !resident(g, ls)) return GPO_OK;
+  GPO_CUDA(g, cudaMemcpyAsync(g->h_flag, ls.running, 2 * sizeof(int), cudaMemcpyDeviceToHost, g->stream));
+  GPO_CUDA(g, cudaEventRecord(g->ev[0], g->stream));
+  return GPO_OK;
+}
+gpo_status gpo_host::read_flags(gpo_graph* g, const gpo::LaunchSet& ls) {
+  if (!ls.ex && !resident(g, ls)) return GPO_OK;
+  GPO_CUDA(g, cudaEventSynchronize(g->ev[0]));
+  if (g->h_flag[1]) return fail(g, GPO_ERR_TIMEOUT, "a bounded device wait in the PCG solve gave up");
   return GPO_OK;
 }
 
@@ -1761,6 +1774,8 @@ gpo_status gpo_optimize(gpo_graph* g, int32_t max_iters, const gpo_lm_params* pa
     sc.need_lin = g->last_need_lin;
     sc.cost = g->last_cost;
   }
+  const double last_cost = g->last_cost;
+  g->cost_valid = g->state_same = false;   // until the call has ended well
   if ((s = upload_scalars(g, sc)) != GPO_OK) return s;
   // the iterations follow without a look at the cost: one that is not finite switches them
   // off on the device
@@ -1768,7 +1783,10 @@ gpo_status gpo_optimize(gpo_graph* g, int32_t max_iters, const gpo_lm_params* pa
   if ((s = begin_solves(g, g->ls)) != GPO_OK) return s;
   for (int it = 0; it < max_iters; ++it) {
     g->cur_lm_iter = it;
-    if ((s = solve_system(g, g->ls, sc.max_it, false)) != GPO_OK) return s;
+    g->ls.debug_wait = held(g, it);
+    s = solve_system(g, g->ls, sc.max_it, false);
+    g->ls.debug_wait = 0;
+    if (s != GPO_OK) return s;
     if ((s = finish_iteration(g, g->ls)) != GPO_OK) return s;
   }
   g->cur_lm_iter = -1;
@@ -1779,7 +1797,7 @@ gpo_status gpo_optimize(gpo_graph* g, int32_t max_iters, const gpo_lm_params* pa
     GPO_CUDA(g, cudaMemcpyAsync(hist.data(), g->dev.hist, nh * sizeof(gpo::IterRecord),
                                 cudaMemcpyDeviceToHost, g->stream));
   if ((s = end_solves(g, g->ls)) != GPO_OK) return s;
-  const double F0 = cont ? g->last_cost : g->h_sc->cost0;
+  const double F0 = cont ? last_cost : g->h_sc->cost0;
   if (!std::isfinite(F0)) return fail(g, GPO_ERR_NUMERIC, "initial cost is not finite (%g)", F0);
   g->hist = std::move(hist);
   if (g->prof.on) prof_resolve(g);
@@ -2187,9 +2205,9 @@ gpo_status gpo_debug_wait_timeout(gpo_graph* g) {
   return fail(g, GPO_ERR_STATE, "the grid barrier did not give up");
 }
 
-gpo_status gpo_debug_hold_waits(gpo_graph* g, int32_t on) {
+gpo_status gpo_debug_hold_waits(gpo_graph* g, int32_t from_iteration) {
   if (!g) return GPO_ERR_ARG;
-  g->ls.debug_wait = g->debug_wait = on ? 1 : 0;
+  g->debug_wait = std::max(0, from_iteration);
   return GPO_OK;
 }
 

@@ -35,7 +35,7 @@ struct BatchSet {
   char* mem = nullptr;
   Scalars* staging = nullptr;    // device [n]
   std::vector<int4> grids;       // problems whose PCG takes a whole grid (ls.xg_host)
-  int n = 0, debug_wait = 0;
+  int n = 0;
 
   void release(cudaStream_t st) {
     if (mem) cudaFreeAsync(mem, st);
@@ -51,7 +51,6 @@ gpo_status build_set(gpo_graph* owner, const std::vector<gpo_graph*>& gs, BatchS
   std::vector<int> xf_prob, xd_prob, cl_prob, xf_base(n), xd_base(n);   // explicit Schur complement
   int ch_max = 32, ns_max = 1, np_max = 1, mf = 0, ex = 0, cl_smem = 0;
   out.grids.clear();
-  out.debug_wait = 0;
   for (int q = 0; q < n; ++q) {
     const gpo_graph* g = gs[q];
     probs[q] = g->dev;
@@ -61,7 +60,6 @@ gpo_status build_set(gpo_graph* owner, const std::vector<gpo_graph*>& gs, BatchS
     ch_prob.insert(ch_prob.end(), g->ls.n_ch, q);
     cb_prob.insert(cb_prob.end(), g->ls.n_cb, q);
     pb_prob.insert(pb_prob.end(), g->ls.n_pb, q);
-    out.debug_wait |= g->debug_wait;
     ch_max = std::max(ch_max, g->ls.ch_max);
     ns_max = std::max(ns_max, g->ls.ns_max);
     np_max = std::max(np_max, g->ls.np_max);
@@ -121,7 +119,6 @@ gpo_status build_set(gpo_graph* owner, const std::vector<gpo_graph*>& gs, BatchS
   ls.err = running_d + 1;
   ls.work = running_d + 2;
   ls.spmv_variant = owner->desc.spmv_variant;
-  ls.debug_wait = out.debug_wait;
   ls.nprob = n;
   ls.n_ch = (int)ch_prob.size();
   ls.n_cb = (int)cb_prob.size();
@@ -165,6 +162,18 @@ gpo_status get_scalars(gpo_graph* owner, BatchSet& bs, std::vector<Scalars>& sc)
                                   owner->stream));
   GPO_CUDA(owner, cudaStreamSynchronize(owner->stream));
   return GPO_OK;
+}
+
+// After a wait gave up: switches the problems whose solve was lost on again (their state is
+// the one before the iteration).  ran[q]: problem q has taken its step.
+gpo_status rearm(gpo_graph* owner, BatchSet& bs, bool stepped, std::vector<char>& ran) {
+  std::vector<Scalars> sc;
+  if (gpo_status s = get_scalars(owner, bs, sc); s != GPO_OK) return s;
+  for (int q = 0; q < bs.n; ++q) {
+    ran[q] = stepped && sc[q].active;
+    sc[q].active = 1;
+  }
+  return put_scalars(owner, bs, sc);
 }
 
 void report_from(const Scalars& s, double initial_cost, gpo_report* r) {
@@ -289,6 +298,7 @@ gpo_status gpo_optimize_batch(gpo_graph* const* graphs, int32_t n, int32_t max_i
   if (s != GPO_OK) return s;
   std::vector<Scalars> sc(n);
   for (int i = 0; i < n; ++i) {
+    graphs[i]->cost_valid = graphs[i]->state_same = false;   // until the call has ended well
     fill_scalars(graphs[i], prm, prm.initial_damping, sc[i]);
     sc[i].full = 0;   // shared launches run the Schur form
     graphs[i]->pcg_full = 0;
@@ -308,6 +318,7 @@ gpo_status gpo_optimize_batch(gpo_graph* const* graphs, int32_t n, int32_t max_i
     if (s == GPO_OK && (s = ensure_runtime(owner)) == GPO_OK) s = begin_solves(owner, bs.ls);
     for (int it = 0; s == GPO_OK && it < max_iters; ++it) {
       owner->cur_lm_iter = -1;
+      bs.ls.debug_wait = std::any_of(gs.begin(), gs.end(), [&](const gpo_graph* g) { return held(g, it); });
       if ((s = solve_system(owner, bs.ls, max_it, false)) != GPO_OK) break;
       s = finish_iteration(owner, bs.ls);
     }
@@ -316,7 +327,6 @@ gpo_status gpo_optimize_batch(gpo_graph* const* graphs, int32_t n, int32_t max_i
       for (int i = 0; i < n; ++i) {
         graphs[i]->last_cost = sc[i].cost;
         graphs[i]->cost_valid = true;
-        graphs[i]->state_same = false;   // a batched run: the next single run starts afresh
         graphs[i]->hist.clear();
         if (reports) report_from(sc[i], F0[i], &reports[i]);
       }
@@ -433,6 +443,7 @@ gpo_status gpo_server_step(gpo_server* sv, int32_t* n_resident, int32_t* n_queue
   gpo_graph* owner = sv->owner;
   GPO_CUDA(owner, cudaSetDevice(owner->desc.device));
   int fin = 0;
+  gpo_status late = GPO_OK;   // a wait that gave up, reported at the end
   // 1. admission: first come, first served, while slots and memory allow; the new
   //    graphs' initial costs are computed together in shared launches
   std::vector<gpo_server::Req> adm;
@@ -492,15 +503,24 @@ gpo_status gpo_server_step(gpo_server* sv, int32_t* n_resident, int32_t* n_queue
     int max_it = 1;
     for (auto& r : sv->resident) max_it = std::max(max_it, r.prm.pcg_max_iters);
     owner->cur_lm_iter = -1;
+    sv->set.ls.debug_wait = std::any_of(sv->resident.begin(), sv->resident.end(),
+                                        [](const gpo_server::Req& r) { return held(r.g, r.done_iters); });
     gpo_status s = begin_solves(owner, sv->set.ls);
     if (s == GPO_OK) s = solve_system(owner, sv->set.ls, max_it, false);
+    const bool stepped = s == GPO_OK;
+    if (s == GPO_OK) s = post_flags(owner, sv->set.ls);
     if (s == GPO_OK) s = finish_iteration(owner, sv->set.ls);
-    if (s == GPO_OK && (sv->set.ls.ex || sv->set.ls.res_m)) s = end_solves(owner, sv->set.ls);
+    if (s == GPO_OK) s = read_flags(owner, sv->set.ls);
+    std::vector<char> ran(sv->resident.size(), 1);
+    if (s == GPO_ERR_TIMEOUT) {   // the solves that were lost are made again by the next step
+      late = s;
+      s = rearm(owner, sv->set, stepped, ran);
+    }
     if (s != GPO_OK) return s;
     ++sv->steps;
     // 3. retirement of graphs that ran all their iterations
     bool any = false;
-    for (auto& r : sv->resident) any |= (++r.done_iters >= r.max_iters);
+    for (size_t i = 0; i < ran.size(); ++i) any |= ((sv->resident[i].done_iters += ran[i]) >= sv->resident[i].max_iters);
     if (any) {
       std::vector<Scalars> sc;
       if ((s = get_scalars(owner, sv->set, sc)) != GPO_OK) return s;
@@ -544,7 +564,7 @@ gpo_status gpo_server_step(gpo_server* sv, int32_t* n_resident, int32_t* n_queue
   if (n_resident) *n_resident = (int32_t)sv->resident.size();
   if (n_queued) *n_queued = (int32_t)sv->queue.size();
   if (n_finished) *n_finished = fin;
-  return GPO_OK;
+  return late;
 }
 
 gpo_status gpo_server_poll(gpo_server* sv, int64_t ticket, int32_t* done, gpo_report* report) {

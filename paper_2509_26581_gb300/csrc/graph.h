@@ -105,7 +105,7 @@ struct gpo_graph {
   gpo::LaunchSet ls{};             // one-problem launch set over `dev`
   bool ex_cluster = false;         // explicit Schur complement: solved by a cluster (else a grid)
   int4 ex_grid{0, 0, 0, 0};        // the solve's launch (problem, CTAs, shared memory)
-  int debug_wait = 0;              // LaunchSet::debug_wait of the graph's solves
+  int debug_wait = 0;              // LaunchSet::debug_wait of the solves from this iteration on (0: never)
   DevBA* dev_desc = nullptr;       // device copy of `dev` (ls.probs)
   Scalars* h_sc = nullptr;         // pinned, read back into
   Scalars* h_up = nullptr;         // pinned, uploaded from
@@ -165,6 +165,11 @@ void plan_resident(const gpo::KernelSet& ks, Prec pr, const std::vector<int2>& p
 // Around the solves of a call: clear their flags; wait, and report a wait that gave up.
 gpo_status begin_solves(gpo_graph* g, const gpo::LaunchSet& ls);
 gpo_status end_solves(gpo_graph* g, const gpo::LaunchSet& ls);
+// The same report without a wait for what is launched in between: the flags behind the solve.
+gpo_status post_flags(gpo_graph* g, const gpo::LaunchSet& ls);
+gpo_status read_flags(gpo_graph* g, const gpo::LaunchSet& ls);
+// Whether the test hook holds the waits of an iteration (counted from 0).
+inline int held(const gpo_graph* g, int iteration) { return g->debug_wait > 0 && iteration + 1 >= g->debug_wait; }
 // Retraction, candidate cost, decision and commit over `ls`.
 gpo_status finish_iteration(gpo_graph* g, const gpo::LaunchSet& ls);
 // Camera render blocks, F(x) and its per-problem reduction over `ls` (no sync).

@@ -673,7 +673,10 @@ __global__ void __launch_bounds__(kExThreads, 1) k_ex_pcg(LaunchSet ls, int prob
   Scalars* sc = d.sc;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (!sc->active || sc->pcg_done) return;   // the same for every CTA of the group
-  if (!kCluster && *reinterpret_cast<volatile int*>(ls.err)) return;   // an earlier solve's wait gave up
+  if (!kCluster && *reinterpret_cast<volatile int*>(ls.err)) {   // an earlier solve's wait gave up
+    if (threadIdx.x == 0) sc->active = 0;                        // no step without a solve
+    return;
+  }
   const int rpc = ex_rows_per_cta(d.C, G), wpr = ex_warps_per_row(rpc), rpp = NW / wpr;
   const int c0 = min(rank * rpc, d.C), nr = min(c0 + rpc, d.C) - c0;
   const int* lcol = d.ex_lcol + d.ex_loff[rank];
@@ -758,7 +761,10 @@ __global__ void __launch_bounds__(kExThreads, 1) k_ex_pcg(LaunchSet ls, int prob
                                       &slot_s[0][0][0], d.ex_red, &fl[3]);
   };
   auto gave_up = [&] {   // leaves the kernel (a cluster's CTAs together: their shared memory is shared)
-    if (tid == 0) atomicExch(ls.err, 1);
+    if (tid == 0) {
+      atomicExch(ls.err, 1);
+      sc->active = 0;   // the rest of the iteration, and the iterations after it, leave the problem alone
+    }
     if constexpr (kCluster) cluster_sync();
   };
   auto receive_z = [&](int o, AT& z) {

@@ -219,7 +219,11 @@ __global__ void __launch_bounds__(kThreads, sizeof(JT) == 2 ? 4 : 3) k_pcg_resid
   unsigned int* const bar = d.sc->bar;
   __syncthreads();
   if (threadIdx.x == 0) coef[2] = sc_inv_n<AT>(&s);
-  if (!s.active || s.pcg_done || *static_cast<volatile int*>(ls.err)) return;
+  if (!s.active || s.pcg_done) return;
+  if (*static_cast<volatile int*>(ls.err)) {   // an earlier wait gave up: no step without a solve
+    if (threadIdx.x == 0) d.sc->active = 0;
+    return;
+  }
   bool ok = true;
 #pragma unroll 1
   for (int it = 0; it < max_launch; ++it) {
@@ -490,7 +494,10 @@ __global__ void __launch_bounds__(kThreads, sizeof(JT) == 2 ? 4 : 3) k_pcg_resid
     if (s.pcg_done) break;
   }
   if (!ok) {
-    if (threadIdx.x == 0) atomicExch(ls.err, 1);
+    if (threadIdx.x == 0) {
+      atomicExch(ls.err, 1);
+      d.sc->active = 0;   // the rest of the iteration, and the iterations after it, leave the problem alone
+    }
     return;
   }
   if (lead) {

@@ -357,9 +357,9 @@ class Graph:
         """gpo_debug_wait_timeout: the status it returns (GPO_ERR_TIMEOUT expected)."""
         return int(lib.gpo_debug_wait_timeout(self.h))
 
-    def debug_hold_waits(self, on: bool) -> None:
+    def debug_hold_waits(self, from_iteration: int) -> None:
         """gpo_debug_hold_waits: makes the bounded waits of this graph's solves give up."""
-        _check(lib.gpo_debug_hold_waits(self.h, int(on)), self.h)
+        _check(lib.gpo_debug_hold_waits(self.h, from_iteration), self.h)
 
     def debug_schur(self, lam: float, n_cams: int, params: gpo_lm_params | None = None, db: int = 9):
         S = np.zeros((n_cams, db, db))

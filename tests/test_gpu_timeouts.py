@@ -39,7 +39,7 @@ def _timeout(gpo, call):
 @pytest.mark.parametrize("kind", list(KINDS))
 def test_a_wait_that_gives_up_is_reported(gpo, kind):
     _, g, _, _ = _build(gpo, kind)
-    g.debug_hold_waits(True)
+    g.debug_hold_waits(1)
     _timeout(gpo, lambda: g.optimize(2))
     _timeout(gpo, lambda: gpo.optimize_batch([g, _build(gpo, kind)[1]], 2))
 
@@ -47,7 +47,7 @@ def test_a_wait_that_gives_up_is_reported(gpo, kind):
 @pytest.mark.parametrize("kind", ["cluster", "matrix_free"])
 def test_a_server_reports_a_wait_that_gives_up(gpo, kind):
     _, g, _, _ = _build(gpo, kind)
-    g.debug_hold_waits(True)
+    g.debug_hold_waits(1)
     sv = gpo.Server(KINDS[kind][1])
     sv.submit(g, 2)
     _timeout(gpo, sv.step)
@@ -60,3 +60,64 @@ def test_the_diagnostic_covers_a_clusters_wait(gpo):
     _, h, d0, _ = _build(gpo, "cluster")
     assert g.optimize(3).final_cost == h.optimize(3).final_cost
     assert np.array_equal(g.get_state(c0, p.n_cams, 9), h.get_state(d0, p.n_cams, 9))
+
+
+def _damped(gpo):
+    """A damping at which the path scenes accept their first steps."""
+    return gpo.default_params(initial_damping=0.1)
+
+
+@pytest.mark.parametrize("kind", list(KINDS))
+def test_a_lost_solve_takes_no_step_and_leaves_no_stale_cost(gpo, kind):
+    """Two iterations, then one whose solve is lost: the graph is where a graph of two
+    iterations is, says so, and goes on from there."""
+    p, g, c0, p0 = _build(gpo, kind)
+    _, h, d0, q0 = _build(gpo, kind)
+    start = g.cost()
+    two = h.optimize(2, _damped(gpo))
+    assert two.accepted == 2
+    g.debug_hold_waits(3)
+    _timeout(gpo, lambda: g.optimize(4, _damped(gpo)))
+    g.debug_hold_waits(0)
+
+    def same():
+        assert np.array_equal(g.get_state(c0, p.n_cams, 9), h.get_state(d0, p.n_cams, 9))
+        assert np.array_equal(g.get_state(p0, p.n_pts, 3), h.get_state(q0, p.n_pts, 3))
+
+    same()
+    assert g.cost() == two.final_cost != start
+    a, b = g.optimize(2, _damped(gpo)), h.optimize(2, _damped(gpo))
+    assert (a.initial_cost, a.final_cost, a.pcg_iters_total) == (b.initial_cost, b.final_cost, b.pcg_iters_total)
+    same()
+
+
+@pytest.mark.parametrize("kind", list(KINDS))
+def test_a_lost_solve_in_a_batch(gpo, kind):
+    p, g, c0, _ = _build(gpo, kind)
+    _, h, d0, _ = _build(gpo, kind)
+    two = h.optimize(2, _damped(gpo))
+    other = _build(gpo, kind)[1]
+    g.debug_hold_waits(3)
+    _timeout(gpo, lambda: gpo.optimize_batch([other, g], 3, _damped(gpo)))
+    for x in (g, other):
+        assert x.cost() == two.final_cost
+        assert np.array_equal(x.get_state(c0, p.n_cams, 9), h.get_state(d0, p.n_cams, 9))
+
+
+@pytest.mark.parametrize("kind", ["cluster", "matrix_free"])
+def test_a_server_makes_a_lost_iteration_again(gpo, kind):
+    p, g, c0, _ = _build(gpo, kind)
+    _, h, d0, _ = _build(gpo, kind)
+    ref = h.optimize(3, _damped(gpo))
+    g.debug_hold_waits(2)
+    sv = gpo.Server(KINDS[kind][1])
+    ticket = sv.submit(g, 3, _damped(gpo))
+    assert sv.step()[0] == 1
+    _timeout(gpo, sv.step)
+    g.debug_hold_waits(0)
+    assert sv.step()[0] == 1 and sv.poll(ticket) is None
+    assert sv.step() == (0, 0, 1)
+    rep = sv.poll(ticket)
+    assert (rep.final_cost, rep.iterations, rep.pcg_iters_total) == (ref.final_cost, 3, ref.pcg_iters_total)
+    assert np.array_equal(g.get_state(c0, p.n_cams, 9), h.get_state(d0, p.n_cams, 9))
+    sv.close()
