@@ -71,50 +71,40 @@ bool sqrt_info(const double* Om, int m, double* U) {
 size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 // Device memory plan: requests are laid out in one arena (256-byte aligned).  Requests
-// with a host source (`up`) come first, so the arena's prefix is one host image that a
-// single copy uploads.
+// with a host source (`up`) come first, whatever the order they are made in, so the arena's
+// prefix is one host image that a single copy uploads.
 struct Plan {
   struct Req { void** ptr; size_t bytes; const void* src; size_t src_bytes; };
-  std::vector<Req> reqs;
+  std::vector<Req> ups, rest;
   template <class T> void add(T** p, size_t count) {
-    reqs.push_back({reinterpret_cast<void**>(p), count * sizeof(T), nullptr, 0});
+    rest.push_back({reinterpret_cast<void**>(p), count * sizeof(T), nullptr, 0});
   }
-  void add_raw(void** p, size_t bytes) { reqs.push_back({p, bytes, nullptr, 0}); }
+  void add_raw(void** p, size_t bytes) { rest.push_back({p, bytes, nullptr, 0}); }
   // an array uploaded from `src` (count elements); the allocation may be larger
   template <class T> void up(T** p, size_t count, const std::vector<T>& src) {
-    reqs.push_back({reinterpret_cast<void**>(p), std::max(count, src.size()) * sizeof(T), src.data(),
-                    src.size() * sizeof(T)});
+    ups.push_back({reinterpret_cast<void**>(p), std::max(count, src.size()) * sizeof(T), src.data(),
+                   src.size() * sizeof(T)});
   }
-  size_t total() const {
+  // calls f(request, offset in the arena) and returns the arena's size
+  template <class F> size_t walk(F&& f) const {
     size_t t = 0;
-    for (auto& r : reqs) t = align_up(t, 256) + align_up(r.bytes, 256);
+    for (auto* list : {&ups, &rest})
+      for (auto& r : *list) {
+        f(r, t);
+        t += align_up(r.bytes, 256);
+      }
     return t;
   }
+  size_t total() const { return walk([](const Req&, size_t) {}); }
   // bytes of the uploaded prefix and its host image
   size_t image(std::vector<char>& out) const {
-    size_t t = 0, end = 0;
-    for (auto& r : reqs) {
-      t = align_up(t, 256);
-      if (r.src) end = t + r.src_bytes;
-      t += align_up(r.bytes, 256);
-    }
+    size_t end = 0;
+    walk([&](const Req& r, size_t t) { if (r.src) end = t + r.src_bytes; });
     out.assign(end, 0);
-    t = 0;
-    for (auto& r : reqs) {
-      t = align_up(t, 256);
-      if (r.src && r.src_bytes) std::memcpy(out.data() + t, r.src, r.src_bytes);
-      t += align_up(r.bytes, 256);
-    }
+    walk([&](const Req& r, size_t t) { if (r.src_bytes) std::memcpy(out.data() + t, r.src, r.src_bytes); });
     return end;
   }
-  void assign(char* base) const {
-    size_t t = 0;
-    for (auto& r : reqs) {
-      t = align_up(t, 256);
-      *r.ptr = base + t;
-      t += align_up(r.bytes, 256);
-    }
-  }
+  void assign(char* base) const { walk([&](const Req& r, size_t t) { *r.ptr = base + t; }); }
 };
 
 constexpr size_t kClusterBytes = 1 << 20;   // see plan_explicit
