@@ -124,8 +124,9 @@ typedef struct {
                                  formed once per damped system and the whole PCG runs in
                                  one launch; it takes device memory for the blocks and
                                  for one row of 3 values per edge and camera coordinate,
-                                 and is left out where the memory budget holds the graph
-                                 only without, a camera sees a point twice, forming the
+                                 and is left out where the memory (the budget, a server's
+                                 budget, the device, the allocator) holds the graph only
+                                 without, a camera sees a point twice, forming the
                                  blocks costs more than it saves, or for bundle
                                  adjustment with BF16 storage, or FP32 and more than
                                  65,536 points; then pipelined for BF16 and FP32

@@ -198,7 +198,8 @@ struct Prepared {
       *xe_kind_d = nullptr, *xo_off_d = nullptr, *xk_off_d = nullptr, *xk_list_d = nullptr, *ch_prob_d = nullptr,
       *cb_prob_d = nullptr, *pb_prob_d = nullptr, *base_d = nullptr, *running_d = nullptr,
       *old2new_d = nullptr;
-  // explicit Schur complement (ex false: not planned)
+  // explicit Schur complement (ex false: not planned), and the memory plan without it
+  Plan plain;
   bool ex = false, ex_cluster = false;
   int ex_nb_max = 0, ex_ctas = 0, ex_res = 0;
   size_t ex_smem = 0;
@@ -214,6 +215,14 @@ struct Prepared {
   DevBA* desc_d = nullptr;
   Plan pl;
 };
+
+// Leaves the explicit Schur complement out of a plan.
+static void leave_matrix_free(Prepared& R) {
+  R.pl = R.plain;
+  R.bytes = R.pl.total();
+  R.ex = false;
+  R.d.ex = 0;
+}
 
 void PrepDeleter::operator()(Prepared* p) const { delete p; }
 
@@ -743,15 +752,14 @@ static gpo_status prepare(gpo_graph* g) {
   R.bytes = pl.total();
   // the explicit Schur complement, unless the memory budget holds the graph only without
   if (explicit_allowed(g, ks, P)) {
-    Plan plain = pl;
-    plan_explicit(g, R, ks, C, P, E, NS);
-    if (R.ex && g->desc.memory_budget && pl.total() > g->desc.memory_budget) R.ex = false;
-    if (R.ex) {
-      R.bytes = pl.total();
-    } else {
-      pl = std::move(plain);
-      d.ex = 0;
+    R.plain = pl;
+    try {
+      plan_explicit(g, R, ks, C, P, E, NS);
+    } catch (const std::bad_alloc&) {   // of host memory: the graph needs none of the tables
+      R.ex = false;
     }
+    R.bytes = pl.total();
+    if (!R.ex || (g->desc.memory_budget && R.bytes > g->desc.memory_budget)) leave_matrix_free(R);
   }
   g->prep.reset(pp.release());
   return GPO_OK;
@@ -771,26 +779,31 @@ gpo_status gpo_host::finalize(gpo_graph* g, size_t* plan_bytes) {
     if (s != GPO_OK) return s;
   }
   Prepared& R = *g->prep;
-  const size_t bytes = R.bytes;
   if (plan_bytes) {
-    *plan_bytes = bytes;
+    *plan_bytes = R.bytes;
     return GPO_OK;
   }
   if (gpo_status s = ensure_stream(g); s != GPO_OK) return s;
-  if (g->desc.memory_budget && bytes > g->desc.memory_budget)
-    return fail(g, GPO_ERR_OOM, "graph needs %zu bytes of device memory, budget is %zu", bytes,
+  if (g->desc.memory_budget && R.bytes > g->desc.memory_budget)
+    return fail(g, GPO_ERR_OOM, "graph needs %zu bytes of device memory, budget is %zu", R.bytes,
                 (size_t)g->desc.memory_budget);
   void* base = nullptr;
-  if (g->desc.alloc && g->desc.free) {
-    base = g->desc.alloc(bytes, g->desc.alloc_ctx);
-    if (!base) return fail(g, GPO_ERR_OOM, "allocator hook returned NULL for %zu bytes", bytes);
-  } else {
-    const cudaError_t e = cudaMalloc(&base, bytes);
-    if (e != cudaSuccess) {
+  for (;;) {   // where the memory does not hold the explicit Schur complement, without it
+    cudaError_t e = cudaSuccess;
+    if (g->desc.alloc && g->desc.free) base = g->desc.alloc(R.bytes, g->desc.alloc_ctx);
+    else if ((e = cudaMalloc(&base, R.bytes)) != cudaSuccess) {
       cudaGetLastError();
-      return fail(g, GPO_ERR_OOM, "cudaMalloc(%zu) failed: %s", bytes, cudaGetErrorString(e));
+      base = nullptr;
     }
+    if (base) break;
+    if (R.ex) {
+      leave_matrix_free(R);
+      continue;
+    }
+    if (e != cudaSuccess) return fail(g, GPO_ERR_OOM, "cudaMalloc(%zu) failed: %s", R.bytes, cudaGetErrorString(e));
+    return fail(g, GPO_ERR_OOM, "allocator hook returned NULL for %zu bytes", R.bytes);
   }
+  const size_t bytes = R.bytes;
   g->arena = base;
   g->arena_bytes = bytes;
   R.pl.assign(static_cast<char*>(base));
@@ -869,6 +882,17 @@ gpo_status gpo_host::finalize(gpo_graph* g, size_t* plan_bytes) {
   g->prep.reset();
   g->state_same = false;
   GPO_CUDA(g, cudaGetLastError());
+  return GPO_OK;
+}
+
+// Plans the graph for at most `budget` bytes where the explicit Schur complement is what
+// makes it larger.
+gpo_status gpo_host::plan_within(gpo_graph* g, size_t budget, size_t* plan_bytes) {
+  if (gpo_status s = finalize(g, plan_bytes); s != GPO_OK) return s;
+  if (g->prep && g->prep->ex && *plan_bytes > budget) {
+    leave_matrix_free(*g->prep);
+    *plan_bytes = g->prep->bytes;
+  }
   return GPO_OK;
 }
 

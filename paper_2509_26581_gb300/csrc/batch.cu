@@ -6,6 +6,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstdint>
 #include <cstring>
 #include <deque>
 #include <map>
@@ -412,7 +413,7 @@ gpo_status gpo_server_submit(gpo_server* sv, gpo_graph* g, int32_t max_iters, co
   if (sv->owner->ks && sv->owner->ks != k)
     return fail(sv->owner, GPO_ERR_ARG, "graph camera kind differs from the server's earlier graphs");
   size_t bytes = 0;
-  gpo_status s = finalize(g, &bytes);
+  gpo_status s = plan_within(g, sv->desc.memory_budget ? sv->desc.memory_budget : SIZE_MAX, &bytes);
   if (s != GPO_OK) {
     sv->owner->err = g->err;
     return s;

@@ -151,6 +151,7 @@ inline const gpo::KernelSet& kernels_of(const gpo_graph* g) {
 
 gpo_status fail(gpo_graph* g, gpo_status st, const char* fmt, ...);
 gpo_status finalize(gpo_graph* g, size_t* plan_bytes = nullptr);
+gpo_status plan_within(gpo_graph* g, size_t budget, size_t* plan_bytes);
 void release_device(gpo_graph* g);
 void fill_scalars(gpo_graph* g, const gpo_lm_params& p, double lambda, Scalars& s);
 gpo_status upload_scalars(gpo_graph* g, const Scalars& s);

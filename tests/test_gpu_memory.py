@@ -1,5 +1,6 @@
-"""Graphs on a caller's allocator: what finalizing a graph writes, and that nothing relies on
-what the memory held before."""
+"""Graphs on a caller's allocator, and memory that holds a graph only without the explicit
+Schur complement: what finalizing writes, that nothing relies on what the memory held before,
+and that such a graph is solved matrix-free rather than refused."""
 import ctypes
 
 import numpy as np
@@ -76,3 +77,58 @@ def test_only_the_uploaded_arrays_are_written(gpo, prec, kernel):
     assert np.array_equal(g.get_state(p0, p.n_pts, 3), h.get_state(q0, p.n_pts, 3))
     g.close()
     assert not arenas.blocks
+
+
+def _sizes(gpo, p, prec):
+    """Planned bytes with the explicit Schur complement, and where a budget leaves it out."""
+    out = []
+    for budget in (0, -1):
+        g = gpo.ba_graph(p.cams0, p.pts0, p.cam_idx, p.pt_idx, p.obs, p.huber_delta, prec, spmv_variant=0,
+                         chunk_edges=512, memory_budget=out[0] + budget if budget else 0)[0]
+        out.append(g.plan())
+        g.close()
+    assert out[0] > 1.1 * out[1]
+    return out
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_an_allocator_that_holds_the_graph_only_without_the_blocks(gpo, prec):
+    p = synth.ba_path(3, 121, 9000, "pareto")
+    full, plain = _sizes(gpo, p, prec)
+    arenas = Arenas(gpo, limit=(full + plain) // 2)
+    g, c0, _ = arenas.graph(gpo, p, prec)
+    rep = g.optimize(2)
+    assert arenas.asked == [full, plain] and g.footprint() == plain and g.info()["spmv_kernel"] != 7
+    h, d0, _ = gpo.ba_graph(p.cams0, p.pts0, p.cam_idx, p.pt_idx, p.obs, p.huber_delta, prec, spmv_variant=0,
+                            chunk_edges=512, memory_budget=(full + plain) // 2)
+    assert rep.final_cost == h.optimize(2).final_cost
+    assert np.array_equal(g.get_state(c0, p.n_cams, 9), h.get_state(d0, p.n_cams, 9))
+    none = Arenas(gpo, limit=plain - 1)
+    with pytest.raises(gpo.GpoError) as e:
+        none.graph(gpo, p, prec)[0].optimize(1)
+    assert e.value.status == gpo.GPO_ERR_OOM and none.asked == [full, plain]
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_a_server_budget_that_holds_the_graph_only_without_the_blocks(gpo, prec):
+    p = synth.ba_path(3, 121, 9000, "pareto")
+    full, plain = _sizes(gpo, p, prec)
+
+    def graph(**kw):
+        return gpo.ba_graph(p.cams0, p.pts0, p.cam_idx, p.pt_idx, p.obs, p.huber_delta, prec, spmv_variant=0,
+                            chunk_edges=512, **kw)
+
+    h, d0, _ = graph(memory_budget=plain)
+    ref = h.optimize(2)
+    g, c0, _ = graph()
+    sv = gpo.Server(prec, memory_budget=plain)
+    ticket = sv.submit(g, 2)
+    while sum(sv.step()[:2]):
+        assert sv.memory() == plain
+    rep = sv.poll(ticket)
+    assert (rep.final_cost, rep.pcg_iters_total) == (ref.final_cost, ref.pcg_iters_total)
+    assert np.array_equal(g.get_state(c0, p.n_cams, 9), h.get_state(d0, p.n_cams, 9))
+    with pytest.raises(gpo.GpoError) as e:
+        gpo.Server(prec, memory_budget=plain - 1).submit(graph()[0], 2)
+    assert e.value.status == gpo.GPO_ERR_OOM
+    sv.close()
