@@ -127,7 +127,9 @@ typedef struct {
                                  and is left out where the memory (the budget, a server's
                                  budget, the device, the allocator) holds the graph only
                                  without, a camera sees a point twice, forming the
-                                 blocks costs more than it saves, or for bundle
+                                 blocks costs more than it saves (in a call whose
+                                 pcg_max_iters or loose relative pcg_tol leaves its
+                                 solves few iterations too), or for bundle
                                  adjustment with BF16 storage, or FP32 and more than
                                  65,536 points; then pipelined for BF16 and FP32
                                  storage, the whole PCG in one launch with the same
@@ -367,7 +369,8 @@ typedef struct {
   int32_t spmv_variant;       /* as requested in gpo_graph_desc */
   int32_t spmv_kernel;        /* the Schur-product kernel the PCG runs, in spmv_variant's
                                  numbering (1 staged, 2 classic, 3 pipelined, 4 dynamic,
-                                 5 warp groups, 7 explicit; 0: no observation edges) */
+                                 5 warp groups, 7 explicit, where a call's solves have
+                                 the iterations to pay for it; 0: no observation edges) */
   int32_t reserved0;
   int64_t j_bytes;            /* device bytes of the stored Jacobian rows (0 with dynamic
                                  Jacobians, which store none) */

@@ -203,6 +203,7 @@ struct Prepared {
   bool ex = false, ex_cluster = false;
   int ex_nb_max = 0, ex_ctas = 0, ex_res = 0;
   size_t ex_smem = 0;
+  double ex_min_it = 0.0;
   std::vector<int32_t> ex_loff, ex_lcol, ex_lidx, ex_lown, ex_xl;
   int *ex_loff_d = nullptr, *ex_lcol_d = nullptr, *ex_lidx_d = nullptr, *ex_lown_d = nullptr, *ex_xl_d = nullptr;
   std::vector<int32_t> ex_row, ex_col, ex_uoff, ex_ublk, ex_crow, ex_slot_y0, ex_doff, ex_dcam, zeros_xf, zeros_xd;
@@ -310,6 +311,12 @@ static void plan_explicit(gpo_graph* g, Prepared& R, const gpo::KernelSet& ks, i
   }
   const size_t NB = R.ex_col.size();
   if (R.ex_nb_max > 5000 || !pays(NB)) return;
+  // The iterations per solve from which the blocks pay (explicit_pays), by the same times; in
+  // FP64 with what an edge costs in the camera rows and diagonals (0.5 ns) and the stereo
+  // model's smaller blocks.  Against the measured crossings: 300 cameras 14.3 (12.4), 150
+  // cameras 9.8 (10.2), 60 cameras of 12-view points 11.2 (8.2), 40 cameras 5.0 (5.6), 200
+  // keyframes 5.7 (3.9), all FP64; 1,000 keyframes BF16 3.3 (4.5), 200 cameras FP32 2.2 (1.0).
+  R.ex_min_it = std::min(15.5, (f64 ? form * EL / 81 + 5e-10 * E : form) / (free_it - (double)NB * EL * sA / 6e12 - 6e-6));
   const int NBU = R.ex_uoff[C];
   R.ex_ublk.resize(2 * (size_t)NBU);
   {
@@ -857,6 +864,7 @@ gpo_status gpo_host::finalize(gpo_graph* g, size_t* plan_bytes) {
     ls.n_xf = d.ex_nbu > 0 ? d.ex_nxf : 0;
     ls.n_xd = (int)R.zeros_xd.size();
     g->ex_cluster = R.ex_cluster;
+    g->ex_min_it = R.ex_min_it;
     g->ex_grid = make_int4(0, R.ex_ctas, (int)R.ex_smem, R.ex_res);
     ls.xg_host = &g->ex_grid;
     (R.ex_cluster ? ls.n_cl : ls.n_xg) = 1;
@@ -1155,6 +1163,23 @@ static gpo_status ensure_full(gpo_graph* g) {
   GPO_CUDA(g, cudaMemcpyAsync(g->dev_desc, &g->dev, sizeof(DevBA), cudaMemcpyHostToDevice, g->stream));
   GPO_CUDA(g, cudaStreamSynchronize(g->stream));   // the host copy of the descriptor stays valid
   return GPO_OK;
+}
+
+// Whether a call's solves take the explicit Schur complement of a graph that has one planned.
+// The plan takes a solve to have 16 iterations; a cap or a loose relative tolerance leaves
+// fewer, and then forming the blocks may cost more than the products (300 cameras FP64, two
+// LM iterations: 5 iterations each 4,475 us matrix-free, 6,756 explicit; 16 each 8,145 and
+// 6,970).  Iterations are taken in proportion to the tolerance's digits, 16 at 1e-6, with
+// an inertial chain 80 (10 to 25 and 83 to 87 measured at a light damping).  The rule reads
+// the parameters that stay the same along a run and not the damping, so that a batch, a
+// server and a run continued call by call solve as one call does; solves under a heavy
+// damping, which have few iterations too, form the blocks all the same (damping 10 there:
+// 4,379 us matrix-free, 6,669 explicit).
+bool gpo_host::explicit_pays(const gpo_graph* g, const gpo_lm_params& p) {
+  double n = std::max(1, p.pcg_max_iters);
+  const double per_digit = (g->dev.NX > 0 ? 80.0 : 16.0) / 6.0;
+  if (p.pcg_tol_relative && p.pcg_tol > 0.0) n = std::min(n, std::max(1.0, per_digit * -std::log10(p.pcg_tol)));
+  return g->ls.ex && n >= g->ex_min_it;
 }
 
 // Plans the resident PCG of a launch set: the fewest chunks per CTA at which the CTAs fit the
@@ -1794,14 +1819,17 @@ gpo_status gpo_optimize(gpo_graph* g, int32_t max_iters, const gpo_lm_params* pa
   // the iterations follow without a look at the cost: one that is not finite switches them
   // off on the device
   if (!cont && (s = launch_initial_cost(g, g->ls)) != GPO_OK) return s;
-  if ((s = begin_solves(g, g->ls)) != GPO_OK) return s;
+  gpo::LaunchSet ls = g->ls;
+  if (ls.ex && !explicit_pays(g, prm)) {
+    ls.ex = ls.n_cl = ls.n_xg = 0;
+    ls.mf = 1;
+  }
+  if ((s = begin_solves(g, ls)) != GPO_OK) return s;
   for (int it = 0; it < max_iters; ++it) {
     g->cur_lm_iter = it;
-    g->ls.debug_wait = held(g, it);
-    s = solve_system(g, g->ls, sc.max_it, false);
-    g->ls.debug_wait = 0;
-    if (s != GPO_OK) return s;
-    if ((s = finish_iteration(g, g->ls)) != GPO_OK) return s;
+    ls.debug_wait = held(g, it);
+    if ((s = solve_system(g, ls, sc.max_it, false)) != GPO_OK) return s;
+    if ((s = finish_iteration(g, ls)) != GPO_OK) return s;
   }
   g->cur_lm_iter = -1;
   GPO_CUDA(g, cudaMemcpyAsync(g->h_sc, g->dev.sc, sizeof(Scalars), cudaMemcpyDeviceToHost, g->stream));
@@ -1810,7 +1838,7 @@ gpo_status gpo_optimize(gpo_graph* g, int32_t max_iters, const gpo_lm_params* pa
   if (nh)
     GPO_CUDA(g, cudaMemcpyAsync(hist.data(), g->dev.hist, nh * sizeof(gpo::IterRecord),
                                 cudaMemcpyDeviceToHost, g->stream));
-  if ((s = end_solves(g, g->ls)) != GPO_OK) return s;
+  if ((s = end_solves(g, ls)) != GPO_OK) return s;
   const double F0 = cont ? last_cost : g->h_sc->cost0;
   if (!std::isfinite(F0)) return fail(g, GPO_ERR_NUMERIC, "initial cost is not finite (%g)", F0);
   g->hist = std::move(hist);

@@ -45,7 +45,8 @@ struct BatchSet {
   }
 };
 
-gpo_status build_set(gpo_graph* owner, const std::vector<gpo_graph*>& gs, BatchSet& out) {
+// ex_of[q]: problem q solves on its explicit Schur complement (empty: only costs are computed).
+gpo_status build_set(gpo_graph* owner, const std::vector<gpo_graph*>& gs, const std::vector<char>& ex_of, BatchSet& out) {
   const int n = (int)gs.size();
   std::vector<DevBA> probs(n);
   std::vector<int> ch_prob, cb_prob, pb_prob, ch_base(n), cb_base(n), pb_base(n);
@@ -55,6 +56,7 @@ gpo_status build_set(gpo_graph* owner, const std::vector<gpo_graph*>& gs, BatchS
   for (int q = 0; q < n; ++q) {
     const gpo_graph* g = gs[q];
     probs[q] = g->dev;
+    probs[q].ex = !ex_of.empty() && ex_of[q];
     ch_base[q] = (int)ch_prob.size();
     cb_base[q] = (int)cb_prob.size();
     pb_base[q] = (int)pb_prob.size();
@@ -66,7 +68,7 @@ gpo_status build_set(gpo_graph* owner, const std::vector<gpo_graph*>& gs, BatchS
     np_max = std::max(np_max, g->ls.np_max);
     xf_base[q] = (int)xf_prob.size();
     xd_base[q] = (int)xd_prob.size();
-    if (!g->ls.ex) {
+    if (!probs[q].ex) {
       mf = 1;
       continue;
     }
@@ -139,7 +141,7 @@ gpo_status build_set(gpo_graph* owner, const std::vector<gpo_graph*>& gs, BatchS
   ls.cl_smem = cl_smem;
   std::vector<int2> sizes;
   for (const gpo_graph* g : gs) sizes.push_back(make_int2(g->ls.n_ch, g->ls.n_cb));
-  if (mf && !cb_prob.empty()) plan_resident(*gs[0]->ks, owner->prec, sizes, ls);
+  if (mf && !ex_of.empty() && !cb_prob.empty()) plan_resident(*gs[0]->ks, owner->prec, sizes, ls);
   out.ls = ls;
   out.mem = mem;
   out.staging = stage_d;
@@ -295,7 +297,9 @@ gpo_status gpo_optimize_batch(gpo_graph* const* graphs, int32_t n, int32_t max_i
   std::vector<gpo_graph*> gs(graphs, graphs + n);
   BatchSet bs;
   gpo_status s = join_uploads(owner, gs);
-  if (s == GPO_OK) s = build_set(owner, gs, bs);
+  std::vector<char> ex;
+  for (const gpo_graph* g : gs) ex.push_back(explicit_pays(g, prm));
+  if (s == GPO_OK) s = build_set(owner, gs, ex, bs);
   if (s != GPO_OK) return s;
   std::vector<Scalars> sc(n);
   for (int i = 0; i < n; ++i) {
@@ -466,7 +470,7 @@ gpo_status gpo_server_step(gpo_server* sv, int32_t* n_resident, int32_t* n_queue
     for (auto& r : adm) gs.push_back(r.g);
     BatchSet bs;
     gpo_status s = join_uploads(owner, gs);
-    if (s == GPO_OK) s = build_set(owner, gs, bs);
+    if (s == GPO_OK) s = build_set(owner, gs, {}, bs);
     if (s != GPO_OK) return s;
     std::vector<Scalars> sc(adm.size());
     for (size_t i = 0; i < adm.size(); ++i) {
@@ -496,8 +500,12 @@ gpo_status gpo_server_step(gpo_server* sv, int32_t* n_resident, int32_t* n_queue
     if (sv->dirty) {
       sv->set.release(owner->stream);
       std::vector<gpo_graph*> gs;
-      for (auto& r : sv->resident) gs.push_back(r.g);
-      gpo_status s = build_set(owner, gs, sv->set);
+      std::vector<char> ex;
+      for (auto& r : sv->resident) {
+        gs.push_back(r.g);
+        ex.push_back(explicit_pays(r.g, r.prm));
+      }
+      gpo_status s = build_set(owner, gs, ex, sv->set);
       if (s != GPO_OK) return s;
       sv->dirty = false;
     }

@@ -103,6 +103,7 @@ struct gpo_graph {
   size_t full_bytes = 0;
   DevBA dev{};
   gpo::LaunchSet ls{};             // one-problem launch set over `dev`
+  double ex_min_it = 0.0;          // iterations per solve from which the explicit Schur complement pays
   bool ex_cluster = false;         // explicit Schur complement: solved by a cluster (else a grid)
   int4 ex_grid{0, 0, 0, 0};        // the solve's launch (problem, CTAs, shared memory)
   int debug_wait = 0;              // LaunchSet::debug_wait of the solves from this iteration on (0: never)
@@ -161,6 +162,8 @@ gpo_lm_params params_or_default(const gpo_lm_params* p);
 gpo_status solve_system(gpo_graph* g, const gpo::LaunchSet& ls, int max_it, bool force_lin);
 // Orders owner's stream after the uploads that are still running on the graphs' own streams.
 gpo_status join_uploads(gpo_graph* owner, const std::vector<gpo_graph*>& graphs);
+// Whether solves with these parameters take the graph's explicit Schur complement.
+bool explicit_pays(const gpo_graph* g, const gpo_lm_params& p);
 // Plans the one-launch matrix-free PCG of a launch set (probs: chunks and camera blocks).
 void plan_resident(const gpo::KernelSet& ks, Prec pr, const std::vector<int2>& probs, gpo::LaunchSet& ls);
 // Around the solves of a call: clear their flags; wait, and report a wait that gave up.

@@ -1,0 +1,101 @@
+"""Calls whose solves have few iterations (a low cap, a loose tolerance) on graphs that have the
+explicit Schur complement planned: matrix-free where forming the blocks would cost more than it
+saves, alone, in a batch and in a server alike (bit for bit), explicit where it still pays."""
+import numpy as np
+import pytest
+
+from paper_2509_26581_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def gpo():
+    from paper_2509_26581_gb300 import gpo as m
+    return m
+
+
+# forming pays at about 10 iterations of the first scene, from the first one of the second
+SCENES = {"path": lambda: synth.ba_path(1, 150, 40_000, "geom"), "ring": lambda: synth.ba_ring(2, 10, 500, 6)}
+
+
+def _build(gpo, name, variant=0):
+    p = SCENES[name]()
+    return (p,) + gpo.ba_graph(p.cams0, p.pts0, p.cam_idx, p.pt_idx, p.obs, p.huber_delta, "fp64", spmv_variant=variant,
+                               chunk_edges=512)
+
+
+def _forms(g):
+    return g.profile()["schur_form"]["launches"] > 0
+
+
+@pytest.mark.parametrize("name,kw,explicit", [
+    ("path", dict(), True), ("path", dict(pcg_max_iters=3), False), ("path", dict(pcg_tol=0.1), False),
+    ("path", dict(pcg_tol=0.1, pcg_tol_relative=0), True), ("path", dict(pcg_max_iters=16, pcg_tol=0.0), True),
+    ("path", dict(pcg_tol=10.0), False), ("ring", dict(pcg_max_iters=1), True), ("ring", dict(pcg_tol=0.1), True)])
+def test_the_product_follows_the_calls_iterations(gpo, name, kw, explicit):
+    params = gpo.default_params(initial_damping=0.1, **kw)
+    p, g, c0, p0 = _build(gpo, name)
+    rep = g.optimize(2, params)
+    assert g.info()["spmv_kernel"] == 7 and _forms(g) == explicit
+    # the classic product on the same graph: rounding apart (as for other orders of summation)
+    _, h, d0, _ = _build(gpo, name, 2)
+    ref = h.optimize(2, params)
+    assert (rep.pcg_iters_total, rep.accepted) == (ref.pcg_iters_total, ref.accepted)
+    cams = g.get_state(c0, p.n_cams, 9)
+    assert np.max(np.abs(cams - h.get_state(d0, p.n_cams, 9))) <= 1e-8 * np.max(np.abs(cams))
+    # the next call decides anew
+    g.optimize(1, gpo.default_params(initial_damping=0.1))
+    assert _forms(g)
+
+
+@pytest.mark.parametrize("kw", [dict(), dict(pcg_max_iters=3), dict(pcg_tol=0.1)], ids=["full", "cap", "loose"])
+def test_batch_server_and_single_iterations_solve_like_one_call(gpo, kw):
+    params = gpo.default_params(initial_damping=0.1, **kw)
+    alone, graphs = [], []
+    for name in SCENES:
+        p, g, c0, p0 = _build(gpo, name)
+        rep = g.optimize(3, params)
+        alone.append((rep.final_cost, rep.pcg_iters_total, g.get_state(c0, p.n_cams, 9), g.get_state(p0, p.n_pts, 3)))
+        graphs.append((p, c0, p0))
+
+    def same(built, reps):
+        for a, (p, c0, p0), g, r in zip(alone, graphs, built, reps):
+            assert (r.final_cost, r.pcg_iters_total) == a[:2]
+            assert np.array_equal(g.get_state(c0, p.n_cams, 9), a[2]) and np.array_equal(g.get_state(p0, p.n_pts, 3), a[3])
+
+    built = [_build(gpo, name)[1] for name in SCENES]
+    same(built, gpo.optimize_batch(built, 3, params))
+    built = [_build(gpo, name)[1] for name in SCENES]
+    sv = gpo.Server("fp64")
+    tickets = [sv.submit(g, 3, params) for g in built]
+    while sum(sv.step()[:2]):
+        pass
+    same(built, [sv.poll(t) for t in tickets])
+    sv.close()
+    for a, (p, c0, p0), name in zip(alone, graphs, SCENES):
+        g = _build(gpo, name)[1]
+        step = gpo.default_params(initial_damping=0.1, **kw)
+        for _ in range(3):
+            r = g.optimize(1, step)
+            step.initial_damping, step.initial_nu = r.final_lambda, r.final_nu
+        assert r.final_cost == a[0] and np.array_equal(g.get_state(c0, p.n_cams, 9), a[2])
+
+
+def test_a_server_of_requests_with_different_caps(gpo):
+    """Each request's own parameters decide, whatever the others of the step ask for."""
+    caps = [100, 3, 100, 3]
+    want = []
+    for cap in caps:
+        p, g, c0, _ = _build(gpo, "path")
+        g.optimize(2, gpo.default_params(initial_damping=0.1, pcg_max_iters=cap))
+        want.append(g.get_state(c0, p.n_cams, 9))
+    sv = gpo.Server("fp64")
+    built = [_build(gpo, "path")[1] for _ in caps]
+    for g, cap in zip(built, caps):
+        sv.submit(g, 2, gpo.default_params(initial_damping=0.1, pcg_max_iters=cap))
+    while sum(sv.step()[:2]):
+        pass
+    for g, w in zip(built, want):
+        assert np.array_equal(g.get_state(c0, w.shape[0], 9), w)
+    sv.close()
