@@ -273,17 +273,33 @@ static void plan_explicit(gpo_graph* g, Prepared& R, const gpo::KernelSet& ks, i
   const int W = (C + 63) / 64;
   std::vector<uint64_t> bits((size_t)C * W, 0);
   std::vector<int32_t> seen(C, -1);
-  std::vector<std::pair<int, uint64_t>> words;
+  std::vector<std::pair<int, uint64_t>> words, before;
   for (int p = 0; p < P; ++p) {
     const int a = R.pt_off[p], b = R.pt_off[p + 1];
+    words.swap(before);
     words.clear();
-    for (int e = a; e < b; ++e) {
-      const int c = R.e_cam_s[e], w = c >> 6;
-      if (seen[c] == p) return;   // the camera sees the point twice
-      seen[c] = p;
-      if (words.empty() || words.back().first != w) words.push_back({w, 0});
-      words.back().second |= (uint64_t)1 << (c & 63);
+    bool ascending = true;
+    int w = -1;
+    uint64_t m = 0;
+    for (int e = a, prev = -1; e < b; ++e) {
+      const int c = R.e_cam_s[e];
+      ascending &= c > prev;
+      prev = c;
+      if (c >> 6 != w) {
+        if (w >= 0) words.push_back({w, m});
+        w = c >> 6;
+        m = 0;
+      }
+      m |= (uint64_t)1 << (c & 63);
     }
+    if (w >= 0) words.push_back({w, m});
+    if (!ascending)
+      for (int e = a; e < b; ++e) {
+        const int c = R.e_cam_s[e];
+        if (seen[c] == p) return;   // the camera sees the point twice
+        seen[c] = p;
+      }
+    if (ascending && words == before) continue;   // the same cameras as the point before
     for (int e = a; e < b; ++e) {
       uint64_t* row = &bits[(size_t)R.e_cam_s[e] * W];
       for (const auto& x : words) row[x.first] |= x.second;
@@ -459,30 +475,44 @@ static gpo_status prepare(gpo_graph* g) {
   // complement may be used, ties go by the largest camera index first: points with the same
   // span of cameras are then adjacent, which makes the rows that a pair of cameras shares
   // (k_ex_form) runs of consecutive ones.
-  std::vector<int32_t> key(P, C), last(P, 0);
-  std::vector<int32_t> deg(P, 0);
-  for (int64_t e = 0; e < Eall; ++e)
-    if (g->e_active[e]) {
-      const int p = g->e_pt[e];
-      key[p] = std::min(key[p], g->e_cam[e]);
-      last[p] = std::max(last[p], g->e_cam[e]);
-      deg[p]++;
+  const bool spans = explicit_allowed(g, ks, P);
+  std::vector<int32_t> key(P, C), deg(P, 0), last(spans ? P : 0);
+  if (spans) {
+    struct Track { int32_t first, last, deg; };   // together: the edges visit points in any order
+    std::vector<Track> track(P, Track{C, 0, 0});
+    for (int64_t e = 0; e < Eall; ++e)
+      if (g->e_active[e]) {
+        Track& t = track[g->e_pt[e]];
+        t.first = std::min(t.first, g->e_cam[e]);
+        t.last = std::max(t.last, g->e_cam[e]);
+        t.deg++;
+      }
+    for (int p = 0; p < P; ++p) {
+      key[p] = track[p].first;
+      last[p] = track[p].last;
+      deg[p] = track[p].deg;
     }
-  std::vector<int32_t> cnt(C + 2, 0), by_last(P);
-  if (explicit_allowed(g, ks, P)) {
+  } else {
+    for (int64_t e = 0; e < Eall; ++e)
+      if (g->e_active[e]) {
+        const int p = g->e_pt[e];
+        key[p] = std::min(key[p], g->e_cam[e]);
+        deg[p]++;
+      }
+  }
+  std::vector<int32_t> cnt(C + 2, 0), by_last(spans ? P : 0);
+  if (spans) {
     for (int p = 0; p < P; ++p) cnt[last[p] + 1]++;
     for (int k = 0; k <= C; ++k) cnt[k + 1] += cnt[k];
     for (int p = 0; p < P; ++p) by_last[cnt[last[p]]++] = p;
     std::fill(cnt.begin(), cnt.end(), 0);
-  } else {
-    for (int p = 0; p < P; ++p) by_last[p] = p;
   }
   for (int p = 0; p < P; ++p) cnt[key[p] + 1]++;
   for (int k = 0; k <= C; ++k) cnt[k + 1] += cnt[k];
   R.pt_new2old.assign(P, 0);
   R.pt_old2new.assign(P, 0);
   for (int q = 0; q < P; ++q) {
-    const int p = by_last[q];
+    const int p = spans ? by_last[q] : q;
     const int np = cnt[key[p]]++;
     R.pt_new2old[np] = p;
     R.pt_old2new[p] = np;
@@ -625,10 +655,20 @@ static gpo_status prepare(gpo_graph* g) {
   // per-edge data in sorted order
   R.obs_s.resize((size_t)M * E);
   R.delta_s.resize(E);
-  for (int i = 0; i < E; ++i) {
-    const int64_t e = R.sorted_edge[i];
-    for (int k = 0; k < M; ++k) R.obs_s[(size_t)M * i + k] = g->e_obs[(size_t)M * e + k];
-    R.delta_s[i] = g->e_delta[e];
+  // in the order of spans, edges that follow one another lie far apart in the caller's order:
+  // the next ones' values are asked for ahead
+  const int block = spans ? 32 : std::max(E, 1);
+  for (int i0 = 0; i0 < E; i0 += block) {
+    const int i1 = std::min(i0 + block, E);
+    for (int i = i1; i < std::min(i1 + 32, E); ++i) {
+      __builtin_prefetch(&g->e_obs[(size_t)M * R.sorted_edge[i]]);
+      __builtin_prefetch(&g->e_delta[R.sorted_edge[i]]);
+    }
+    for (int i = i0; i < i1; ++i) {
+      const int64_t e = R.sorted_edge[i];
+      for (int k = 0; k < M; ++k) R.obs_s[(size_t)M * i + k] = g->e_obs[(size_t)M * e + k];
+      R.delta_s[i] = g->e_delta[e];
+    }
   }
   if (g->any_info) {
     R.info_s.resize((size_t)NQ * E);
