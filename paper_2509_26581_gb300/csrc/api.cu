@@ -1100,6 +1100,10 @@ static void capture_pcg_group(gpo_graph* g, const gpo::LaunchSet& ls) {
 // The resident PCG (profiling times the launches of an iteration apart).
 static bool resident(const gpo_graph* g, const gpo::LaunchSet& ls) { return ls.res_m > 0 && !g->pcg_full && !g->prof.on; }
 
+// Products of a solve at most: restart iterations (at most one per four PCG iterations) come
+// on top of max_it; the device stops at max_it counted PCG iterations.
+static int max_products(int max_it) { return (int)std::min<int64_t>((int64_t)max_it + max_it / 4 + 1, INT32_MAX); }
+
 // PCG iterations with early exit: iterations are launched in groups; after each
 // group the done flag is copied back, and the flag of the previous group decides
 // whether to launch more (one group of look-ahead keeps the GPU busy).  Full groups
@@ -1108,14 +1112,12 @@ static gpo_status pcg_solve(gpo_graph* g, const gpo::LaunchSet& ls, int max_it) 
   if (gpo_status s = gpo_host::ensure_runtime(g); s != GPO_OK) return s;
   if (resident(g, ls)) {
     int n = 0;
-    run(g, KK_EX_PCG, [&] { n = g->ks->pcg_resident(ls, g->prec, max_it + max_it / 4 + 1, g->stream); return std::max(n, 0); });
+    run(g, KK_EX_PCG, [&] { n = g->ks->pcg_resident(ls, g->prec, max_products(max_it), g->stream); return std::max(n, 0); });
     return n < 0 ? fail(g, GPO_ERR_CUDA, "the launch of the PCG solve was refused") : GPO_OK;
   }
   const int kGroup = kPcgGroup;
   int launched = 0, slot = 0, pending = -1;
-  // restart iterations (at most one per four PCG iterations) are launched on top of
-  // max_it; the device stops at max_it counted PCG iterations
-  const int max_launch = max_it + max_it / 4 + 1;
+  const int max_launch = max_products(max_it);
   while (launched < max_launch) {
     const int n = std::min(kGroup, max_launch - launched);
     const bool graph_ok = !g->prof.on && !g->pcg_graph_off && n == kGroup;
