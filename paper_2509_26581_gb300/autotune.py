@@ -15,7 +15,8 @@ The best choice depends on the problem's size (how many chunks fill the GPU, how
 slots a chunk has) and on the storage precision.  `tune` times every candidate on a
 representative problem of a size class -- a few LM iterations after a warm-up, wall
 clock around `gpo_optimize` with the device synchronised on both sides -- and keeps the
-fastest.  The winners form a table keyed by device name, model, precision and size
+fastest (`pick`); a class tuned before keeps its chunk size unless `--rechunk` is given.
+The winners form a table keyed by device name, model, precision and size
 class (`tuning.json` beside this file, written by `python -m
 paper_2509_26581_gb300.autotune --write` on the target GPU); `choose` looks a graph's
 knobs up in it, and `gpo.ba_graph` / `gpo.vi_graph` apply it when no knob is given.
@@ -81,9 +82,17 @@ def choose(n_edges: int, precision: str, model: str = "ba", table: dict | None =
     return dict(entry["best"]) if entry else dict(DEFAULT)
 
 
-def tune(build, candidates=CANDIDATES + AUTOMATIC, iters: int = 3, warmup: int = 1, repeats: int = 2) -> dict:
+def pick(timings: list, chunk: int | None = None) -> dict:
+    """The knobs to use: the fastest, but the library's own choice (variant 0) unless a fixed
+    product is faster by more than 1 %; of the given chunk size only, if one is given."""
+    of = [t for t in timings if chunk is None or t["knobs"]["chunk_edges"] == chunk]
+    return dict(min(of, key=lambda t: t["s_per_iter"] * (1.0 if t["knobs"]["spmv_variant"] == 0 else 1.01))["knobs"])
+
+
+def tune(build, candidates=CANDIDATES + AUTOMATIC, iters: int = 3, warmup: int = 1, repeats: int = 2,
+         chunk: int | None = None) -> dict:
     """Times build(**knobs).optimize(iters) for every candidate (after `warmup` LM
-    iterations on the same graph, state reset in between); returns the fastest and all
+    iterations on the same graph, state reset in between); returns what `pick` takes and all
     timings (seconds per LM iteration, best of `repeats`)."""
     import torch
     timings = []
@@ -100,8 +109,7 @@ def tune(build, candidates=CANDIDATES + AUTOMATIC, iters: int = 3, warmup: int =
             best = min(best, (time.perf_counter() - t0) / iters)
         g.close()
         timings.append(dict(knobs=knobs, s_per_iter=best))
-    fastest = min(timings, key=lambda t: t["s_per_iter"] * (1.0 if t["knobs"].get("spmv_variant") == 0 else 1.01))
-    return dict(best=fastest["knobs"], timings=timings)
+    return dict(best=pick(timings, chunk), timings=timings)
 
 
 def _ba_builder(p, precision):
@@ -147,7 +155,9 @@ def representative(model: str, cls: str):
 
 
 def tune_all(models=("ba", "vi"), precisions=("fp64", "fp32", "bf16"),
-             classes=("window", "small", "medium"), path: str = TABLE) -> dict:
+             classes=("window", "small", "medium"), path: str = TABLE, rechunk: bool = False) -> dict:
+    """Times every class and writes the table.  A class that has an entry keeps its chunk size
+    (the chunks group the sums: another size gives other roundings) unless `rechunk`."""
     table = load_table(path)
     dev = device_name()
     for model in models:
@@ -155,9 +165,11 @@ def tune_all(models=("ba", "vi"), precisions=("fp64", "fp32", "bf16"),
             p = representative(model, cls)
             for prec in precisions:
                 build = _ba_builder(p, prec) if model == "ba" else _vi_builder(p, prec)
-                res = tune(build)
+                key = f"{dev}|{model}|{prec}|{cls}"
+                held = None if rechunk or key not in table else table[key]["best"]["chunk_edges"]
+                res = tune(build, chunk=held)
                 n_edges = int(p.n_edges)
-                table[f"{dev}|{model}|{prec}|{cls}"] = dict(res, edges=n_edges)
+                table[key] = dict(res, edges=n_edges)
                 print(model, cls, prec, n_edges, res["best"],
                       {f"{t['knobs']['chunk_edges']}/{t['knobs']['spmv_variant']}": round(t['s_per_iter'] * 1e3, 3)
                        for t in res["timings"]}, flush=True)
@@ -169,6 +181,6 @@ def tune_all(models=("ba", "vi"), precisions=("fp64", "fp32", "bf16"),
 if __name__ == "__main__":
     import sys
     if "--write" in sys.argv:
-        tune_all()
+        tune_all(rechunk="--rechunk" in sys.argv)
     else:
         print(__doc__)
