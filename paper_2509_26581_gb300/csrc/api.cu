@@ -1281,20 +1281,22 @@ static gpo_status solve_matrix_free(gpo_graph* g, const gpo::LaunchSet& ls, int 
   return GPO_OK;
 }
 
-// The flags and counters of the one-launch PCG solves start at zero; end_solves waits for
-// the stream and reports a solve one of whose waits gave up.  Such a solve has switched its
-// problem off, so no step was taken from it.
+// The flags and counters of the one-launch PCG solves start at zero.  A solve one of whose
+// waits gave up raises the flag and switches its problem off, so that no step is taken from
+// it; the scalars read back at the end of a call say so (lost_solve), a server reads the flag.
+// end_solves waits for the stream.
 gpo_status gpo_host::begin_solves(gpo_graph* g, const gpo::LaunchSet& ls) {
   if (ls.ex || resident(g, ls)) GPO_CUDA(g, cudaMemsetAsync(ls.running, 0, 6 * sizeof(int), g->stream));
   return GPO_OK;
 }
-gpo_status gpo_host::end_solves(gpo_graph* g, const gpo::LaunchSet& ls) {
-  const bool flag = ls.ex || resident(g, ls);
-  if (flag) GPO_CUDA(g, cudaMemcpyAsync(g->h_flag, ls.running, 2 * sizeof(int), cudaMemcpyDeviceToHost, g->stream));
+gpo_status gpo_host::end_solves(gpo_graph* g) {
   GPO_CUDA(g, cudaStreamSynchronize(g->stream));
   g->up_busy = g->uploading = false;
-  if (flag && g->h_flag[1]) return fail(g, GPO_ERR_TIMEOUT, "a bounded device wait in the PCG solve gave up");
   return GPO_OK;
+}
+gpo_status gpo_host::lost_solve(gpo_graph* g, const Scalars& s) {
+  if (s.active) return GPO_OK;
+  return fail(g, GPO_ERR_TIMEOUT, "a bounded device wait in the PCG solve gave up");
 }
 
 gpo_status gpo_host::post_flags(gpo_graph* g, const gpo::LaunchSet& ls) {
@@ -1880,9 +1882,10 @@ gpo_status gpo_optimize(gpo_graph* g, int32_t max_iters, const gpo_lm_params* pa
   if (nh)
     GPO_CUDA(g, cudaMemcpyAsync(hist.data(), g->dev.hist, nh * sizeof(gpo::IterRecord),
                                 cudaMemcpyDeviceToHost, g->stream));
-  if ((s = end_solves(g, ls)) != GPO_OK) return s;
+  if ((s = end_solves(g)) != GPO_OK) return s;
   const double F0 = cont ? last_cost : g->h_sc->cost0;
   if (!std::isfinite(F0)) return fail(g, GPO_ERR_NUMERIC, "initial cost is not finite (%g)", F0);
+  if ((s = lost_solve(g, *g->h_sc)) != GPO_OK) return s;
   g->hist = std::move(hist);
   if (g->prof.on) prof_resolve(g);
   g->last_cost = g->h_sc->cost;
@@ -2215,8 +2218,9 @@ gpo_status gpo_debug_step(gpo_graph* g, double lambda, const gpo_lm_params* para
   if ((s = fetch(g, xraw, static_cast<const char*>(d.x), (size_t)DB * d.C * sA)) != GPO_OK) return s;
   if ((s = fetch(g, xbraw, static_cast<const char*>(d.xbest), (size_t)DB * d.C * sA)) != GPO_OK) return s;
   if ((s = fetch(g, praw, static_cast<const char*>(d.dp), 3 * (size_t)d.P * sA)) != GPO_OK) return s;
-  if ((s = end_solves(g, g->ls)) != GPO_OK) return s;
+  if ((s = end_solves(g)) != GPO_OK) return s;
   const Scalars* hs = reinterpret_cast<const Scalars*>(sraw.data());
+  if ((s = lost_solve(g, *hs)) != GPO_OK) return s;
   const std::vector<char>& xs = hs->use_best ? xbraw : xraw;
   if (pcg_iters) *pcg_iters = hs->pcg_it;
   size_t off = 0;

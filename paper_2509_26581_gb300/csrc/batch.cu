@@ -327,8 +327,9 @@ gpo_status gpo_optimize_batch(gpo_graph* const* graphs, int32_t n, int32_t max_i
       if ((s = solve_system(owner, bs.ls, max_it, false)) != GPO_OK) break;
       s = finish_iteration(owner, bs.ls);
     }
-    if (s == GPO_OK) s = end_solves(owner, bs.ls);
-    if (s == GPO_OK && (s = get_scalars(owner, bs, sc)) == GPO_OK) {
+    if (s == GPO_OK && (s = get_scalars(owner, bs, sc)) == GPO_OK)
+      for (int i = 0; s == GPO_OK && i < n; ++i) s = lost_solve(owner, sc[i]);
+    if (s == GPO_OK) {
       for (int i = 0; i < n; ++i) {
         graphs[i]->last_cost = sc[i].cost;
         graphs[i]->cost_valid = true;

@@ -166,9 +166,10 @@ gpo_status join_uploads(gpo_graph* owner, const std::vector<gpo_graph*>& graphs)
 bool explicit_pays(const gpo_graph* g, const gpo_lm_params& p);
 // Plans the one-launch matrix-free PCG of a launch set (probs: chunks and camera blocks).
 void plan_resident(const gpo::KernelSet& ks, Prec pr, const std::vector<int2>& probs, gpo::LaunchSet& ls);
-// Around the solves of a call: clear their flags; wait, and report a wait that gave up.
+// Around the solves of a call: clear their flags; wait; report a wait that gave up.
 gpo_status begin_solves(gpo_graph* g, const gpo::LaunchSet& ls);
-gpo_status end_solves(gpo_graph* g, const gpo::LaunchSet& ls);
+gpo_status end_solves(gpo_graph* g);
+gpo_status lost_solve(gpo_graph* g, const Scalars& s);
 // The same report without a wait for what is launched in between: the flags behind the solve.
 gpo_status post_flags(gpo_graph* g, const gpo::LaunchSet& ls);
 gpo_status read_flags(gpo_graph* g, const gpo::LaunchSet& ls);
