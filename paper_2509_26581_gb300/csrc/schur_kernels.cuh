@@ -133,6 +133,26 @@ __device__ void warp_spd_inverse(const AT* A, AT* M, int lane) {
 
 __device__ __forceinline__ int xrows(int kind) { return kind == XK_IMU ? 9 : 6; }
 
+// The sum of n values `stride` apart (partial sums of the explicit Schur complement's diagonal
+// blocks): FP32 values by eight chains of type T, FP64 values, which need no such care, by one.
+template <class T, class AT>
+__device__ __forceinline__ T ex_chains(const AT* v, int stride, int n) {
+  if constexpr (sizeof(AT) == 8) {
+    T s = (T)0;
+    for (int k = 0; k < n; ++k) s += v[(size_t)k * stride];
+    return s;
+  } else {
+    T s[8] = {};
+    int k = 0;
+    for (; k + 8 <= n; k += 8) {
+#pragma unroll
+      for (int j = 0; j < 8; ++j) s[j] += (T)v[(size_t)(k + j) * stride];
+    }
+    for (; k < n; ++k) s[0] += (T)v[(size_t)k * stride];
+    return ((s[0] + s[1]) + (s[2] + s[3])) + ((s[4] + s[5]) + (s[6] + s[7]));
+  }
+}
+
 // ---------------------------------------------------------------- camera render blocks
 
 template <class Mo>
@@ -606,13 +626,12 @@ __global__ void __launch_bounds__(kCamPerBlock * 32) k_cam_finalize(LaunchSet ls
     const int sa = d.cam_s_off[c], sb = d.cam_s_off[c + 1];
     // 2 NG groups of nine outputs; lanes stride over the camera's slots, then a fixed
     // shuffle tree sums the lanes.  With the explicit Schur complement the second NG
-    // groups are the camera's diagonal partials, added in order
+    // groups are the camera's diagonal partials, added in a fixed order
     if (ex) {
       const AT* dp = reinterpret_cast<const AT*>(d.ex_dpart);
       for (int t = lane; t < NPA; t += 32) {
-        AT s = (AT)0;
-        for (int k = d.ex_doff[c]; k < d.ex_doff[c + 1]; ++k) s += dp[(size_t)k * NPA + t];
-        vals[warp][NPA + t] = s;
+        const int k = d.ex_doff[c];
+        vals[warp][NPA + t] = (AT)ex_chains<double>(dp + (size_t)k * NPA + t, NPA, d.ex_doff[c + 1] - k);
       }
     }
     for (int grp = 0; grp < (ex ? NG : 2 * NG); ++grp) {
