@@ -153,9 +153,10 @@ typedef struct {
                                  FP32 storage).  1, 3 and 5 need chunks of at most 1024
                                  edges, 4 of at most 512, else classic runs (5 with
                                  FP64 storage too).  1..3 give bit-identical results;
-                                 the explicit product and 5 sum in another order and 4
-                                 uses unrounded rows, so their products agree with the
-                                 others up to rounding. */
+                                 0 may order the points otherwise (where the explicit
+                                 product may be taken), the explicit product and 5 sum
+                                 in another order and 4 uses unrounded rows, so these
+                                 agree with the others up to rounding. */
 } gpo_graph_desc;
 
 /* Linear solver of the LM step (gpo_lm_params.solver). */
@@ -440,7 +441,9 @@ typedef struct {
   int32_t precision;          /* of every graph it serves */
   int32_t device;
   void* cuda_stream;          /* NULL = the server creates one */
-  size_t memory_budget;       /* device bytes of resident graphs; 0 = unlimited */
+  size_t memory_budget;       /* device bytes of resident graphs; 0 = unlimited.  A graph
+                                 that fits only without the blocks of the explicit Schur
+                                 complement is taken without them. */
   int32_t max_resident;       /* slots: graphs solved concurrently (default 1024) */
   int32_t reserved0;
 } gpo_server_desc;

@@ -29,8 +29,8 @@ constexpr int kMaxDevices = 64;     // per-device launch caches
 constexpr int kGroupEdges = 64;     // edges of a warp group (two per lane) of a chunk
 constexpr int kMaxGroups = 16;      // warp groups per chunk
 constexpr int kMaxHistory = 4096;
+constexpr int kResChunks = 2;       // chunks per CTA of the resident PCG at most (schur_resident.cuh)
 // explicit Schur complement (schur_explicit.cuh)
-constexpr int kResChunks = 2;      // chunks per CTA of the resident PCG at most
 constexpr int kExThreads = 512;     // CTA size of the PCG solve
 constexpr int kExCluster = 8;       // CTAs of a small problem's solve (a cluster)
 constexpr int kExGrid = 152;        // CTAs of a larger one's (one per SM)

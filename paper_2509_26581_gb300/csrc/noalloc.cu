@@ -71,8 +71,9 @@ __device__ double edge_rho(const double* c, const double* X, double2 z, double d
 // cosine, a square root, three divisions), and observations usually come in runs of one
 // camera, so a CTA forms it once per run: a thread whose edge starts a run writes the camera's
 // block to shared memory, and the run's edges read it there.  Edges in no order make every
-// thread its own run.  FP64-bound: 400 cameras, 0.97 million edges in camera order 240 ->
-// 112 us; RMS error over 16 scenes 6.3e-16 -> 5.7e-16.
+// thread its own run.  FP64-bound: 400 cameras, 1.01 million edges in camera order 248 ->
+// 113 us, in point order or none (a camera block per edge) 248 -> 227; RMS error over 16
+// scenes 6.3e-16 -> 5.7e-16.
 __global__ void __launch_bounds__(kThreads) k_cost_noalloc(const double* cams, const double* pts, const int* ci,
                                                           const int* pi, const double* obs, long long n, double delta,
                                                           double* out, Scratch* scr) {

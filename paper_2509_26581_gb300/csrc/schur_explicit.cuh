@@ -518,12 +518,12 @@ struct ExWait {
   __device__ __forceinline__ bool again() const { return sm_clock() - t0 < kWaitClocks; }
 };
 
-// Sum over a warp, the same in every lane.  FP64 additions take a sub-partition's pipe some 70 clocks each on this part, so the
-// values are added as 64-bit integers on the scale of the largest: a value's 53-bit
+// Sum over a warp of the lanes' v, n values in all (the lanes past n hold zero), the same in
+// every lane.  FP64 additions take a sub-partition's pipe some 70 clocks each on this part, so
+// the values are added as 64-bit integers on the scale of the largest: a value's 53-bit
 // significand is shifted to leave room for n terms (bits below 2^-52 of the largest term and
 // less are cut, as roundings of a floating sum cut them), and the order does not matter.
 // Infinities, NaN and values near the smallest exponents are added as they are.
-// Here: the sum of the lanes' v, n values in all (the lanes past n hold zero).
 static __device__ __noinline__ double ex_warp_sum(double v, int n) {
   constexpr unsigned full = 0xffffffffu;
   const long long b = __double_as_longlong(v);

@@ -16,8 +16,8 @@ from . import gpo
 
 
 # Schedule of served windows: the automatic product with 512-edge chunks (the whole PCG in
-# one launch while the resident windows' chunks fit the device at once, else pipelined).  The same knobs solve a window alone, so served
-# and lone results stay equal.
+# one launch while the resident windows' chunks fit the device at once, else pipelined).  The
+# same knobs solve a window alone, so served and lone results stay equal.
 SERVED_KNOBS = dict(chunk_edges=512, spmv_variant=0)
 
 
