@@ -299,7 +299,8 @@ __device__ __forceinline__ AT ex_dot3(const AT* x, const AT* y, AT acc) {
 // a row per lane, the lanes added in a fixed order.  S_cc = H_cc + lambda D_c - sum Y Y^T
 // cancels and the squares on its diagonal all have one sign, so that in FP32 a long chain of
 // additions shows in the solve: the lanes, and the segments in k_cam_finalize, are added by
-// ex_chains.  RMS error of S_cc relative to its diagonal, in 2^-23, with one chain throughout
+// ex_chains (64 segments and more in FP64, whose conversions took 4 us of a damped system of
+// 100 cameras).  RMS error of S_cc relative to its diagonal, in 2^-23, with one chain throughout
 // and so, the matrix-free kernels' on the same graph in brackets: 6 cameras of 33,000 rows
 // 0.46, 0.36 (0.37); 4 of 45,000 0.86, 0.52 (0.57).
 template <class Mo, class AT>

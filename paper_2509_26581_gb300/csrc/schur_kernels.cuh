@@ -630,8 +630,9 @@ __global__ void __launch_bounds__(kCamPerBlock * 32) k_cam_finalize(LaunchSet ls
     if (ex) {
       const AT* dp = reinterpret_cast<const AT*>(d.ex_dpart);
       for (int t = lane; t < NPA; t += 32) {
-        const int k = d.ex_doff[c];
-        vals[warp][NPA + t] = (AT)ex_chains<double>(dp + (size_t)k * NPA + t, NPA, d.ex_doff[c + 1] - k);
+        const int k = d.ex_doff[c], n = d.ex_doff[c + 1] - k;
+        const AT* v = dp + (size_t)k * NPA + t;
+        vals[warp][NPA + t] = n < 64 ? ex_chains<AT>(v, NPA, n) : (AT)ex_chains<double>(v, NPA, n);
       }
     }
     for (int grp = 0; grp < (ex ? NG : 2 * NG); ++grp) {
