@@ -127,9 +127,9 @@ typedef struct {
                                  and is left out where the memory (the budget, a server's
                                  budget, the device, the allocator) holds the graph only
                                  without, a camera sees a point twice, forming the
-                                 blocks costs more than it saves (in a call whose
-                                 pcg_max_iters or loose relative pcg_tol leaves its
-                                 solves few iterations too), or for bundle
+                                 blocks costs more than it saves (also in solves to
+                                 which pcg_max_iters, a loose relative pcg_tol or a
+                                 heavy damping leaves few iterations), or for bundle
                                  adjustment with BF16 storage, or FP32 and more than
                                  65,536 points; then pipelined for BF16 and FP32
                                  storage, the whole PCG in one launch with the same

@@ -1214,21 +1214,30 @@ static gpo_status ensure_full(gpo_graph* g) {
   return GPO_OK;
 }
 
-// Whether a call's solves take the explicit Schur complement of a graph that has one planned.
-// The plan takes a solve to have 16 iterations; a cap or a loose relative tolerance leaves
-// fewer, and then forming the blocks may cost more than the products (300 cameras FP64, two
-// LM iterations: 5 iterations each 4,475 us matrix-free, 6,756 explicit; 16 each 8,145 and
-// 6,970).  Iterations are taken in proportion to the tolerance's digits, 16 at 1e-6, with
-// an inertial chain 80 (10 to 25 and 83 to 87 measured at a light damping).  The rule reads
-// the parameters that stay the same along a run and not the damping, so that a batch, a
-// server and a run continued call by call solve as one call does; solves under a heavy
-// damping, which have few iterations too, form the blocks all the same (damping 10 there:
-// 4,379 us matrix-free, 6,669 explicit).
-bool gpo_host::explicit_pays(const gpo_graph* g, const gpo_lm_params& p) {
+// Which damped systems of a call take the explicit Schur complement of a graph that has one
+// planned.  The plan takes a solve to have 16 iterations; a cap, a loose relative tolerance or
+// a heavy damping leaves fewer, and then forming the blocks may cost more than the products
+// (300 cameras FP64, two LM iterations: 5 iterations each 4,475 us matrix-free, 6,756
+// explicit; 16 each 8,145 and 6,970).  Iterations are taken in proportion to the tolerance's
+// digits, 16 at 1e-6, with an inertial chain 80 (10 to 25 and 83 to 87 measured at a light
+// damping); under the damping lambda diag(H), where the preconditioned system's eigenvalues
+// lie about in [lambda / (1 + lambda), 1], by the bound of conjugate gradients on that
+// interval: tol = 2 ((k - 1) / (k + 1))^n after n iterations, k = sqrt(1 + 1 / lambda), so n
+// is at least a given number while lambda is at most sinh^2(log(2 / tol) / 2 n) (at 1e-6 the
+// bound gives 23, 8, 4 and 2 iterations for lambda = 0.1, 1, 10 and 100; measured on 300
+// cameras 25, 9, 4 and 2).  Graphs with an inertial chain gained at every damping.  The rule
+// reads nothing but the parameters and the damping of the system at hand, so a batch, a
+// server and a run continued call by call solve as one call does; the host reads the damping
+// only where it may have crossed the limit (DampingRange).
+double gpo_host::explicit_up_to(const gpo_graph* g, const gpo_lm_params& p) {
+  const bool relative = p.pcg_tol_relative && p.pcg_tol > 0.0;
   double n = std::max(1, p.pcg_max_iters);
   const double per_digit = (g->dev.NX > 0 ? 80.0 : 16.0) / 6.0;
-  if (p.pcg_tol_relative && p.pcg_tol > 0.0) n = std::min(n, std::max(1.0, per_digit * -std::log10(p.pcg_tol)));
-  return g->ls.ex && n >= g->ex_min_it;
+  if (relative) n = std::min(n, std::max(1.0, per_digit * -std::log10(p.pcg_tol)));
+  if (!g->ls.ex || n < g->ex_min_it) return -1.0;
+  if (!relative || p.damping_mode != 0 || g->dev.NX > 0 || g->ex_min_it <= 1.0) return HUGE_VAL;
+  const double s = std::sinh(std::log(2.0 / p.pcg_tol) / (2.0 * g->ex_min_it));
+  return s * s;
 }
 
 // Plans the resident PCG of a launch set: the fewest chunks per CTA at which the CTAs fit the
@@ -1870,17 +1879,26 @@ gpo_status gpo_optimize(gpo_graph* g, int32_t max_iters, const gpo_lm_params* pa
   // the iterations follow without a look at the cost: one that is not finite switches them
   // off on the device
   if (!cont && (s = launch_initial_cost(g, g->ls)) != GPO_OK) return s;
-  gpo::LaunchSet ls = g->ls;
-  if (ls.ex && !explicit_pays(g, prm)) {
-    ls.ex = ls.n_cl = ls.n_xg = 0;
-    ls.mf = 1;
-  }
-  if ((s = begin_solves(g, ls)) != GPO_OK) return s;
+  if ((s = begin_solves(g, g->ls)) != GPO_OK) return s;
+  const double limit = explicit_up_to(g, prm);
+  DampingRange damping;
+  damping.start(sc);
   for (int it = 0; it < max_iters; ++it) {
     g->cur_lm_iter = it;
+    if (damping.within(limit) < 0) {   // the damping may have crossed the limit
+      GPO_CUDA(g, cudaMemcpyAsync(g->h_sc, g->dev.sc, sizeof(Scalars), cudaMemcpyDeviceToHost, g->stream));
+      if ((s = end_solves(g)) != GPO_OK) return s;
+      damping.start(*g->h_sc);
+    }
+    gpo::LaunchSet ls = g->ls;
+    if (ls.ex && !damping.within(limit)) {
+      ls.ex = ls.n_cl = ls.n_xg = 0;
+      ls.mf = 1;
+    }
     ls.debug_wait = held(g, it);
     if ((s = solve_system(g, ls, sc.max_it, false)) != GPO_OK) return s;
     if ((s = finish_iteration(g, ls)) != GPO_OK) return s;
+    damping.iteration(sc);
   }
   g->cur_lm_iter = -1;
   GPO_CUDA(g, cudaMemcpyAsync(g->h_sc, g->dev.sc, sizeof(Scalars), cudaMemcpyDeviceToHost, g->stream));

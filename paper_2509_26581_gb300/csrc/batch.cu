@@ -252,6 +252,10 @@ struct gpo_server {
     int done_iters;
     size_t bytes;
     double initial_cost;
+    DampingRange damping;
+    Scalars start;          // the parameters
+    double limit;           // explicit_up_to
+    bool ex;                // solves on its explicit Schur complement
     gpo_graph_desc saved;   // the graph's own stream and allocator, restored at retirement
     bool adopted_stream;
   };
@@ -297,17 +301,26 @@ gpo_status gpo_optimize_batch(gpo_graph* const* graphs, int32_t n, int32_t max_i
   std::vector<gpo_graph*> gs(graphs, graphs + n);
   BatchSet bs;
   gpo_status s = join_uploads(owner, gs);
-  std::vector<char> ex;
-  for (const gpo_graph* g : gs) ex.push_back(explicit_pays(g, prm));
-  if (s == GPO_OK) s = build_set(owner, gs, ex, bs);
   if (s != GPO_OK) return s;
   std::vector<Scalars> sc(n);
+  std::vector<DampingRange> damping(n);
+  std::vector<double> limit(n);
   for (int i = 0; i < n; ++i) {
     graphs[i]->cost_valid = graphs[i]->state_same = false;   // until the call has ended well
     fill_scalars(graphs[i], prm, prm.initial_damping, sc[i]);
     sc[i].full = 0;   // shared launches run the Schur form
     graphs[i]->pcg_full = 0;
+    damping[i].start(sc[i]);
+    limit[i] = explicit_up_to(graphs[i], prm);
   }
+  const Scalars first = sc[0];   // the parameters, alike for all
+  auto choice = [&] {
+    std::vector<char> ex(n);
+    for (int i = 0; i < n; ++i) ex[i] = damping[i].within(limit[i]) > 0;
+    return ex;
+  };
+  std::vector<char> ex = choice();
+  if ((s = build_set(owner, gs, ex, bs)) != GPO_OK) return s;
   int max_it = 1;
   for (auto& x : sc) max_it = std::max(max_it, x.max_it);
   if ((s = put_scalars(owner, bs, sc)) == GPO_OK && (s = launch_initial_cost(owner, bs.ls)) == GPO_OK &&
@@ -323,6 +336,18 @@ gpo_status gpo_optimize_batch(gpo_graph* const* graphs, int32_t n, int32_t max_i
     if (s == GPO_OK && (s = ensure_runtime(owner)) == GPO_OK) s = begin_solves(owner, bs.ls);
     for (int it = 0; s == GPO_OK && it < max_iters; ++it) {
       owner->cur_lm_iter = -1;
+      bool read = false;
+      for (int i = 0; i < n; ++i) read |= damping[i].within(limit[i]) < 0;
+      if (read) {   // a damping may have crossed its limit
+        if ((s = get_scalars(owner, bs, sc)) != GPO_OK) break;
+        for (int i = 0; i < n; ++i) damping[i].start(sc[i]);
+      }
+      if (std::vector<char> now = choice(); now != ex) {
+        ex = std::move(now);
+        bs.release(owner->stream);
+        if ((s = build_set(owner, gs, ex, bs)) != GPO_OK || (s = begin_solves(owner, bs.ls)) != GPO_OK) break;
+      }
+      for (auto& d : damping) d.iteration(first);
       bs.ls.debug_wait = std::any_of(gs.begin(), gs.end(), [&](const gpo_graph* g) { return held(g, it); });
       if ((s = solve_system(owner, bs.ls, max_it, false)) != GPO_OK) break;
       s = finish_iteration(owner, bs.ls);
@@ -427,7 +452,7 @@ gpo_status gpo_server_submit(gpo_server* sv, gpo_graph* g, int32_t max_iters, co
     return fail(sv->owner, GPO_ERR_OOM, "graph needs %zu bytes, more than the server budget %zu", bytes,
                 (size_t)sv->desc.memory_budget);
   sv->owner->ks = k;
-  gpo_server::Req r{g, max_iters, params_or_default(params), sv->next_ticket++, 0, bytes, 0.0, g->desc, false};
+  gpo_server::Req r{g, max_iters, params_or_default(params), sv->next_ticket++, 0, bytes, 0.0, {}, {}, -1.0, false, g->desc, false};
   // a graph without a stream of its own runs on the server's; a graph without an
   // allocator hook takes its arena from the server's pool
   if (!g->stream) {
@@ -485,6 +510,10 @@ gpo_status gpo_server_step(gpo_server* sv, int32_t* n_resident, int32_t* n_queue
     if (s != GPO_OK) return s;
     for (size_t i = 0; i < adm.size(); ++i) {
       adm[i].initial_cost = sc[i].cost;
+      adm[i].start = sc[i];
+      adm[i].damping.start(sc[i]);
+      adm[i].limit = explicit_up_to(adm[i].g, adm[i].prm);
+      adm[i].ex = adm[i].damping.within(adm[i].limit) > 0;
       if (adm[i].max_iters == 0 || !std::isfinite(adm[i].initial_cost)) {
         gpo_report rep;
         report_from(sc[i], adm[i].initial_cost, &rep);
@@ -504,7 +533,7 @@ gpo_status gpo_server_step(gpo_server* sv, int32_t* n_resident, int32_t* n_queue
       std::vector<char> ex;
       for (auto& r : sv->resident) {
         gs.push_back(r.g);
-        ex.push_back(explicit_pays(r.g, r.prm));
+        ex.push_back(r.ex);
       }
       gpo_status s = build_set(owner, gs, ex, sv->set);
       if (s != GPO_OK) return s;
@@ -529,8 +558,23 @@ gpo_status gpo_server_step(gpo_server* sv, int32_t* n_resident, int32_t* n_queue
     if (s != GPO_OK) return s;
     ++sv->steps;
     // 3. retirement of graphs that ran all their iterations
-    bool any = false;
-    for (size_t i = 0; i < ran.size(); ++i) any |= ((sv->resident[i].done_iters += ran[i]) >= sv->resident[i].max_iters);
+    bool any = false, read = false;
+    for (size_t i = 0; i < ran.size(); ++i) {
+      gpo_server::Req& r = sv->resident[i];
+      any |= (r.done_iters += ran[i]) >= r.max_iters;
+      if (ran[i]) r.damping.iteration(r.start);
+      read |= r.damping.within(r.limit) < 0;
+    }
+    if (read) {   // a damping may have crossed its limit
+      std::vector<Scalars> sc;
+      if ((s = get_scalars(owner, sv->set, sc)) != GPO_OK) return s;
+      for (size_t i = 0; i < sc.size(); ++i) sv->resident[i].damping.start(sc[i]);
+    }
+    for (auto& r : sv->resident) {
+      const bool ex = r.damping.within(r.limit) > 0;
+      sv->dirty |= ex != r.ex;
+      r.ex = ex;
+    }
     if (any) {
       std::vector<Scalars> sc;
       if ((s = get_scalars(owner, sv->set, sc)) != GPO_OK) return s;

@@ -3,6 +3,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <memory>
 #include <string>
@@ -162,8 +163,25 @@ gpo_lm_params params_or_default(const gpo_lm_params* p);
 gpo_status solve_system(gpo_graph* g, const gpo::LaunchSet& ls, int max_it, bool force_lin);
 // Orders owner's stream after the uploads that are still running on the graphs' own streams.
 gpo_status join_uploads(gpo_graph* owner, const std::vector<gpo_graph*>& graphs);
-// Whether solves with these parameters take the graph's explicit Schur complement.
-bool explicit_pays(const gpo_graph* g, const gpo_lm_params& p);
+// What the host knows of a problem's damping without reading it: exact at a run's start and
+// after a read, then within the factors that an iteration can change it by.
+struct DampingRange {
+  double low, high, nu;
+  void start(const Scalars& s) {
+    low = high = s.lambda;
+    nu = s.nu;
+  }
+  void iteration(const Scalars& s) {   // accepted: by 1/3 to 2; rejected: by nu, which doubles
+    low = std::min(std::max(low / 3.0, s.lambda_min), s.lambda_max);
+    high = std::min(std::max(high * nu, s.lambda_min), s.lambda_max);
+    nu *= 2.0;
+  }
+  // whether the damping is at most `limit`: 1 yes, 0 no, -1 it may or may not be
+  int within(double limit) const { return high <= limit ? 1 : low > limit ? 0 : -1; }
+};
+// The damping up to which solves with these parameters take the graph's explicit Schur
+// complement (negative: none does).
+double explicit_up_to(const gpo_graph* g, const gpo_lm_params& p);
 // Plans the one-launch matrix-free PCG of a launch set (probs: chunks and camera blocks).
 void plan_resident(const gpo::KernelSet& ks, Prec pr, const std::vector<int2>& probs, gpo::LaunchSet& ls);
 // Around the solves of a call: clear their flags; wait; report a wait that gave up.

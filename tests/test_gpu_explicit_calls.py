@@ -1,6 +1,7 @@
-"""Calls whose solves have few iterations (a low cap, a loose tolerance) on graphs that have the
-explicit Schur complement planned: matrix-free where forming the blocks would cost more than it
-saves, alone, in a batch and in a server alike (bit for bit), explicit where it still pays."""
+"""Solves of few iterations (a low cap, a loose tolerance, a heavy damping) on graphs that have
+the explicit Schur complement planned: matrix-free where forming the blocks would cost more
+than it saves, alone, in a batch, in a server and call by call alike (bit for bit), explicit
+where it still pays."""
 import numpy as np
 import pytest
 
@@ -32,9 +33,11 @@ def _forms(g):
 @pytest.mark.parametrize("name,kw,explicit", [
     ("path", dict(), True), ("path", dict(pcg_max_iters=3), False), ("path", dict(pcg_tol=0.1), False),
     ("path", dict(pcg_tol=0.1, pcg_tol_relative=0), True), ("path", dict(pcg_max_iters=16, pcg_tol=0.0), True),
-    ("path", dict(pcg_tol=10.0), False), ("ring", dict(pcg_max_iters=1), True), ("ring", dict(pcg_tol=0.1), True)])
+    ("path", dict(pcg_tol=10.0), False), ("ring", dict(pcg_max_iters=1), True), ("ring", dict(pcg_tol=0.1), True),
+    ("path", dict(initial_damping=10.0), False), ("ring", dict(initial_damping=10.0), True),
+    ("path", dict(initial_damping=10.0, damping_mode=1), True)])
 def test_the_product_follows_the_calls_iterations(gpo, name, kw, explicit):
-    params = gpo.default_params(initial_damping=0.1, **kw)
+    params = gpo.default_params(**{"initial_damping": 0.1, **kw})
     p, g, c0, p0 = _build(gpo, name)
     rep = g.optimize(2, params)
     assert g.info()["spmv_kernel"] == 7 and _forms(g) == explicit
@@ -49,13 +52,21 @@ def test_the_product_follows_the_calls_iterations(gpo, name, kw, explicit):
     assert _forms(g)
 
 
-@pytest.mark.parametrize("kw", [dict(), dict(pcg_max_iters=3), dict(pcg_tol=0.1)], ids=["full", "cap", "loose"])
+# the last two cross the limit of the path scene (about 0.7) during the run: accepted steps lower
+# the damping from 10; a rejected one raises it from 1e-4 to 10 first
+@pytest.mark.parametrize("kw", [dict(), dict(pcg_max_iters=3), dict(pcg_tol=0.1), dict(initial_damping=10.0),
+                                dict(initial_damping=1e-4, initial_nu=1e5)], ids=["full", "cap", "loose", "down", "up"])
 def test_batch_server_and_single_iterations_solve_like_one_call(gpo, kw):
-    params = gpo.default_params(initial_damping=0.1, **kw)
+    start = {"initial_damping": 0.1, **kw}
+    iters = 9 if "initial_damping" in kw else 3
+    params = gpo.default_params(**start)
     alone, graphs = [], []
     for name in SCENES:
         p, g, c0, p0 = _build(gpo, name)
-        rep = g.optimize(3, params)
+        rep = g.optimize(iters, params)
+        lam, formed = [h["lam"] for h in g.history()], g.profile()["schur_form"]["launches"]
+        if name == "path" and iters == 9:   # both products took part
+            assert min(lam) < 0.2 and max(lam) > 2.0 and 0 < formed < 9 * 4
         alone.append((rep.final_cost, rep.pcg_iters_total, g.get_state(c0, p.n_cams, 9), g.get_state(p0, p.n_pts, 3)))
         graphs.append((p, c0, p0))
 
@@ -65,18 +76,18 @@ def test_batch_server_and_single_iterations_solve_like_one_call(gpo, kw):
             assert np.array_equal(g.get_state(c0, p.n_cams, 9), a[2]) and np.array_equal(g.get_state(p0, p.n_pts, 3), a[3])
 
     built = [_build(gpo, name)[1] for name in SCENES]
-    same(built, gpo.optimize_batch(built, 3, params))
+    same(built, gpo.optimize_batch(built, iters, params))
     built = [_build(gpo, name)[1] for name in SCENES]
     sv = gpo.Server("fp64")
-    tickets = [sv.submit(g, 3, params) for g in built]
+    tickets = [sv.submit(g, iters, params) for g in built]
     while sum(sv.step()[:2]):
         pass
     same(built, [sv.poll(t) for t in tickets])
     sv.close()
     for a, (p, c0, p0), name in zip(alone, graphs, SCENES):
         g = _build(gpo, name)[1]
-        step = gpo.default_params(initial_damping=0.1, **kw)
-        for _ in range(3):
+        step = gpo.default_params(**start)
+        for _ in range(iters):
             r = g.optimize(1, step)
             step.initial_damping, step.initial_nu = r.final_lambda, r.final_nu
         assert r.final_cost == a[0] and np.array_equal(g.get_state(c0, p.n_cams, 9), a[2])
