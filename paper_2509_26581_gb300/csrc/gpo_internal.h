@@ -110,7 +110,7 @@ struct IterRecord {       // mirrors gpo_iter_record
 // camera tangent block (9 / 15), DC = camera columns of an observation's Jacobian
 // (9 / 6), M = observation rows (2 / 3), NJ = Jacobian row (24 / 32), NPA = slot
 // partial row (54 / 27), TB = packed camera block (45 / 120).
-struct DevBA {
+struct alignas(16) DevBA {
   int C, P, E, NCH, NS;
   int NX;                    // extra (camera-side) edges
   int model;                 // ModelKind
@@ -191,7 +191,8 @@ struct DevBA {
   int ch_max;                // max edges per chunk
   int ns_max, np_max;        // max slots / points of a chunk
   int ncblk;                 // CTAs of the camera kernels
-  // explicit Schur complement (ex = 0: none planned, the product is matrix-free).  Block
+  // explicit Schur complement (ex = 0: none planned, the product is matrix-free; last: the
+  // matrix-free products do not copy the fields from here on).  Block
   // rows hold the cameras that share points with a camera, both triangles, columns
   // ascending; "upper" blocks are those right of the diagonal, numbered row by row
   int ex;
@@ -224,6 +225,8 @@ struct DevBA {
   unsigned long long* ex_red;   // [2][kExMaxCtas][4] posted partial sums of the PCG solve, and their count
   unsigned long long* ex_z;     // [C][DB] posted z (one word in FP32, two in FP64)
 };
+
+constexpr int kProductWords = (int)(offsetof(DevBA, ex) / 4);   // what a matrix-free product reads
 
 enum class Prec { F64 = 0, F32 = 1, BF16 = 2 };
 

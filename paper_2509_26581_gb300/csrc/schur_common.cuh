@@ -356,12 +356,13 @@ __device__ __forceinline__ ChunkRange chunk_range(const DevBA& d, int k) {
   return c;
 }
 
-// Copies a problem's descriptor into shared memory (all threads cooperate).
+// Copies a problem's descriptor into shared memory (all threads cooperate), in 16-byte pieces:
+// one round of loads for 68 threads and more.
 __device__ __forceinline__ void bind_problem(DevBA& dst, const DevBA* src) {
-  static_assert(sizeof(DevBA) % 4 == 0, "DevBA must be a whole number of words");
-  const int* s4 = reinterpret_cast<const int*>(src);
-  int* d4 = reinterpret_cast<int*>(&dst);
-  for (int i = threadIdx.x; i < (int)(sizeof(DevBA) / 4); i += blockDim.x) d4[i] = s4[i];
+  static_assert(sizeof(DevBA) % 16 == 0, "DevBA must be a whole number of 16-byte pieces");
+  const int4* s4 = reinterpret_cast<const int4*>(src);
+  int4* d4 = reinterpret_cast<int4*>(&dst);
+  for (int i = threadIdx.x; i < (int)(sizeof(DevBA) / 16); i += blockDim.x) d4[i] = s4[i];
   __syncthreads();
 }
 

@@ -482,7 +482,6 @@ __global__ void __launch_bounds__(kThreads, PipeOcc<JT>::value) k_spmv_pp(Launch
   using Dm = Dims<Mo>;
   constexpr int DC = Mo::DC, DB = Mo::DB, NJ = Mo::NJ;
   constexpr size_t PRB = (6 * sizeof(AT) + 8 + 15) & ~(size_t)15;
-  constexpr int kWords = (int)(sizeof(DevBA) / 4);
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ DevBA d;
   __shared__ PipeChunk ck[3];
@@ -602,7 +601,7 @@ __global__ void __launch_bounds__(kThreads, PipeOcc<JT>::value) k_spmv_pp(Launch
     const PipeChunk cn = ck[(n + 1) % 3];
     if (c.q != bound_q) {        // CTA-uniform: bind the chunk's problem
       __syncthreads();           // every thread is past the previous use of d
-      for (int i = threadIdx.x; i < kWords; i += kThreads)
+      for (int i = threadIdx.x; i < kProductWords; i += kThreads)
         reinterpret_cast<int*>(&d)[i] = reinterpret_cast<const int*>(ls.probs + c.q)[i];
       bound_q = c.q;
       __syncthreads();

@@ -212,7 +212,6 @@ template <class Mo, class JT>
 __global__ void __launch_bounds__(kThreads, WgOcc<JT>::value) k_spmv_wg(LaunchSet ls) {
   using AT = float;
   constexpr int DC = Mo::DC, DB = Mo::DB, NJ = Mo::NJ;
-  constexpr int kWords = (int)(sizeof(DevBA) / 4);
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ DevBA d;
   __shared__ PipeChunk ck[4];
@@ -298,7 +297,7 @@ __global__ void __launch_bounds__(kThreads, WgOcc<JT>::value) k_spmv_wg(LaunchSe
     const PipeChunk cn = ck[(n + 1) & 3];
     if (c.q != bound_q) {        // CTA-uniform: bind the chunk's problem
       __syncthreads();           // every thread is past the previous use of d (and the gather)
-      for (int i = threadIdx.x; i < kWords; i += kThreads)
+      for (int i = threadIdx.x; i < kProductWords; i += kThreads)
         reinterpret_cast<int*>(&d)[i] = reinterpret_cast<const int*>(ls.probs + c.q)[i];
       bound_q = c.q;
       __syncthreads();
