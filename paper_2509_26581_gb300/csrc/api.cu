@@ -920,8 +920,8 @@ gpo_status gpo_host::finalize(gpo_graph* g, size_t* plan_bytes) {
     g->ks->ex_plan(ls, g->prec, d.C, R.ex_nb_max, d.E, st);
     ls.ex_scratch = nullptr;
   }
-  if (ls.mf && ls.n_ch && ls.n_cb) gpo_host::plan_resident(*g->ks, g->prec, {make_int2(ls.n_ch, ls.n_cb)}, ls);
   g->ls = ls;
+  g->alone_planned = false;
   g->dev_desc = R.desc_d;
   g->ch_max = R.ch;
   g->j_elems = R.jpos;
@@ -1252,6 +1252,14 @@ void gpo_host::plan_resident(const gpo::KernelSet& ks, Prec pr, const std::vecto
     if (ls.res_ctas <= slots) return;
   }
   ls.res_m = ls.res_ctas = 0;
+}
+
+// The same for a graph solved alone, at its first solve: a graph of a server never needs it.
+static void plan_alone(gpo_graph* g) {
+  if (g->alone_planned) return;
+  g->alone_planned = true;
+  gpo::LaunchSet& ls = g->ls;
+  if (ls.mf && ls.n_ch && ls.n_cb) gpo_host::plan_resident(*g->ks, g->prec, {make_int2(ls.n_ch, ls.n_cb)}, ls);
 }
 
 static gpo_status solve_matrix_free(gpo_graph* g, const gpo::LaunchSet& ls, int max_it);
@@ -1879,6 +1887,7 @@ gpo_status gpo_optimize(gpo_graph* g, int32_t max_iters, const gpo_lm_params* pa
   // the iterations follow without a look at the cost: one that is not finite switches them
   // off on the device
   if (!cont && (s = launch_initial_cost(g, g->ls)) != GPO_OK) return s;
+  plan_alone(g);
   if ((s = begin_solves(g, g->ls)) != GPO_OK) return s;
   const double limit = explicit_up_to(g, prm);
   DampingRange damping;
@@ -2233,6 +2242,7 @@ gpo_status gpo_debug_step(gpo_graph* g, double lambda, const gpo_lm_params* para
   fill_scalars(g, prm, lambda, sc);
   if ((s = upload_scalars(g, sc)) != GPO_OK) return s;
   g->ks->cam_prepare(g->ls, false, g->stream);
+  plan_alone(g);
   if ((s = begin_solves(g, g->ls)) != GPO_OK) return s;
   if ((s = solve_system(g, g->ls, sc.max_it, true)) != GPO_OK) return s;
   const DevBA& d = g->dev;
@@ -2277,6 +2287,7 @@ gpo_status gpo_debug_wait_timeout(gpo_graph* g) {
   if ((s = upload_scalars(g, sc)) != GPO_OK) return s;
   g->ks->cam_prepare(g->ls, false, g->stream);
   g->ks->linearize(g->ls, g->prec, true, g->stream);
+  plan_alone(g);
   gpo::LaunchSet ls = g->ls;
   if (!ls.n_xg) ls.ex = 0;   // a cluster's solve, below, and the matrix-free camera kernel
   if (ls.ex) g->ks->ex_form(ls, g->prec, g->stream);

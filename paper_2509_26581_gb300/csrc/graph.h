@@ -105,6 +105,7 @@ struct gpo_graph {
   DevBA dev{};
   gpo::LaunchSet ls{};             // one-problem launch set over `dev`
   double ex_min_it = 0.0;          // iterations per solve from which the explicit Schur complement pays
+  bool alone_planned = false;      // ls says whether the graph's PCG alone runs in one launch
   bool ex_cluster = false;         // explicit Schur complement: solved by a cluster (else a grid)
   int4 ex_grid{0, 0, 0, 0};        // the solve's launch (problem, CTAs, shared memory)
   int debug_wait = 0;              // LaunchSet::debug_wait of the solves from this iteration on (0: never)
